@@ -358,8 +358,8 @@ gridspt_status gridspt_multi_destroy(gridspt_multi multi);
  * a sixth and seventh (5, 6) that transform two outputs of one input at a
  * time. The z
  * expansion and the contiguous-axis forward pass have a third that runs one z
- * row per group of warp lanes without block-wide barriers (power-of-two
- * N <= 512; other sizes run variant 0 when it is chosen); the z expansion's
+ * row per group of warp lanes without block-wide barriers (every N but 12,
+ * which runs variant 0 when it is chosen); the z expansion's
  * choice also applies to the pair products fused into it and to the z pass of
  * the bispectrum shells. gridspt_autotune times the
  * variants of every pass on `scratch` (device, >= gridspt_autotune_scratch_size

@@ -240,10 +240,11 @@ __device__ __forceinline__ void fft_column(float2 (&x)[fft_elems(L)], int p, flo
 
 // ------------------------------------------------------- warp-row variant
 // The same transform with the P threads of one length-L row on P consecutive
-// lanes of one warp (P <= 32 and 32 % P == 0, so a warp holds 32 / P rows):
-// the stage exchanges go through a per-warp buffer, ordered by __syncwarp, so
-// rows never wait on a block-wide barrier. Stage arithmetic and twiddle values
-// are those of fft_stage, so results are bitwise equal.
+// lanes of one warp (P <= 32 and 32 % P == 0, so a warp holds 32 / P rows), or
+// of two warps for P = 64 (L = 512): the stage exchanges go through a buffer of
+// those warps, ordered by __syncwarp or a 64-thread named barrier (row_sync),
+// so rows never wait on a block-wide barrier. Stage arithmetic and twiddle
+// values are those of fft_stage, so results are bitwise equal.
 //
 // Exchange buffer: element n of a row at xpad(n) = n + n / 16 (one float2 of
 // padding per 16). With it every stage's scatter writes and gather reads of a
@@ -252,6 +253,14 @@ __device__ __forceinline__ void fft_column(float2 (&x)[fft_elems(L)], int p, flo
 // Stage twiddles are read from a lane-major table twl[j][p] (conflict-free,
 // identical for every row): j enumerates (stage S >= 1, butterfly q, t >= 1).
 __device__ __forceinline__ int xpad(int n) { return n + (n >> 4); }
+
+// Barrier of the threads that share a row: the warp, or for P > 32 the P
+// threads of named barrier `bar` (1 .. 15, one per team of the block).
+template <int P>
+__device__ __forceinline__ void row_sync(int bar) {
+    if constexpr (P <= 32) __syncwarp();
+    else asm volatile("bar.sync %0, %1;\n" ::"r"(bar), "n"(P) : "memory");
+}
 
 template <int L>
 __host__ __device__ constexpr int fft_row_tw_count(int S) {   // stage twiddles of stages < S
@@ -283,7 +292,7 @@ __device__ __forceinline__ void fft_row_twiddles(float2* twl, const float2* tw, 
 
 template <int L, int S, int DIR>
 __device__ __forceinline__ void fft_row_stage(float2 (&x)[fft_elems(L)], int p, float2* row,
-                                              const float2* __restrict__ twl) {
+                                              const float2* __restrict__ twl, int bar) {
     constexpr int E = fft_elems(L);
     constexpr int P = L / E;
     constexpr int R = fft_radix(L, S);
@@ -321,28 +330,29 @@ __device__ __forceinline__ void fft_row_stage(float2 (&x)[fft_elems(L)], int p, 
 #pragma unroll
         for (int i = 0; i < E; ++i) x[i] = y[i];
     } else {
-        __syncwarp();
+        row_sync<P>(bar);
 #pragma unroll
         for (int i = 0; i < E; ++i) x[i] = row[xpad(p + P * i)];
-        __syncwarp();
+        row_sync<P>(bar);
     }
 }
 
 template <int L, int S, int DIR>
 __device__ __forceinline__ void fft_row_stages(float2 (&x)[fft_elems(L)], int p, float2* row,
-                                               const float2* __restrict__ twl) {
+                                               const float2* __restrict__ twl, int bar) {
     if constexpr (S < fft_nstages(L)) {
-        fft_row_stage<L, S, DIR>(x, p, row, twl);
-        fft_row_stages<L, S + 1, DIR>(x, p, row, twl);
+        fft_row_stage<L, S, DIR>(x, p, row, twl, bar);
+        fft_row_stages<L, S + 1, DIR>(x, p, row, twl, bar);
     }
 }
 
 // Full length-L transform of one row held by P lanes (exchange buffer `row`,
-// padded layout). Every lane of the warp must call it the same number of times.
+// padded layout). Every lane of the warp (for P > 32: of the team with named
+// barrier `bar`) must call it the same number of times.
 template <int L, int DIR>
 __device__ __forceinline__ void fft_row(float2 (&x)[fft_elems(L)], int p, float2* row,
-                                        const float2* __restrict__ twl) {
-    fft_row_stages<L, 0, DIR>(x, p, row, twl);
+                                        const float2* __restrict__ twl, int bar = 0) {
+    fft_row_stages<L, 0, DIR>(x, p, row, twl, bar);
 }
 
 

@@ -267,7 +267,7 @@ __device__ void q_tile(const QStage& st, long long tile, float2* sm, bool tr) {
         case Q_ZR2C: q_zr2c<N>(st, tile, sm, tr); break;
         case Q_Z: {
             const bool band = st.z.z.band > 0;
-            if constexpr (RowCfg<N>::ok) {   // power-of-two rows: the z pass of k_zrow (staged partners, prefetch)
+            if constexpr ((N & (N - 1)) == 0) {   // power-of-two rows: the z pass of k_zrow (staged partners, prefetch)
                 constexpr long long one = 1LL << 40;   // a stride past every group: one group per warp
                 const long long g0 = tile * (kQueueThreads / 32);
                 if (st.z.ntargets == 0) {
@@ -415,7 +415,7 @@ k_queue(const QStage* __restrict__ stages, const long long* __restrict__ starts,
 
 template <int N>
 constexpr size_t q_smem_n() {
-    constexpr size_t z = RowCfg<N>::ok ? RowCfg<N>::smem(2) : QRow<N>::smem;
+    constexpr size_t z = (N & (N - 1)) == 0 ? RowCfg<N>::smem(kMaxPartners) : QRow<N>::smem;
     return z > col_smem<N>() ? z : col_smem<N>();
 }
 

@@ -939,21 +939,44 @@ k_zexp_pairs(ZPairArgs args, const float2* __restrict__ twg, float kF) {
 // The only block barrier follows the twiddle table set-up. Persistent grid:
 // each warp strides over the row groups. Results are bitwise those of the
 // tile kernels (same transform arithmetic, same accumulation order).
+//
+// Rows of 12 elements a thread (N = 3 * 2^a) and rows of 64 lanes (N = 1024, a
+// team of two warps ordered by a named barrier) take the same form: the tile
+// kernels' block barriers at 8 warps a block leave the SM waiting (1024^3: a
+// tile c2r z launch of 8.6 GB takes 3.55 ms, the c2r 9.28 ms against 7.18 here). Recursion, tile z
+// passes -> warp rows: 192^3 3.15 -> 2.60 ms, 384^3 24.3 -> 16.5, 768^3 (third
+// order) 108 -> 72, 1024^3 (second order) 78.5 -> 52.7.
 constexpr int kRowWarps = 8;
 
 template <int N>
 struct RowCfg {
     static constexpr int M = N / 2, E = fft_elems(M), P = M / E;
-    static constexpr bool ok = (M & (M - 1)) == 0 && P <= 32 && 32 % P == 0;
-    static constexpr int RW = ok ? 32 / P : 1;               // rows per warp
+    static constexpr int TL = P > 32 ? P : 32;               // lanes of a team (the threads that share rows)
+    static constexpr int RW = P <= TL ? TL / P : 1;          // rows per team
+    static constexpr bool ok = P <= 64 && TL % P == 0 && (N * N) % RW == 0;
     static constexpr int XROW = M + (M >> 4);                 // padded exchange row
     static constexpr int NTW = fft_row_tw_total<M>();
     static constexpr int HDR = ((NTW + E) * P + 1) / 2 * 2;   // twiddle tables, 16-byte multiple
     static constexpr int MAXP = kMaxPartners;
-    static constexpr int WIN = RW * M;                        // input rows of a warp
-    // per warp: two input buffers (current, next), MAXP partner buffers, exchange rows
-    __host__ __device__ static constexpr int wstride(int nt) { return WIN * (2 + (nt ? MAXP : 0)) + RW * XROW; }
-    static constexpr size_t smem(int nt) { return sizeof(float2) * (HDR + (size_t)kRowWarps * wstride(nt)); }
+    static constexpr int WIN = RW * M;                        // input rows of a team
+    static constexpr int PIECES = WIN / (2 * TL);             // 16-byte pieces of them per lane
+    static_assert(!ok || (WIN % (2 * TL) == 0 && (RW * XROW) % 2 == 0), "16-byte row copies by the team's lanes");
+    // per team: two input buffers (current, next), exchange rows, np partner buffers
+    __host__ __device__ static constexpr int wstride(int np) { return WIN * (2 + np) + RW * XROW; }
+    static constexpr size_t smem(int np, int warps = kRowWarps) {
+        return sizeof(float2) * (HDR + (size_t)(warps * 32 / TL) * wstride(np));
+    }
+};
+
+// Warps per block and blocks per SM of k_zrow. Eight elements a thread: 8
+// warps, two blocks (128 registers; three without accumulators). Twelve
+// elements a thread: two targets hold 96 accumulator registers, so one block
+// of up to 12 warps (168 registers; 11 where the shared buffers of 12 do not fit).
+template <int N, int NT>
+struct ZRowLaunch {
+    static constexpr bool big = RowCfg<N>::E > 8;
+    static constexpr int WARPS = big && NT == 2 ? (RowCfg<N>::smem(kMaxPartners, 12) <= 232448 ? 12 : 11) : kRowWarps;
+    static constexpr int MINB = big ? (NT == 2 ? 1 : 2) : (NT == 0 ? 3 : 2);
 };
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
@@ -980,27 +1003,28 @@ __device__ __forceinline__ void zrow_tables(float2* twl, float2* twp, const floa
     __syncthreads();
 }
 
-// Body of the warp-row z pass: warp w of the block handles the row groups
-// grp0 + w, grp0 + w + gstride, ... (the kernel: grp0 = blockIdx.x * kRowWarps,
-// gstride = gridDim.x * kRowWarps; a tile of the persistent queue: one group
-// per warp). Inputs, partners and partial sums are read through L2 (cp.async.cg
+// Body of the warp-row z pass: team w of the block (a warp, or two for P = 64)
+// handles the row groups grp0 + w, grp0 + w + gstride, ... (the kernel: grp0 =
+// blockIdx.x * teams, gstride = gridDim.x * teams; a tile of the persistent
+// queue: one group per warp). maxp: partner buffers per team. Inputs, partners and partial sums are read through L2 (cp.async.cg
 // and ordinary loads), never through the read-only data path, so the body is
 // also correct for fields written earlier in the same launch.
 template <int N, int NT, bool BAND>
 __device__ __forceinline__ void zrow_body(const ZPairArgs& args, const float2* __restrict__ twg, float kF,
-                                          long long grp0, long long gstride, float2* sm, bool table_ready = false) {
+                                          long long grp0, long long gstride, float2* sm, bool table_ready = false,
+                                          int maxp = kMaxPartners) {
     using C = RowCfg<N>;
-    constexpr int M = C::M, E = C::E, P = C::P, RW = C::RW, WIN = C::WIN;
+    constexpr int M = C::M, E = C::E, P = C::P, RW = C::RW, WIN = C::WIN, TL = C::TL, PIECES = C::PIECES;
     constexpr int NA = NT > 0 ? NT : 1;
-    static_assert(C::ok, "warp-row z pass needs P <= 32, 32 % P == 0 and a power-of-two row");
+    static_assert(C::ok, "warp-row z pass needs rows that tile a team of 32 or 64 lanes");
     float2* twl = sm;                                  // [NTW][P] stage twiddles
     float2* twp = twl + C::NTW * P;                    // [E][P] pack twiddles tw[p + P i]
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int r = lane / P, p = lane - r * P;
+    const int lane = threadIdx.x % TL, warp = threadIdx.x / TL;   // of the team, the team
+    const int r = lane / P, p = lane - r * P, bar = 1 + warp;
     if (!table_ready) zrow_tables<N>(twl, twp, twg);
-    float2* wbase = sm + C::HDR + warp * C::wstride(NT);
-    float2* wpt = wbase + 2 * WIN;                                                 // [MAXP][RW][M] partners
-    float2* xrow = wbase + WIN * (NT ? 2 + C::MAXP : 2) + r * C::XROW;              // this row's exchange buffer
+    float2* wbase = sm + C::HDR + warp * C::wstride(maxp);
+    float2* xrow = wbase + 2 * WIN + r * C::XROW;                 // this row's exchange buffer
+    float2* wpt = wbase + 2 * WIN + RW * C::XROW;                 // [maxp][RW][M] partners
     const YZExpArgs& z = args.z;
     // BAND, z.band > 0 (even): inputs nonzero only at kz < B. Only those are
     // read; the rest of the input buffers is zero-filled by the copies, so the
@@ -1009,8 +1033,8 @@ __device__ __forceinline__ void zrow_body(const ZPairArgs& args, const float2* _
     const int B = BAND ? z.band : 0;
     unsigned inb = 0;            // bit u: this lane's 16-byte piece u of a row window lies at kz < B
 #pragma unroll
-    for (int u = 0; u < WIN / 64; ++u)
-        if (B <= 0 || (2 * (lane + 32 * u)) % M < B) inb |= 1u << u;
+    for (int u = 0; u < PIECES; ++u)
+        if (B <= 0 || (2 * (lane + TL * u)) % M < B) inb |= 1u << u;
     const long long rows = (long long)N * N;
     const long long groups = rows / RW;
     const long long fstride2 = args.cells / 2;
@@ -1027,7 +1051,7 @@ __device__ __forceinline__ void zrow_body(const ZPairArgs& args, const float2* _
         for (int f = 0; f < z.nout; ++f) {
             const int code = z.codes[f];
             const int in = code & 255, g = (code >> 8) & 3, cc = (code >> 12) & 3, slot = code >> 16;
-            __syncwarp();                                  // earlier reads of the buffers are done
+            row_sync<P>(bar);                                  // earlier reads of the buffers are done
             int np = 0;
             if constexpr (NT > 0) {
 #pragma unroll
@@ -1039,8 +1063,8 @@ __device__ __forceinline__ void zrow_body(const ZPairArgs& args, const float2* _
                         const float2* src = reinterpret_cast<const float2*>(T.partner) +
                                             (long long)T.pfield[slot][q] * fstride2 + row0 * M;
 #pragma unroll
-                        for (int u = 0; u < WIN / 64; ++u)
-                            cp_async16(wpt + np * WIN + 2 * (lane + 32 * u), src + 2 * (lane + 32 * u));
+                        for (int u = 0; u < PIECES; ++u)
+                            cp_async16(wpt + np * WIN + 2 * (lane + TL * u), src + 2 * (lane + TL * u));
                         ++np;
                     }
                 }
@@ -1050,13 +1074,13 @@ __device__ __forceinline__ void zrow_body(const ZPairArgs& args, const float2* _
                     buf ^= 1;
                 } else {                                   // the warp's first input
                     const float4* src = reinterpret_cast<const float4*>(z.in + in * z.in_stride + row0 * M);
-                    float4 v[WIN / 64];
+                    float4 v[PIECES];
 #pragma unroll
-                    for (int u = 0; u < WIN / 64; ++u)
-                        v[u] = ((inb >> u) & 1u) ? src[lane + 32 * u] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int u = 0; u < PIECES; ++u)
+                        v[u] = ((inb >> u) & 1u) ? src[lane + TL * u] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                    for (int u = 0; u < WIN / 64; ++u) reinterpret_cast<float4*>(wbase + buf * WIN)[lane + 32 * u] = v[u];
-                    __syncwarp();
+                    for (int u = 0; u < PIECES; ++u) reinterpret_cast<float4*>(wbase + buf * WIN)[lane + TL * u] = v[u];
+                    row_sync<P>(bar);
                 }
                 cur = in;
                 have_next = false;
@@ -1069,8 +1093,8 @@ __device__ __forceinline__ void zrow_body(const ZPairArgs& args, const float2* _
                     const float2* src = z.in + nin * z.in_stride + nrow0 * M;
                     float2* dst = wbase + (buf ^ 1) * WIN;
 #pragma unroll
-                    for (int u = 0; u < WIN / 64; ++u)
-                        cp_async16z(dst + 2 * (lane + 32 * u), src + 2 * (lane + 32 * u), (inb >> u) & 1u);
+                    for (int u = 0; u < PIECES; ++u)
+                        cp_async16z(dst + 2 * (lane + TL * u), src + 2 * (lane + TL * u), (inb >> u) & 1u);
                     have_next = true;
                 }
             }
@@ -1099,7 +1123,7 @@ __device__ __forceinline__ void zrow_body(const ZPairArgs& args, const float2* _
                 const float2 Ov = cmul(csub(Xk, Xm), twp[i * P + p]);
                 x[i] = make_float2(Ev.x - Ov.y, Ev.y + Ov.x);
             }
-            fft_row<M, +1>(x, p, xrow, twl);              // x[i]: real cells 2n, 2n + 1, n = p + P i
+            fft_row<M, +1>(x, p, xrow, twl, bar);              // x[i]: real cells 2n, 2n + 1, n = p + P i
             float2* dst = NT > 0 ? (args.store ? reinterpret_cast<float2*>(args.store) + slot * fstride2 : nullptr)
                                  : z.out + slot * z.out_stride;
             if (dst) {
@@ -1107,7 +1131,7 @@ __device__ __forceinline__ void zrow_body(const ZPairArgs& args, const float2* _
                 for (int i = 0; i < E; ++i) dst[row * M + p + P * i] = x[i];
             }
             cp_async_wait_all();
-            __syncwarp();                                  // partner and next-input rows of every lane have landed
+            row_sync<P>(bar);                                  // partner and next-input rows of every lane have landed
             if constexpr (NT > 0) {
                 np = 0;
 #pragma unroll
@@ -1158,10 +1182,12 @@ __device__ __forceinline__ void zrow_body(const ZPairArgs& args, const float2* _
 }
 
 template <int N, int NT, bool BAND>
-__global__ void __launch_bounds__(kRowWarps * 32, NT == 0 ? 3 : 2)
-k_zrow(const __grid_constant__ ZPairArgs args, const float2* __restrict__ twg, float kF) {
+__global__ void __launch_bounds__(ZRowLaunch<N, NT>::WARPS * 32, ZRowLaunch<N, NT>::MINB)
+k_zrow(const __grid_constant__ ZPairArgs args, const float2* __restrict__ twg, float kF, int maxp) {
     extern __shared__ __align__(16) float2 sm[];
-    zrow_body<N, NT, BAND>(args, twg, kF, (long long)blockIdx.x * kRowWarps, (long long)gridDim.x * kRowWarps, sm);
+    constexpr int teams = ZRowLaunch<N, NT>::WARPS * 32 / RowCfg<N>::TL;
+    zrow_body<N, NT, BAND>(args, twg, kF, (long long)blockIdx.x * teams, (long long)gridDim.x * teams, sm, false,
+                           maxp);
 }
 
 // ------------------------------------------------- TMA-staged y expansion
@@ -1424,7 +1450,7 @@ k_zrow_shell(const float2* __restrict__ in, long long in_stride, int band, const
     using C = RowCfg<N>;
     constexpr int M = C::M, E = C::E, P = C::P, RW = C::RW;
     constexpr int G = Cfg<N>::TZZ0;
-    static_assert(C::ok && G % RW == 0, "warp-row shell pass: whole rows per warp and per group");
+    static_assert(C::ok && P <= 32 && G % RW == 0, "warp-row shell pass: whole rows per warp and per group");
     extern __shared__ __align__(16) float2 sm[];
     float2* twl = sm;
     float2* twp = twl + C::NTW * P;
@@ -1495,34 +1521,34 @@ k_zrow_shell(const float2* __restrict__ in, long long in_stride, int band, const
 }
 
 template <int N>
-__global__ void __launch_bounds__(kRowWarps * 32, 3)
+__global__ void __launch_bounds__(kRowWarps * 32, RowCfg<N>::E > 8 ? 2 : 3)
 k_zrow_r2c(const float2* in, float2* out, long long fstride, int count, const float2* __restrict__ twg,
            float scale, int band) {
     using C = RowCfg<N>;
-    constexpr int M = C::M, E = C::E, P = C::P, RW = C::RW;
-    static_assert(C::ok, "warp-row z pass needs P <= 32, 32 % P == 0 and a power-of-two row");
+    constexpr int M = C::M, E = C::E, P = C::P, RW = C::RW, TL = C::TL, TEAMS = kRowWarps * 32 / TL;
+    static_assert(C::ok, "warp-row z pass needs rows that tile a team of 32 or 64 lanes");
     extern __shared__ __align__(16) float2 sm[];
     float2* twl = sm;
     float2* twp = twl + C::NTW * P;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int r = lane / P, p = lane - r * P;
+    const int lane = threadIdx.x % TL, warp = threadIdx.x / TL;
+    const int r = lane / P, p = lane - r * P, bar = 1 + warp;
     zrow_tables<N>(twl, twp, twg);
     float2* xrow = sm + C::HDR + (warp * RW + r) * C::XROW;
     const long long per = (long long)N * N / RW;        // row groups per field
     const long long groups = per * count;
     const float half = 0.5f * scale;
-    for (long long grp = (long long)blockIdx.x * kRowWarps + warp; grp < groups;
-         grp += (long long)gridDim.x * kRowWarps) {
+    for (long long grp = (long long)blockIdx.x * TEAMS + warp; grp < groups;
+         grp += (long long)gridDim.x * TEAMS) {
         const long long fld = grp / per, row = (grp - fld * per) * RW + r;
         const float2* src = in + fld * fstride + row * M;
         float2* dst = out + fld * fstride + row * M;
         float2 x[E];
 #pragma unroll
         for (int i = 0; i < E; ++i) x[i] = src[p + P * i];
-        fft_row<M, -1>(x, p, xrow, twl);
+        fft_row<M, -1>(x, p, xrow, twl, bar);
 #pragma unroll
         for (int i = 0; i < E; ++i) xrow[xpad(p + P * i)] = x[i];
-        __syncwarp();
+        row_sync<P>(bar);
 #pragma unroll
         for (int i = 0; i < E; ++i) {
             const int k = p + P * i;
@@ -1532,7 +1558,7 @@ k_zrow_r2c(const float2* in, float2* out, long long fstride, int count, const fl
             const float2 t = cmul(cconj(twp[i * P + p]), csub(Z, Zr));  // e^{-2 pi i k/N} 2i O[k]
             if (band <= 0 || k < band) dst[k] = make_float2(half * (S.x + t.y), half * (S.y - t.x));
         }
-        __syncwarp();                                    // exchange buffer free for the next row
+        row_sync<P>(bar);                                    // exchange buffer free for the next row
     }
 }
 
@@ -1576,7 +1602,8 @@ struct Launch {
         if constexpr (!C::ok) {
             return cudaErrorNotSupported;
         } else {
-            const size_t smem = sizeof(float2) * (C::HDR + (size_t)kRowWarps * C::RW * C::XROW);
+            constexpr int TEAMS = kRowWarps * 32 / C::TL;
+            const size_t smem = sizeof(float2) * (C::HDR + (size_t)TEAMS * C::RW * C::XROW);
             cudaError_t e = set_smem(k_zrow_r2c<N>, smem);
             if (e != cudaSuccess) return e;
             int dev = 0, sms = 0, per = 0;
@@ -1586,7 +1613,7 @@ struct Launch {
                 cudaSuccess)
                 return e;
             const long long groups = (long long)N * N / C::RW * count;
-            const long long need = (groups + kRowWarps - 1) / kRowWarps;
+            const long long need = (groups + TEAMS - 1) / TEAMS;
             const long long resident = (long long)(per > 0 ? per : 1) * sms;
             k_zrow_r2c<N><<<(unsigned)(need < resident ? need : resident), kRowWarps * 32, smem, s>>>(
                 in, out, fs, count, g.tw, scale, band > 0 && band < M ? band : 0);
@@ -1716,29 +1743,39 @@ struct Launch {
         if constexpr (!C::ok) {
             return cudaErrorNotSupported;
         } else {
-            const size_t smem = C::smem(NT);
+            constexpr int WARPS = ZRowLaunch<N, NT>::WARPS, TEAMS = WARPS * 32 / C::TL;
+            int maxp = 0;                                // partner rows staged for one output
+            for (int sl = 0; sl < 17; ++sl) {
+                int c = 0;
+                for (int t = 0; t < a.ntargets; ++t)
+                    for (int q = 0; q < a.t[t].pcount[sl]; ++q) c += a.t[t].pfield[sl][q] >= 0 ? 1 : 0;
+                maxp = c > maxp ? c : maxp;
+            }
+            const size_t smem = C::smem(maxp, WARPS);
             cudaError_t e = set_smem(k_zrow<N, NT, BAND>, smem);
             if (e != cudaSuccess) return e;
             int dev = 0, sms = 0, per = 0;
             if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
             if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_zrow<N, NT, BAND>, kRowWarps * 32,
+            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_zrow<N, NT, BAND>, WARPS * 32,
                                                                      smem)) != cudaSuccess)
                 return e;
             const long long groups = (long long)N * N / C::RW;
-            const long long need = (groups + kRowWarps - 1) / kRowWarps;
+            const long long need = (groups + TEAMS - 1) / TEAMS;
             const long long resident = (long long)(per > 0 ? per : 1) * sms;
-            k_zrow<N, NT, BAND><<<(unsigned)(need < resident ? need : resident), kRowWarps * 32, smem, s>>>(
-                a, g.tw, kDerivUnit);
+            k_zrow<N, NT, BAND><<<(unsigned)(need < resident ? need : resident), WARPS * 32, smem, s>>>(
+                a, g.tw, kDerivUnit, maxp);
             return cudaGetLastError();
         }
     }
+    static constexpr bool row_shell = RowCfg<N>::ok && RowCfg<N>::P <= 32 && Cfg<N>::TZZ0 % RowCfg<N>::RW == 0 &&
+                                      (N * N) % Cfg<N>::TZZ0 == 0;
     static int shell_blocks() { return (int)(((long long)N * N + TZZ - 1) / TZZ); }
     template <int NF, bool TRI>
     static cudaError_t zrow_shell(const Geo& g, const float2* in, long long st, int band, double* partial,
                                   cudaStream_t s) {
         using C = RowCfg<N>;
-        if constexpr (!C::ok) {
+        if constexpr (!row_shell) {
             return cudaErrorNotSupported;
         } else {
             const size_t smem = sizeof(float2) * (C::HDR + (size_t)kRowWarps * C::RW * C::XROW);
@@ -1771,7 +1808,7 @@ struct Launch {
     // nf: data fields (2: a, b; 3 with tri: a, b, c) plus J when present
     static cudaError_t zshell(const Geo& g, const float2* in, long long st, int band, int nf, int tri,
                               double* partial, cudaStream_t s) {
-        if (g.var[TV_ZEXP] == 2 && RowCfg<N>::ok && TZZ == Cfg<N>::TZZ0) {
+        if (g.var[TV_ZEXP] == 2 && row_shell && TZZ == Cfg<N>::TZZ0) {
             if (tri) return nf == 4 ? zrow_shell<4, true>(g, in, st, band, partial, s)
                                     : zrow_shell<3, true>(g, in, st, band, partial, s);
             return nf == 3 ? zrow_shell<3, false>(g, in, st, band, partial, s)
