@@ -368,6 +368,7 @@ gridspt_status gridspt_multi_destroy(gridspt_multi multi);
  * NULL). It synchronises `stream`. gridspt_set_tuning / gridspt_get_tuning
  * store and read the choices (0 or 1; 0..3 for pass 1; 0..6 for pass 2; 0..2 for passes 3 and 4), e.g.
  * from a cache kept by the caller.
+ * A plan that was neither autotuned nor set uses variants chosen by its N.
  * Results are bitwise identical for all variants: they only change how
  * columns and rows are grouped into thread blocks and warps. */
 gridspt_status gridspt_autotune_scratch_size(gridspt_plan plan, size_t* bytes);

@@ -332,6 +332,15 @@ gridspt_status gridspt_plan_create(const gridspt_desc* d, gridspt_plan* out) {
     } else {
         p->s2_nl = -1;
     }
+    // Pass variants of a plan that is not autotuned (all variants are bitwise
+    // equal). Warp-row z passes from N = 64 on: run_orders (n_max = 5) with tiles
+    // / warp rows takes 0.217 / 0.273 ms at 32^3, 0.312 / 0.367 at 48^3, 0.253 /
+    // 0.236 at 64^3, 0.460 / 0.456 at 96^3, 0.92 / 0.59 at 128^3, 3.15 / 2.60 at
+    // 192^3, 6.38 / 3.90 at 256^3, 41.6 / 29.8 at 512^3. The z forward pass from
+    // N = 256 on: r2c 0.048 / 0.052 ms at 192^3, 0.089 / 0.085 at 256^3, 0.70 /
+    // 0.64 at 512^3.
+    p->geo.var[TV_ZEXP] = N >= 64 ? 2 : 0;
+    p->geo.var[TV_ZR2C] = N >= 256 ? 2 : 0;
     cudaError_t e = cudaGetDevice(&p->device);
     if (e != cudaSuccess) { delete p; return cuda_fail(e, "cudaGetDevice"); }
     // roots of unity of size N, then of every smaller supported size (the

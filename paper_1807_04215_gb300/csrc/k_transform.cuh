@@ -1768,8 +1768,12 @@ struct Launch {
             return cudaGetLastError();
         }
     }
-    static constexpr bool row_shell = RowCfg<N>::ok && RowCfg<N>::P <= 32 && Cfg<N>::TZZ0 % RowCfg<N>::RW == 0 &&
-                                      (N * N) % Cfg<N>::TZZ0 == 0;
+    // The shell z pass runs warp rows from N = 192 on (tile / warp rows: 7.8 /
+    // 22 us at 64, 12 / 37 at 96, 16 / 20 at 128, 49 / 43 at 192, 70 / 57 at 256,
+    // 301 / 201 at 384, 547 / 356 at 512: one warp sums a whole row group, so
+    // small grids have too few warps).
+    static constexpr bool row_shell = RowCfg<N>::ok && RowCfg<N>::P <= 32 && N >= 192 &&
+                                      Cfg<N>::TZZ0 % RowCfg<N>::RW == 0 && (N * N) % Cfg<N>::TZZ0 == 0;
     static int shell_blocks() { return (int)(((long long)N * N + TZZ - 1) / TZZ); }
     template <int NF, bool TRI>
     static cudaError_t zrow_shell(const Geo& g, const float2* in, long long st, int band, double* partial,
