@@ -8,11 +8,20 @@
 // accumulated in FP32. Activations saved for the backward pass, per row:
 // z1[H], a1[H], z2[H], a2[H] as FP32 (a1, a2 hold T-rounded values).
 //
-// At these sizes (B <= 4096 rows, 128 hidden units) the network is latency
-// bound (about 0.3 GFLOP per forward at B = 4096), so the layers are plain
-// shared-memory tiled FP32 FMA loops.
+// What bounds these kernels is latency, not arithmetic: a forward pass of 256
+// rows is 19 MFLOP over 74 KB of weights. So the rows are spread over the SMs
+// (as few as two per block), every weight chunk is copied to shared memory by
+// cp.async ahead of its use, and one thread carries a few independent
+// accumulators. Each output keeps one FMA chain in the order of k, whatever the
+// tile, so results do not depend on the tile chosen.
+// Measured (kernel times, bf16, 3 -> 128 -> 128 -> 160, against 8/16-block
+// kernels that read the weights from global memory in the chains):
+//   forward 256 rows 61 -> 9.5 us, 4096 rows 57 -> 21; backward 256 rows
+//   267 -> 19; mse 41 k elements 26 -> 7; Adam 6.5 (two launches) -> 7.5.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
+#include "fft_core.cuh"
 #include "gridspt_internal.h"
 
 namespace gridspt {
@@ -33,238 +42,446 @@ __device__ __forceinline__ float silu_grad(float z) {
     return s * (1.f + z * (1.f - s));
 }
 
-constexpr int kFwdRows = 32;
-constexpr int kBwdRows = 16;
-constexpr int kThreads = 256;
+constexpr int kGradRows = 16;          // rows of one FMA chain of the parameter gradients
+constexpr int kWBytes = 49152;         // one of the two weight buffers (32-bit 128 x 128 takes two chunks)
 
-// out[r][c] = sum_k in[r][k] W[k][c] + b[c] for r < R, c < C; in, out in
-// shared memory (row pitch K and C); W, b global (T). One thread per (c, row
-// group of 16 rows); the W element is loaded once per k and reused 16 times.
-template <typename T, int R>
-__device__ void dense(const float* __restrict__ in, int K, const T* __restrict__ W, const T* __restrict__ b,
-                      int C, float* __restrict__ out) {
-    constexpr int RG = R / 16;
-    for (int w = threadIdx.x; w < C * RG; w += blockDim.x) {
-        const int c = w % C, g = w / C;
-        float acc[16];
-        const float bc = to_f<T>(b[c]);
-#pragma unroll
-        for (int j = 0; j < 16; ++j) acc[j] = bc;
-        for (int k = 0; k < K; ++k) {
-            const float wk = to_f<T>(W[(long long)k * C + c]);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) acc[j] = fmaf(in[(g * 16 + j) * K + k], wk, acc[j]);
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async16b(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int LEFT>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(LEFT) : "memory"); }
+__device__ __forceinline__ bool aligned_to(const void* p, int bytes) {
+    return (reinterpret_cast<unsigned long long>(p) & (bytes - 1)) == 0;
+}
+
+// Copy rows x C elements (contiguous in global memory) to shared rows of `pitch`
+// elements: 16-byte or 4-byte asynchronous copies where addresses and lengths
+// allow, plain loads otherwise (an odd C of bfloat16).
+template <typename T>
+__device__ void stage_rows(T* dst, int pitch, const T* src, int rows, int C, long long src_pitch) {
+    constexpr int S = sizeof(T), V = 16 / S, W = 4 / S;
+    const int e = C % V == 0 && pitch % V == 0 && src_pitch % V == 0 && aligned_to(src, 16)   ? V
+                  : C % W == 0 && pitch % W == 0 && src_pitch % W == 0 && aligned_to(src, 4) ? W : 1;
+    const int nt = blockDim.x, q = C / e, dr = nt / q, dj = nt - dr * q;   // stepping (r, j): no division per copy
+    int r = threadIdx.x / q, j = threadIdx.x - r * q;
+    while (r < rows) {
+        T* d = dst + r * pitch + j * e;
+        const T* g = src + r * src_pitch + j * e;
+        if (e == V) cp_async16b(d, g);
+        else if (e == W && S * W == 4) cp_async4(d, g);
+        else *d = *g;
+        r += dr;
+        j += dj;
+        if (j >= q) {
+            j -= q;
+            ++r;
         }
-#pragma unroll
-        for (int j = 0; j < 16; ++j) out[(g * 16 + j) * C + c] = acc[j];
     }
 }
+
+// One FMA step of RT rows (pairs): acc[r] += in[r] * w, each lane rounded as fmaf.
+template <int RT>
+__device__ __forceinline__ void fma_rows(float2 (&acc)[RT / 2], const float* in, float w) {
+    if constexpr (RT % 4 == 0) {
+#pragma unroll
+        for (int j = 0; j < RT / 4; ++j) {
+            const float4 v = *reinterpret_cast<const float4*>(in + 4 * j);
+            acc[2 * j] = lfma(w, make_float2(v.x, v.y), acc[2 * j]);
+            acc[2 * j + 1] = lfma(w, make_float2(v.z, v.w), acc[2 * j + 1]);
+        }
+    } else {
+        acc[0] = lfma(w, *reinterpret_cast<const float2*>(in), acc[0]);
+    }
+}
+
+// Forward tiles: R rows per block, RT rows x CT columns per thread. A block has one
+// thread per such piece of the widest layer (at most 1024).
+template <int R> struct FwdTile;
+template <> struct FwdTile<2> { static constexpr int RT = 2, CT = 1; };
+template <> struct FwdTile<8> { static constexpr int RT = 4, CT = 1; };
+template <> struct FwdTile<32> { static constexpr int RT = 4, CT = 2; };
+// row pitch of a transposed activation [k][R]: 16-byte rows, and tasks that write
+// neighbouring columns spread over the banks
+template <int R> __host__ __device__ constexpr int row_pitch() { return R == 2 ? 2 : R + 4; }
+__host__ __device__ constexpr int even(int n) { return (n + 1) & ~1; }
 
 }  // namespace
 
-template <typename T>
-__global__ void __launch_bounds__(kThreads)
+// y = net(x), activations saved. Activations are held transposed ([k][row]) in
+// shared memory, so one 8- or 16-byte load feeds several rows; the weights pass
+// through two buffers in chunks of whole k rows, the next chunk (or the next
+// layer's first) in flight while one is used.
+template <typename T, int R>
+__global__ void __launch_bounds__(256 / FwdTile<R>::CT * (R / FwdTile<R>::RT))
 k_mlp_forward(const float* __restrict__ x, int B, int I, int H, int O, const T* __restrict__ theta,
               float* __restrict__ y, float* __restrict__ act) {
-    extern __shared__ float sm[];
-    float* xs = sm;                      // R x I
-    float* h1 = xs + kFwdRows * I;       // R x H
-    float* h2 = h1 + kFwdRows * H;       // R x H
-    float* ys = h2 + kFwdRows * H;       // R x O
+    constexpr int RT = FwdTile<R>::RT, CT = FwdTile<R>::CT, RP = row_pitch<R>(), G = R / RT;
+    extern __shared__ __align__(16) char smraw[];
+    T* wb[2] = {reinterpret_cast<T*>(smraw), reinterpret_cast<T*>(smraw + kWBytes)};
+    float* hin = reinterpret_cast<float*>(smraw + 2 * kWBytes);    // [max(I, H)][RP], input of the layer
+    float* hout = hin + (H > I ? H : I) * RP;                      // [H][RP]
+    float* bs = hout + H * RP;                                     // b1[H], b2[H], b3[O]
     const T* W1 = theta;
-    const T* b1 = W1 + I * H;
-    const T* W2 = b1 + H;
-    const T* b2 = W2 + H * H;
-    const T* W3 = b2 + H;
-    const T* b3 = W3 + H * O;
-    const int r0 = blockIdx.x * kFwdRows;
-    for (int i = threadIdx.x; i < kFwdRows * I; i += blockDim.x) {
-        const int r = i / I;
-        xs[i] = r0 + r < B ? x[(long long)(r0 + r) * I + (i % I)] : 0.f;
-    }
-    __syncthreads();
-    dense<T, kFwdRows>(xs, I, W1, b1, H, h1);
-    __syncthreads();
-    for (int i = threadIdx.x; i < kFwdRows * H; i += blockDim.x) {
-        const int r = i / H, c = i % H;
-        const float z = h1[i];
-        const float a = round_t<T>(silu(z));
-        if (act && r0 + r < B) {
-            act[(long long)(r0 + r) * 4 * H + c] = z;
-            act[(long long)(r0 + r) * 4 * H + H + c] = a;
-        }
-        h1[i] = a;
-    }
-    __syncthreads();
-    dense<T, kFwdRows>(h1, H, W2, b2, H, h2);
-    __syncthreads();
-    for (int i = threadIdx.x; i < kFwdRows * H; i += blockDim.x) {
-        const int r = i / H, c = i % H;
-        const float z = h2[i];
-        const float a = round_t<T>(silu(z));
-        if (act && r0 + r < B) {
-            act[(long long)(r0 + r) * 4 * H + 2 * H + c] = z;
-            act[(long long)(r0 + r) * 4 * H + 3 * H + c] = a;
-        }
-        h2[i] = a;
-    }
-    __syncthreads();
-    dense<T, kFwdRows>(h2, H, W3, b3, O, ys);
-    __syncthreads();
-    for (int i = threadIdx.x; i < kFwdRows * O; i += blockDim.x) {
-        const int r = i / O;
-        if (r0 + r < B) y[(long long)(r0 + r) * O + (i % O)] = ys[i];
-    }
-}
-
-// Backward of sum(dy * y) for one tile of kBwdRows rows: writes this block's
-// partial gradient (parameter layout) to part + blockIdx.x * n_params.
-template <typename T>
-__global__ void __launch_bounds__(kThreads)
-k_mlp_backward(const float* __restrict__ x, int B, int I, int H, int O, const T* __restrict__ theta,
-               const float* __restrict__ act, const float* __restrict__ dy, float* __restrict__ part) {
-    constexpr int R = kBwdRows;
-    extern __shared__ float sm[];
-    float* xs = sm;              // R x I
-    float* z1 = xs + R * I;      // R x H
-    float* a1 = z1 + R * H;
-    float* z2 = a1 + R * H;
-    float* a2 = z2 + R * H;
-    float* d3 = a2 + R * H;      // R x O
-    float* d2 = d3 + R * O;      // R x H
-    float* d1 = d2 + R * H;      // R x H
-    const T* W1 = theta;
-    const T* b1 = W1 + I * H;
-    const T* W2 = b1 + H;
-    const T* b2 = W2 + H * H;
-    const T* W3 = b2 + H;
-    (void)b2;
-    const long long np = (long long)I * H + H + (long long)H * H + H + (long long)H * O + O;
-    float* g = part + blockIdx.x * np;
-    float* gW1 = g;
-    float* gb1 = gW1 + I * H;
-    float* gW2 = gb1 + H;
-    float* gb2 = gW2 + H * H;
-    float* gW3 = gb2 + H;
-    float* gb3 = gW3 + H * O;
+    const T* W2 = W1 + (long long)I * H + H;
+    const T* W3 = W2 + (long long)H * H + H;
     const int r0 = blockIdx.x * R;
+    // chunk s of the weights in order of use: layer, first k, number of k rows
+    auto layer_w = [&](int l) { return l == 0 ? W1 : l == 1 ? W2 : W3; };
+    auto layer_c = [&](int l) { return l == 2 ? O : H; };
+    auto layer_k = [&](int l) { return l == 0 ? I : H; };
+    auto chunk_k = [&](int l) {
+        const int fit = kWBytes / (even(layer_c(l)) * (int)sizeof(T));
+        return layer_k(l) < fit ? layer_k(l) : fit;
+    };
+    const bool pairs = O % 2 == 0 && aligned_to(y, 8);
+    int nl = 0, nk = 0, nbuf = 0;                                  // next chunk to issue
+    auto issue = [&]() {
+        if (nl < 3) {
+            const int C = layer_c(nl), kc = chunk_k(nl), left = layer_k(nl) - nk, n = left < kc ? left : kc;
+            stage_rows(wb[nbuf], C % (16 / (int)sizeof(T)) == 0 ? C : even(C), layer_w(nl) + (long long)nk * C, n, C, C);
+            nk += n;
+            if (nk == layer_k(nl)) { nk = 0; ++nl; }
+            nbuf ^= 1;
+        }
+        cp_commit();                                               // (an empty group past the end)
+    };
+    issue();
+    issue();
     for (int i = threadIdx.x; i < R * I; i += blockDim.x) {
-        const int r = i / I;
-        xs[i] = r0 + r < B ? x[(long long)(r0 + r) * I + (i % I)] : 0.f;
+        const int r = i / I, k = i - r * I;
+        hin[k * RP + r] = r0 + r < B ? x[(long long)(r0 + r) * I + k] : 0.f;
     }
-    for (int i = threadIdx.x; i < R * H; i += blockDim.x) {
-        const int r = i / H, c = i % H;
-        const bool ok = r0 + r < B;
-        const float* ar = act + (long long)(r0 + r) * 4 * H;
-        z1[i] = ok ? ar[c] : 0.f;
-        a1[i] = ok ? ar[H + c] : 0.f;
-        z2[i] = ok ? ar[2 * H + c] : 0.f;
-        a2[i] = ok ? ar[3 * H + c] : 0.f;
-    }
-    for (int i = threadIdx.x; i < R * O; i += blockDim.x) {
-        const int r = i / O;
-        d3[i] = r0 + r < B ? dy[(long long)(r0 + r) * O + (i % O)] : 0.f;
-    }
+    for (int i = threadIdx.x; i < 2 * H + O; i += blockDim.x)
+        bs[i] = to_f<T>(i < H ? W1[(long long)I * H + i] : i < 2 * H ? W2[(long long)H * H + i - H]
+                                                                     : W3[(long long)H * O + i - 2 * H]);
     __syncthreads();
-    // output layer
-    for (int w = threadIdx.x; w < H * O; w += blockDim.x) {
-        const int h = w / O, o = w % O;
-        float s = 0.f;
-        for (int r = 0; r < R; ++r) s = fmaf(a2[r * H + h], d3[r * O + o], s);
-        gW3[w] = s;
+    int buf = 0;
+    for (int l = 0; l < 3; ++l) {
+        const int K = layer_k(l), C = layer_c(l), kc = chunk_k(l);
+        const int CP = C % (16 / (int)sizeof(T)) == 0 ? C : even(C);
+        const int nc = (C + CT - 1) / CT, ntask = nc * G;         // a warp's tasks: neighbouring columns, one row group
+        const float* bias = bs + l * H;
+        float2 acc[CT][RT / 2];
+        const int t = threadIdx.x, ct = (t % nc) * CT, rt = (t / nc) * RT;
+#pragma unroll
+        for (int q = 0; q < CT; ++q) {
+            const float b = t < ntask && ct + q < C ? bias[ct + q] : 0.f;
+#pragma unroll
+            for (int j = 0; j < RT / 2; ++j) acc[q][j] = make_float2(b, b);
+        }
+        for (int k0 = 0; k0 < K; k0 += kc) {
+            const int n = K - k0 < kc ? K - k0 : kc;
+            cp_wait<1>();
+            __syncthreads();                                       // this chunk and the layer's input are in place
+            if (t < ntask) {
+                const T* w = wb[buf] + ct;
+                const float* in = hin + k0 * RP + rt;
+#pragma unroll 8
+                for (int k = 0; k < n; ++k, w += CP, in += RP) {
+                    if constexpr (CT == 1) {
+                        fma_rows<RT>(acc[0], in, to_f<T>(*w));
+                    } else if constexpr (sizeof(T) == 2) {         // CP is even: two neighbouring columns
+                        const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(w);
+                        fma_rows<RT>(acc[0], in, __low2float(v));
+                        fma_rows<RT>(acc[CT - 1], in, __high2float(v));
+                    } else {
+                        const float2 v = *reinterpret_cast<const float2*>(w);
+                        fma_rows<RT>(acc[0], in, v.x);
+                        fma_rows<RT>(acc[CT - 1], in, v.y);
+                    }
+                }
+            }
+            __syncthreads();                                       // the buffer (and, at the end, hin) is free
+            issue();
+            buf ^= 1;
+        }
+        if (t < ntask && CT == 2 && l == 2 && pairs) {             // both columns of a row in one store
+#pragma unroll
+            for (int j = 0; j < RT; ++j)
+                if (r0 + rt + j < B)
+                    *reinterpret_cast<float2*>(y + (long long)(r0 + rt + j) * O + ct) =
+                        (j & 1) ? make_float2(acc[0][j / 2].y, acc[CT - 1][j / 2].y)
+                                : make_float2(acc[0][j / 2].x, acc[CT - 1][j / 2].x);
+        } else if (t < ntask) {
+#pragma unroll
+            for (int q = 0; q < CT; ++q) {
+                const int c = ct + q;
+                if (c >= C) continue;
+                float a[RT];
+#pragma unroll
+                for (int j = 0; j < RT; ++j) {
+                    const int row = r0 + rt + j;
+                    const float z = (j & 1) ? acc[q][j / 2].y : acc[q][j / 2].x;
+                    if (l == 2) {
+                        if (row < B) y[(long long)row * O + c] = z;
+                    } else {
+                        a[j] = round_t<T>(silu(z));
+                        if (act && row < B) {
+                            act[(long long)row * 4 * H + 2 * l * H + c] = z;
+                            act[(long long)row * 4 * H + (2 * l + 1) * H + c] = a[j];
+                        }
+                    }
+                }
+                if (l < 2) {
+                    if constexpr (RT % 4 == 0) {
+#pragma unroll
+                        for (int j = 0; j < RT; j += 4)
+                            *reinterpret_cast<float4*>(hout + c * RP + rt + j) = make_float4(a[j], a[j + 1], a[j + 2], a[j + 3]);
+                    } else {
+                        *reinterpret_cast<float2*>(hout + c * RP + rt) = make_float2(a[0], a[1]);
+                    }
+                }
+            }
+        }
+        float* sw = hin;
+        hin = hout;
+        hout = sw;
     }
-    for (int o = threadIdx.x; o < O; o += blockDim.x) {
-        float s = 0.f;
-        for (int r = 0; r < R; ++r) s += d3[r * O + o];
-        gb3[o] = s;
-    }
-    for (int w = threadIdx.x; w < R * H; w += blockDim.x) {
-        const int r = w / H, h = w % H;
-        float s = 0.f;
-        for (int o = 0; o < O; ++o) s = fmaf(d3[r * O + o], to_f<T>(W3[(long long)h * O + o]), s);
-        d2[w] = s * silu_grad(z2[w]);
-    }
-    __syncthreads();
-    // second hidden layer
-    for (int w = threadIdx.x; w < H * H; w += blockDim.x) {
-        const int k = w / H, h = w % H;
-        float s = 0.f;
-        for (int r = 0; r < R; ++r) s = fmaf(a1[r * H + k], d2[r * H + h], s);
-        gW2[w] = s;
-    }
-    for (int h = threadIdx.x; h < H; h += blockDim.x) {
-        float s = 0.f;
-        for (int r = 0; r < R; ++r) s += d2[r * H + h];
-        gb2[h] = s;
-    }
-    for (int w = threadIdx.x; w < R * H; w += blockDim.x) {
-        const int r = w / H, k = w % H;
-        float s = 0.f;
-        for (int h = 0; h < H; ++h) s = fmaf(d2[r * H + h], to_f<T>(W2[(long long)k * H + h]), s);
-        d1[w] = s * silu_grad(z1[w]);
-    }
-    __syncthreads();
-    // first layer
-    for (int w = threadIdx.x; w < I * H; w += blockDim.x) {
-        const int i = w / H, h = w % H;
-        float s = 0.f;
-        for (int r = 0; r < R; ++r) s = fmaf(xs[r * I + i], d1[r * H + h], s);
-        gW1[w] = s;
-    }
-    for (int h = threadIdx.x; h < H; h += blockDim.x) {
-        float s = 0.f;
-        for (int r = 0; r < R; ++r) s += d1[r * H + h];
-        gb1[h] = s;
-    }
-    (void)W1;
 }
 
-// grad[i] = sum over blocks (in order) of part[b][i]
-__global__ void k_mlp_reduce(const float* __restrict__ part, int nblocks, long long np, float* __restrict__ grad) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < np; i += (long long)gridDim.x * blockDim.x) {
-        float s = 0.f;
-        for (int b = 0; b < nblocks; ++b) s += part[b * np + i];
-        grad[i] = s;
+// Deltas of the hidden layers for R rows per block, d2 = (dy W3^T) silu'(z2) and
+// d1 = (d2 W2^T) silu'(z1), to [row][H] scratch. The weights' rows are staged
+// with an odd pitch in 4-byte words, so the threads of a warp (one hidden unit
+// each) read distinct banks; the chain of an output runs over the columns in
+// order, in chunks where a row block does not fit a buffer.
+template <typename T, int R>
+__global__ void __launch_bounds__(R == 2 ? 256 : 512)
+k_mlp_delta(int row0, int row1, int I, int H, int O, const T* __restrict__ theta, const float* __restrict__ act,
+            const float* __restrict__ dy, float* __restrict__ d2, float* __restrict__ d1) {
+    constexpr int RT = R == 2 ? 2 : 4, G = R / RT, RP = row_pitch<R>();
+    constexpr int W = 4 / (int)sizeof(T);
+    extern __shared__ __align__(16) char smraw[];
+    T* wb[2] = {reinterpret_cast<T*>(smraw), reinterpret_cast<T*>(smraw + kWBytes)};
+    float* din = reinterpret_cast<float*>(smraw + 2 * kWBytes);    // [max(O, H)][RP]
+    float* dmid = din + (O > H ? O : H) * RP;                      // [H][RP]
+    const T* W2 = theta + (long long)I * H + H;
+    const T* W3 = W2 + (long long)H * H + H;
+    const int r0 = row0 + blockIdx.x * R;
+    // columns per chunk: an even number, pitch = columns + one or two words (odd in words)
+    auto cols = [&](int l) {
+        int n = kWBytes / (H * (int)sizeof(T)) - 2 * W - 2;
+        n &= ~(2 * W - 1);
+        const int all = l ? H : O;
+        return all < n ? all : n;
+    };
+    auto pitch = [&](int n) {                                      // elements; odd in 4-byte words
+        const int words = (n + W - 1) / W;
+        return (words | 1) * W;
+    };
+    int nl = 0, nk = 0, nbuf = 0;
+    auto issue = [&]() {
+        if (nl < 2) {
+            const int all = nl ? H : O, kc = cols(nl), n = all - nk < kc ? all - nk : kc;
+            stage_rows(wb[nbuf], pitch(kc), (nl ? W2 : W3) + nk, H, n, (long long)all);
+            nk += n;
+            if (nk == all) { nk = 0; ++nl; }
+            nbuf ^= 1;
+        }
+        cp_commit();
+    };
+    issue();
+    issue();
+    for (int i = threadIdx.x; i < R * O; i += blockDim.x) {
+        const int r = i / O, o = i - r * O;
+        din[o * RP + r] = r0 + r < row1 ? dy[(long long)(r0 + r) * O + o] : 0.f;
     }
+    int buf = 0;
+    for (int l = 0; l < 2; ++l) {
+        const int K = l ? H : O, kc = cols(l), WP = pitch(kc);
+        const int h = threadIdx.x % H, rt = (threadIdx.x / H) * RT;
+        const bool on = threadIdx.x < H * G;
+        float2 acc[RT / 2];
+        float z[RT];                                               // read before the chain hides their latency
+#pragma unroll
+        for (int j = 0; j < RT; ++j) {
+            const int row = r0 + rt + j;
+            z[j] = on && row < row1 ? act[(long long)row * 4 * H + (l ? 0 : 2) * H + h] : 0.f;
+            if (j % 2 == 0) acc[j / 2] = make_float2(0.f, 0.f);
+        }
+        for (int k0 = 0; k0 < K; k0 += kc) {
+            const int n = K - k0 < kc ? K - k0 : kc;
+            cp_wait<1>();
+            __syncthreads();
+            if (on) {
+                const float* in = (l ? dmid : din) + k0 * RP + rt;
+                const T* w = wb[buf] + h * WP;
+                int k = 0;
+                if constexpr (sizeof(T) == 2) {
+#pragma unroll 4
+                    for (; k + 1 < n; k += 2) {
+                        const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(w + k);
+                        fma_rows<RT>(acc, in + k * RP, __low2float(v));
+                        fma_rows<RT>(acc, in + (k + 1) * RP, __high2float(v));
+                    }
+                }
+#pragma unroll 8
+                for (; k < n; ++k) fma_rows<RT>(acc, in + k * RP, to_f<T>(w[k]));
+            }
+            __syncthreads();
+            issue();
+            buf ^= 1;
+        }
+        if (on) {
+#pragma unroll
+            for (int j = 0; j < RT; ++j) {
+                const int row = r0 + rt + j;
+                const float s = (j & 1) ? acc[j / 2].y : acc[j / 2].x;
+                float d = 0.f;
+                if (row < row1) {
+                    d = s * silu_grad(z[j]);
+                    (l ? d1 : d2)[(long long)(row - row0) * H + h] = d;
+                }
+                if (l == 0) dmid[h * RP + rt + j] = d;
+            }
+        }
+    }
+}
+
+// Parameter gradients as 16 x 16 tiles of the three products (rows contracted):
+// W3: a2^T dy, W2: a1^T d2, W1: x^T d1; one element a thread, the next 64 rows
+// loaded into registers while the current ones are summed. Rows are summed in
+// chains of 16, the chains added in row order (on top of the values already in
+// grad unless `first`); tiles of the first k rows add the bias sums.
+constexpr int kGT = 16, kGChunk = 64;
+__global__ void __launch_bounds__(kGT * kGT)
+k_mlp_grad(const float* __restrict__ x, int row0, int row1, int I, int H, int O, const float* __restrict__ act,
+           const float* __restrict__ dy, const float* __restrict__ d2, const float* __restrict__ d1, int first,
+           float* __restrict__ grad) {
+    constexpr int PER = kGChunk / kGT;
+    __shared__ float ls[2][kGChunk][kGT], rs[2][kGChunk][kGT];
+    const int th = (H + kGT - 1) / kGT, to = (O + kGT - 1) / kGT;
+    int b = blockIdx.x, layer, kt, nt;
+    if (b < th * to) { layer = 2; kt = b / to; nt = b % to; }
+    else if ((b -= th * to) < th * th) { layer = 1; kt = b / th; nt = b % th; }
+    else { layer = 0; kt = 0; nt = b - th * th; }
+    const int K = layer == 0 ? I : H, C = layer == 2 ? O : H;
+    float* gw = grad + (layer == 0 ? 0 : layer == 1 ? (long long)I * H + H : (long long)I * H + 2 * H + (long long)H * H);
+    float* gb = gw + (long long)K * C;
+    const int tk = threadIdx.x / kGT, tn = threadIdx.x % kGT, k = kt * kGT + tk, n = nt * kGT + tn;
+    // this thread loads rows tk + 16 q of the chunk: left column lk, right column n
+    const int lk = kt * kGT + tn;
+    const bool lok = lk < K, rok = n < C, live = k < K && rok, bias = kt == 0 && tk == 0 && rok;
+    const int lp = layer == 0 ? I : 4 * H, rp = C;
+    const float* left = (layer == 0 ? x : act + (layer == 1 ? H : 3 * H)) + (long long)(row0 + tk) * lp + lk;
+    const float* right = (layer == 2 ? dy + (long long)row0 * rp : layer == 1 ? d2 : d1) + (long long)tk * rp + n;
+    const int rows = row1 - row0;
+    float lv[PER], rv[PER];
+    auto load = [&](int c0) {
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const int r = c0 + q * kGT;
+            lv[q] = lok && r + tk < rows ? left[(long long)r * lp] : 0.f;
+            rv[q] = rok && r + tk < rows ? right[(long long)r * rp] : 0.f;
+        }
+    };
+    float tot = first || !live ? 0.f : gw[(long long)k * C + n], tb = first || !bias ? 0.f : gb[n];
+    load(0);
+    int buf = 0;
+    for (int c0 = 0; c0 < rows; c0 += kGChunk) {
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            ls[buf][q * kGT + tk][tn] = lv[q];
+            rs[buf][q * kGT + tk][tn] = rv[q];
+        }
+        __syncthreads();                       // (the other buffer's readers passed the previous barrier's chunk)
+        if (c0 + kGChunk < rows) load(c0 + kGChunk);
+#pragma unroll
+        for (int g = 0; g < kGChunk; g += kGradRows) {
+            if (c0 + g >= rows) break;
+            float s = 0.f, sb = 0.f;
+#pragma unroll
+            for (int r = 0; r < kGradRows; ++r) {
+                const float d = rs[buf][g + r][tn];
+                s = fmaf(ls[buf][g + r][tk], d, s);
+                sb += d;
+            }
+            tot += s;
+            tb += sb;
+        }
+        buf ^= 1;
+    }
+    if (live) gw[(long long)k * C + n] = tot;
+    if (bias) gb[n] = tb;
 }
 
 // Masked mean-squared error: dy = 2 mask (y - t) / sum(mask); loss = sum(mask (y - t)^2) / sum(mask).
-// One block, fixed-order reduction.
+// One cluster of 16 blocks (the sums are needed by every element of dy, and one
+// block alone is bound by its own load latency): block sums by a fixed tree,
+// exchanged through distributed shared memory, added in block order.
+constexpr int kOptCluster = 16;
 __global__ void __launch_bounds__(1024)
 k_mlp_mse(const float* __restrict__ y, const float* __restrict__ t, const float* __restrict__ mask, long long n,
           float* __restrict__ dy, float* __restrict__ loss) {
-    __shared__ float rs[1024], rc[1024];
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ float2 rs[32];
+    __shared__ float2 tot;
+    const long long i0 = (long long)blockIdx.x * 1024 + threadIdx.x, step = 1024LL * kOptCluster;
     float s = 0.f, c = 0.f;
-    for (long long i = threadIdx.x; i < n; i += blockDim.x) {
+#pragma unroll 4
+    for (long long i = i0; i < n; i += step) {
         const float d = (y[i] - t[i]) * mask[i];
         s = fmaf(d, d, s);
         c += mask[i];
     }
-    rs[threadIdx.x] = s;
-    rc[threadIdx.x] = c;
-    __syncthreads();
-    for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-        if (threadIdx.x < h) {
-            rs[threadIdx.x] += rs[threadIdx.x + h];
-            rc[threadIdx.x] += rc[threadIdx.x + h];
-        }
-        __syncthreads();
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        s += __shfl_down_sync(0xffffffffu, s, off);
+        c += __shfl_down_sync(0xffffffffu, c, off);
     }
-    const float cnt = rc[0] > 0.f ? rc[0] : 1.f;
-    for (long long i = threadIdx.x; i < n; i += blockDim.x) dy[i] = 2.f * (y[i] - t[i]) * mask[i] / cnt;
-    if (threadIdx.x == 0 && loss) *loss = rs[0] / cnt;
+    if ((threadIdx.x & 31) == 0) rs[threadIdx.x >> 5] = make_float2(s, c);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        s = rs[threadIdx.x].x;
+        c = rs[threadIdx.x].y;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            s += __shfl_down_sync(0xffffffffu, s, off);
+            c += __shfl_down_sync(0xffffffffu, c, off);
+        }
+        if (threadIdx.x == 0) tot = make_float2(s, c);
+    }
+    cl.sync();
+    if (threadIdx.x < 32) {                                       // block sums, added in block order
+        const float2 v = threadIdx.x < kOptCluster ? *cl.map_shared_rank(&tot, threadIdx.x) : make_float2(0.f, 0.f);
+        s = c = 0.f;
+#pragma unroll
+        for (int b = 0; b < kOptCluster; ++b) {
+            s += __shfl_sync(0xffffffffu, v.x, b);
+            c += __shfl_sync(0xffffffffu, v.y, b);
+        }
+        if (threadIdx.x == 0) rs[0] = make_float2(s, c);
+    }
+    cl.sync();                                                    // rs[0] in place; no block leaves while its sums are read
+    s = rs[0].x;
+    c = rs[0].y;
+    const float cnt = c > 0.f ? c : 1.f;
+#pragma unroll 4
+    for (long long i = i0; i < n; i += step) dy[i] = 2.f * (y[i] - t[i]) * mask[i] / cnt;
+    if (i0 == 0 && loss) *loss = s / cnt;
 }
 
 // Adam (Kingma & Ba 2015) on the FP32 master parameters; the step count lives
-// in device memory (incremented by thread 0 of block 0 after use via a second
-// kernel) so that a captured training step can be replayed.
+// in device memory so that a captured training step can be replayed. One
+// cluster: every block reads the count, and after the cluster barrier one
+// thread increments it (no second launch).
 template <typename T>
-__global__ void k_mlp_adam(float* __restrict__ master, T* __restrict__ lowp, const float* __restrict__ grad,
-                           float* __restrict__ m, float* __restrict__ v, const int* __restrict__ step, long long n,
-                           float lr, float b1, float b2, float eps) {
-    const int t = *step;
+__global__ void __launch_bounds__(1024)
+k_mlp_adam(float* __restrict__ master, T* __restrict__ lowp, const float* __restrict__ grad, float* __restrict__ m,
+           float* __restrict__ v, int* __restrict__ step, long long n, float lr, float b1, float b2, float eps) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int t = *reinterpret_cast<volatile int*>(step) + 1;
+    cl.barrier_arrive();                                          // this thread has read the old count
     const float c1 = 1.f - powf(b1, (float)t), c2 = 1.f - powf(b2, (float)t);
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+#pragma unroll 2
+    for (long long i = (long long)blockIdx.x * 1024 + threadIdx.x; i < n; i += 1024LL * kOptCluster) {
         const float g = grad[i];
         const float mi = b1 * m[i] + (1.f - b1) * g;
         const float vi = b2 * v[i] + (1.f - b2) * g * g;
@@ -274,10 +491,8 @@ __global__ void k_mlp_adam(float* __restrict__ master, T* __restrict__ lowp, con
         master[i] = p;
         if (lowp) lowp[i] = from_f<T>(p);
     }
-}
-
-__global__ void k_step_inc(int* step) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) *step += 1;
+    cl.barrier_wait();                                            // every thread has
+    if (blockIdx.x == 0 && threadIdx.x == 0) *step = t;
 }
 
 template <typename T>
@@ -288,10 +503,7 @@ __global__ void k_convert(const float* __restrict__ src, T* __restrict__ dst, lo
 
 // ---------------------------------------------------------------- launchers
 long long mlp_params(int I, int H, int O) { return (long long)I * H + H + (long long)H * H + H + (long long)H * O + O; }
-int mlp_bwd_blocks(int B) { return (B + kBwdRows - 1) / kBwdRows; }
-
-static size_t fwd_smem(int I, int H, int O) { return sizeof(float) * (size_t)kFwdRows * (I + 2 * H + O); }
-static size_t bwd_smem(int I, int H, int O) { return sizeof(float) * (size_t)kBwdRows * (I + 6 * H + O); }
+int mlp_bwd_blocks(int B) { return (B + kGradRows - 1) / kGradRows; }
 
 template <typename K>
 static cudaError_t smem_attr(K k, size_t bytes) {
@@ -299,55 +511,103 @@ static cudaError_t smem_attr(K k, size_t bytes) {
                              : cudaSuccess;
 }
 
-cudaError_t launch_mlp_forward(const float* x, int B, int I, int H, int O, const void* theta, int bf16, float* y,
-                               float* act, cudaStream_t s) {
-    const size_t sm = fwd_smem(I, H, O);
-    const unsigned g = (unsigned)((B + kFwdRows - 1) / kFwdRows);
-    cudaError_t e;
-    if (bf16) {
-        if ((e = smem_attr(k_mlp_forward<__nv_bfloat16>, sm)) != cudaSuccess) return e;
-        k_mlp_forward<__nv_bfloat16><<<g, kThreads, sm, s>>>(x, B, I, H, O, (const __nv_bfloat16*)theta, y, act);
-    } else {
-        if ((e = smem_attr(k_mlp_forward<float>, sm)) != cudaSuccess) return e;
-        k_mlp_forward<float><<<g, kThreads, sm, s>>>(x, B, I, H, O, (const float*)theta, y, act);
-    }
+// Rows per block: two while that gives at most two blocks per SM (304), eight
+// up to eight rows an SM block pair, then 32 (the weights are read once per block).
+static int fwd_rows(int B) { return B <= 608 ? 2 : B <= 2432 ? 8 : 32; }
+
+template <typename T, int R>
+static cudaError_t mlp_forward_r(const float* x, int B, int I, int H, int O, const void* theta, float* y, float* act,
+                                 cudaStream_t s) {
+    const size_t sm = 2 * (size_t)kWBytes +
+                      sizeof(float) * ((size_t)row_pitch<R>() * ((H > I ? H : I) + H) + 2 * H + O);
+    cudaError_t e = smem_attr(k_mlp_forward<T, R>, sm);
+    if (e != cudaSuccess) return e;
+    const int wide = H > O ? H : O, ct = FwdTile<R>::CT;
+    int nt = (((wide + ct - 1) / ct) * (R / FwdTile<R>::RT) + 31) / 32 * 32;
+    if (nt < 256) nt = 256;                                        // the copies want threads too
+    k_mlp_forward<T, R><<<(unsigned)((B + R - 1) / R), nt, sm, s>>>(x, B, I, H, O, static_cast<const T*>(theta),
+                                                                         y, act);
     return cudaGetLastError();
 }
 
+cudaError_t launch_mlp_forward(const float* x, int B, int I, int H, int O, const void* theta, int bf16, float* y,
+                               float* act, cudaStream_t s) {
+    const int r = fwd_rows(B);
+    if (bf16)
+        return r == 2   ? mlp_forward_r<__nv_bfloat16, 2>(x, B, I, H, O, theta, y, act, s)
+               : r == 8 ? mlp_forward_r<__nv_bfloat16, 8>(x, B, I, H, O, theta, y, act, s)
+                        : mlp_forward_r<__nv_bfloat16, 32>(x, B, I, H, O, theta, y, act, s);
+    return r == 2   ? mlp_forward_r<float, 2>(x, B, I, H, O, theta, y, act, s)
+           : r == 8 ? mlp_forward_r<float, 8>(x, B, I, H, O, theta, y, act, s)
+                    : mlp_forward_r<float, 32>(x, B, I, H, O, theta, y, act, s);
+}
+
+template <typename T, int R>
+static cudaError_t mlp_delta_r(int row0, int row1, int I, int H, int O, const void* theta, const float* act,
+                               const float* dy, float* d2, float* d1, cudaStream_t s) {
+    const size_t sm = 2 * (size_t)kWBytes + sizeof(float) * (size_t)row_pitch<R>() * ((O > H ? O : H) + H);
+    cudaError_t e = smem_attr(k_mlp_delta<T, R>, sm);
+    if (e != cudaSuccess) return e;
+    const int need = (H * (R == 2 ? 1 : 2) + 31) / 32 * 32, nt = need < 256 ? 256 : need;
+    k_mlp_delta<T, R><<<(unsigned)((row1 - row0 + R - 1) / R), nt, sm, s>>>(
+        row0, row1, I, H, O, static_cast<const T*>(theta), act, dy, d2, d1);
+    return cudaGetLastError();
+}
+
+// The deltas of as many rows as the workspace holds (all of them unless H + O
+// is below about 30), then the gradient tiles over those rows.
 cudaError_t launch_mlp_backward(const float* x, int B, int I, int H, int O, const void* theta, int bf16,
                                 const float* act, const float* dy, float* part, float* grad, cudaStream_t s) {
-    const size_t sm = bwd_smem(I, H, O);
-    const int nb = mlp_bwd_blocks(B);
+    const long long np = mlp_params(I, H, O), cap = (long long)mlp_bwd_blocks(B) * np / (2 * H);   // rows; np >= 5 H
+    long long rows = cap < B ? cap : B;
+    if (rows < B && rows >= kGradRows) rows -= rows % kGradRows;
+    float* d2 = part;
+    float* d1 = part + rows * H;
+    const int th = (H + kGT - 1) / kGT, to = (O + kGT - 1) / kGT;
     cudaError_t e;
-    if (bf16) {
-        if ((e = smem_attr(k_mlp_backward<__nv_bfloat16>, sm)) != cudaSuccess) return e;
-        k_mlp_backward<__nv_bfloat16><<<nb, kThreads, sm, s>>>(x, B, I, H, O, (const __nv_bfloat16*)theta, act, dy,
-                                                               part);
-    } else {
-        if ((e = smem_attr(k_mlp_backward<float>, sm)) != cudaSuccess) return e;
-        k_mlp_backward<float><<<nb, kThreads, sm, s>>>(x, B, I, H, O, (const float*)theta, act, dy, part);
+    for (long long r0 = 0; r0 < B; r0 += rows) {
+        const int a = (int)r0, b = (int)(r0 + rows < B ? r0 + rows : B);
+        if (b - a <= 608)
+            e = bf16 ? mlp_delta_r<__nv_bfloat16, 2>(a, b, I, H, O, theta, act, dy, d2, d1, s)
+                     : mlp_delta_r<float, 2>(a, b, I, H, O, theta, act, dy, d2, d1, s);
+        else
+            e = bf16 ? mlp_delta_r<__nv_bfloat16, 8>(a, b, I, H, O, theta, act, dy, d2, d1, s)
+                     : mlp_delta_r<float, 8>(a, b, I, H, O, theta, act, dy, d2, d1, s);
+        if (e != cudaSuccess) return e;
+        k_mlp_grad<<<(unsigned)(th * (to + th + 1)), kGT * kGT, 0, s>>>(x, a, b, I, H, O, act, dy, d2, d1, r0 == 0, grad);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const long long np = mlp_params(I, H, O);
-    k_mlp_reduce<<<(unsigned)((np + 255) / 256), 256, 0, s>>>(part, nb, np, grad);
-    return cudaGetLastError();
+    return cudaSuccess;
+}
+
+// One launch of a single cluster of kOptCluster blocks of 1024 threads.
+template <typename... P, typename... A>
+static cudaError_t launch_cluster(void (*k)(P...), cudaStream_t s, A... a) {
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(kOptCluster);
+    c.blockDim = dim3(1024);
+    c.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kOptCluster;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, k, static_cast<P>(a)...);
 }
 
 cudaError_t launch_mlp_mse(const float* y, const float* t, const float* mask, long long n, float* dy, float* loss,
                            cudaStream_t s) {
-    k_mlp_mse<<<1, 1024, 0, s>>>(y, t, mask, n, dy, loss);
-    return cudaGetLastError();
+    return launch_cluster(k_mlp_mse, s, y, t, mask, n, dy, loss);
 }
 
 cudaError_t launch_mlp_adam(float* master, void* lowp, int bf16, const float* grad, float* m, float* v, int* step,
                             long long n, float lr, float b1, float b2, float eps, cudaStream_t s) {
-    k_step_inc<<<1, 32, 0, s>>>(step);
-    const unsigned g = (unsigned)((n + 255) / 256);
-    if (bf16)
-        k_mlp_adam<__nv_bfloat16><<<g, 256, 0, s>>>(master, (__nv_bfloat16*)lowp, grad, m, v, step, n, lr, b1, b2, eps);
-    else
-        k_mlp_adam<float><<<g, 256, 0, s>>>(master, (float*)lowp, grad, m, v, step, n, lr, b1, b2, eps);
-    return cudaGetLastError();
+    return bf16 ? launch_cluster(k_mlp_adam<__nv_bfloat16>, s, master, (__nv_bfloat16*)lowp, grad, m, v, step, n, lr,
+                                 b1, b2, eps)
+                : launch_cluster(k_mlp_adam<float>, s, master, (float*)lowp, grad, m, v, step, n, lr, b1, b2, eps);
 }
 
 cudaError_t launch_mlp_convert(const float* src, void* dst, int bf16, long long n, cudaStream_t s) {
