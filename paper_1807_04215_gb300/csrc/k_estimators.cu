@@ -7,13 +7,19 @@
 // integer ranges of |s|^2 precomputed on the host from the FP64 edges, so
 // the bin decision equals the FP64 test edges[i] <= k_F sqrt(|s|^2).
 //
-// Determinism: one warp per (kx, ky) row, chunks of 32 consecutive kz (two
-// chunks per step, scanned side by side). Along a row the bin index is
+// Rows (kx, ky) with the same {|sx|, |sy|} (up to eight) hold the same |s|^2 at
+// every kz, hence the same bins: a warp adds the terms of one such set lane by
+// lane (kz) first, then bins the sums. Only sets inside the top edge are
+// visited. A scan per row, over all N^2 rows with a 64-bit division each, took
+// 121 us per spectrum at 512^3 (top edge |s| = 127, 69 MB of modes); a set-wise
+// one @POW@ us.
+// Determinism: one warp per set, chunks of 32 consecutive kz (two chunks per
+// step, scanned side by side). Along a row the bin index is
 // non-decreasing in kz, so lanes with equal bins are contiguous: a segmented
 // shuffle scan sums each run and its last lane adds the run to the warp's FP64
 // accumulator (one writer per bin per chunk, chunks in kz order). Warps
 // and blocks are then summed in a fixed order: results are bitwise repeatable.
-// The scan runs in FP32 with each addition's rounding error carried exactly
+// The sums run in FP32 with each addition's rounding error carried exactly
 // (Knuth's two-sum) and added at the tail, so a run's sum is good to about
 // FP32^2 while the FP64 pipe (a small fraction of the FP32 rate here) sees
 // one addition per run; the mode counts are exact in FP32. With the FP64
@@ -29,6 +35,7 @@
 namespace gridspt {
 
 constexpr int kPowWarps = 8;
+constexpr int kPowBlocks = 456;         // blocks launched at most (the scratch holds power_blocks())
 
 int power_blocks(const Geo& g) {
     const long long rows = (long long)g.N * g.N;
@@ -66,9 +73,23 @@ __device__ __forceinline__ void seg_scan(T (&v)[2], T (&e)[2], float (&c)[2], co
     }
 }
 
+// v + x with the rounding error carried in e (T = float), or a plain FP64 add.
 template <typename T>
-__global__ void __launch_bounds__(kPowWarps * 32)
-k_power(const float2* __restrict__ a, const float2* __restrict__ b, BinSpec bins, int N, int M,
+__device__ __forceinline__ void add_term(T& v, T& e, T x) {
+    if constexpr (sizeof(T) == 4) {
+        const float t = __fadd_rn(v, x);
+        const float bv = __fsub_rn(t, v);
+        e = __fadd_rn(e, __fadd_rn(__fsub_rn(v, __fsub_rn(t, bv)), __fsub_rn(x, bv)));
+        v = t;
+    } else {
+        v += x;
+    }
+}
+
+// sets: number of row sets (i, j), 0 <= j <= i < R, in the order t = i (i + 1) / 2 + j
+template <typename T>
+__global__ void __launch_bounds__(kPowWarps * 32, 2)
+k_power(const float2* __restrict__ a, const float2* __restrict__ b, BinSpec bins, int N, int M, int sets,
         double* __restrict__ partial) {
     __shared__ double acc[kPowWarps][2 * kMaxBins];
     __shared__ int thr[kMaxBins + 1];
@@ -78,16 +99,25 @@ k_power(const float2* __restrict__ a, const float2* __restrict__ b, BinSpec bins
     for (int i = threadIdx.x; i <= nb; i += blockDim.x) thr[i] = bins.thr[i];
     __syncthreads();
     const int top = thr[nb];
-    const long long rows = (long long)N * N;
-    for (long long row = (long long)blockIdx.x * kPowWarps + w; row < rows;
-         row += (long long)gridDim.x * kPowWarps) {
-        const int kx = (int)(row / N), ky = (int)(row % N);
-        const int sx = kx < N / 2 ? kx : kx - N;
-        const int sy = ky < N / 2 ? ky : ky - N;
-        const int sxy = sx * sx + sy * sy;
+    const bool same = a == b;
+    for (int t = blockIdx.x * kPowWarps + w; t < sets; t += gridDim.x * kPowWarps) {
+        int i = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+        while (i * (i + 1) / 2 > t) --i;
+        while ((i + 1) * (i + 2) / 2 <= t) ++i;
+        const int j = t - i * (i + 1) / 2;
+        const int sxy = i * i + j * j;
         if (sxy >= top) continue;
-        const float2* ar = a + row * M;
-        const float2* br = b + row * M;
+        // the set's rows: (+-i, +-j) and, for i > j, (+-j, +-i)
+        long long row[8];
+        int nrow = 0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int u = q & 4 ? j : i, v = q & 4 ? i : j;
+            const bool distinct = !((q & 1) && u == 0) && !((q & 2) && v == 0) && !((q & 4) && i == j);
+            const int kx = (q & 1) && u ? N - u : u, ky = (q & 2) && v ? N - v : v;
+            row[q] = distinct ? ((long long)kx * N + ky) * M : -1;
+            nrow += distinct;
+        }
         // two chunks of 32 kz per step: their scans are independent chains
         // (latency hiding); their sums reach acc in chunk order, as one at a time
         for (int kz0 = 0; kz0 < M; kz0 += 64) {
@@ -115,13 +145,22 @@ k_power(const float2* __restrict__ a, const float2* __restrict__ b, BinSpec bins
                 e[h] = T(0);
                 c[h] = 0.f;
                 if (bin[h] >= 0 && bin[h] < nb) {
-                    const float2 x = ar[kz], y = br[kz];
                     const float wgt = kz == 0 ? 1.f : 2.f;
-                    if constexpr (sizeof(T) == 4)
-                        v[h] = wgt * fmaf(x.x, y.x, x.y * y.y);
-                    else
-                        v[h] = (double)wgt * ((double)x.x * (double)y.x + (double)x.y * (double)y.y);
-                    c[h] = wgt;
+                    c[h] = wgt * (float)nrow;
+                    float2 x[8], y[8];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        x[q] = row[q] >= 0 ? a[row[q] + kz] : make_float2(0.f, 0.f);
+                        y[q] = same ? x[q] : row[q] >= 0 ? b[row[q] + kz] : make_float2(0.f, 0.f);
+                    }
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        if constexpr (sizeof(T) == 4)
+                            add_term<T>(v[h], e[h], wgt * fmaf(x[q].x, y[q].x, x[q].y * y[q].y));
+                        else
+                            add_term<T>(v[h], e[h], (double)wgt * ((double)x[q].x * (double)y[q].x +
+                                                                   (double)x[q].y * (double)y[q].y));
+                    }
                 }
             }
             seg_scan<T>(v, e, c, bin, lane);
@@ -130,7 +169,8 @@ k_power(const float2* __restrict__ a, const float2* __restrict__ b, BinSpec bins
                 const int nxt = __shfl_down_sync(0xffffffffu, bin[h], 1);
                 const bool tail = (lane == 31) || (nxt != bin[h]);
                 if (tail && bin[h] >= 0 && bin[h] < nb) {
-                    acc[w][bin[h]] += (double)v[h] + (double)e[h];
+                    // (the error of an infinite sum is not a number)
+                    acc[w][bin[h]] += isinf(v[h]) ? (double)v[h] : (double)v[h] + (double)e[h];
                     acc[w][kMaxBins + bin[h]] += (double)c[h];
                 }
                 __syncwarp();
@@ -182,11 +222,16 @@ k_power_final(const double* __restrict__ partial, int G, int nb, double vol,
 cudaError_t launch_power(const Geo& g, const float2* a, const float2* b, const BinSpec& bins,
                          double* partial, double* p_out, int64_t* nk_out, double volume,
                          cudaStream_t s) {
-    const int G = power_blocks(g);
+    // row sets with i below the top edge: R = smallest integer with R^2 >= top
+    int R = 0;
+    while (R < g.M && R * R < bins.thr[bins.nbins]) ++R;
+    const int sets = R * (R + 1) / 2;
+    const int need = (sets + kPowWarps - 1) / kPowWarps, most = power_blocks(g) < kPowBlocks ? power_blocks(g) : kPowBlocks;
+    const int G = need < 1 ? 1 : need < most ? need : most;
     if (g.accum == kAccumFp64)
-        k_power<double><<<G, kPowWarps * 32, 0, s>>>(a, b, bins, g.N, g.M, partial);
+        k_power<double><<<G, kPowWarps * 32, 0, s>>>(a, b, bins, g.N, g.M, sets, partial);
     else
-        k_power<float><<<G, kPowWarps * 32, 0, s>>>(a, b, bins, g.N, g.M, partial);
+        k_power<float><<<G, kPowWarps * 32, 0, s>>>(a, b, bins, g.N, g.M, sets, partial);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_power_final<<<bins.nbins, 256, 0, s>>>(partial, G, bins.nbins, volume, p_out, nk_out, g.status);
