@@ -33,7 +33,9 @@ struct gridspt_plan_s {
     long long pb_top = -1;  // cache of the last power-launch byte count (profiling only)
     double pb_modes = 0.0;
     double* j3 = nullptr;   // device [kMaxBins]: sum_x J^3 per bispectrum shell (data independent)
-    double* ic_table = nullptr;   // device [ic_s2 + 1]: mode amplitude per |s|^2 (same allocation as j3)
+    float4* ic_angles = nullptr;  // device: angle, then logarithm table of the initial field (same allocation as j3)
+    double* ic_parts = nullptr;   // device [kIcParts]: partial sums of the sigma_8 integral (same allocation)
+    float2* ic_table = nullptr;   // device [ic_s2 + 1]: mode amplitude per |s|^2 (same allocation)
     long long ic_s2 = 0;
     int* status = nullptr;  // device status word (bounded waits that gave up)
     int j3_nb = 0;          // shells the cache holds (0: empty) and their thresholds
@@ -235,6 +237,11 @@ double sigma8_sq_unit(const gridspt_cosmo* c) {
     return h / 3.0 * s / (2.0 * M_PI * M_PI);
 }
 
+gridspt_status check_spectrum(const gridspt_cosmo* c) {
+    if (!(c->sigma8 > 0) || !(gamma_of(c) > 0)) return fail(GRIDSPT_E_INVALID, "sigma8 and Gamma must be > 0");
+    return GRIDSPT_OK;
+}
+
 gridspt_status check_plan(gridspt_plan p) {
     if (!p) return fail(GRIDSPT_E_INVALID, "plan is NULL");
     return GRIDSPT_OK;
@@ -360,21 +367,39 @@ gridspt_status gridspt_plan_create(const gridspt_desc* d, gridspt_plan* out) {
     e = cudaMalloc(&p->tw, sizeof(float2) * tw.size());
     if (e != cudaSuccess) { delete p; return fail(GRIDSPT_E_NOMEM, "twiddle table: %s", cudaGetErrorString(e)); }
     // one small block: the shell cache (kMaxBins doubles), the status word (4
-    // ints) and the initial field's amplitude table (|s|^2 = 0..ic_s2)
+    // ints), the initial field's angle and logarithm tables, its partial sums
+    // and its amplitude table (|s|^2 = 0..ic_s2)
+    std::vector<float> ict;
+    auto pairs = [&ict](double u, double v) {
+        const float uh = (float)u, vh = (float)v;
+        for (float x : {uh, vh, (float)(u - uh), (float)(v - vh)}) ict.push_back(x);
+    };
+    for (int j = 0; j < kIcAngles; ++j) pairs(std::cos(2.0 * M_PI * j / kIcAngles), std::sin(2.0 * M_PI * j / kIcAngles));
+    for (int i = 128; i <= 256; ++i) {
+        const double v = -std::log((double)((131072 + i / 2) / i) / 512.0);
+        ict.push_back((float)v);
+        ict.push_back((float)(v - (float)v));
+    }
+    static_assert((4 * kIcAngles + 2 * kIcLogs) % 2 == 0, "whole doubles");
+    const size_t ic_head = kMaxBins + 2 + ict.size() / 2 + kIcParts;
     p->ic_s2 = std::min<long long>(p->s2_lin, 3LL * (N / 2) * (N / 2));
     e = fault_inject("plan_alloc") ? cudaErrorMemoryAllocation
-                                   : cudaMalloc(&p->j3, sizeof(double) * (kMaxBins + 2 + p->ic_s2 + 1));
+                                   : cudaMalloc(&p->j3, sizeof(double) * (ic_head + p->ic_s2 + 1));
     if (e != cudaSuccess) {
         cudaFree(p->tw);
         delete p;
         return fail(GRIDSPT_E_NOMEM, "shell cache: %s", cudaGetErrorString(e));
     }
     p->status = reinterpret_cast<int*>(p->j3 + kMaxBins);
-    p->ic_table = p->j3 + kMaxBins + 2;
+    p->ic_angles = reinterpret_cast<float4*>(p->j3 + kMaxBins + 2);
+    p->ic_parts = p->j3 + kMaxBins + 2 + ict.size() / 2;
+    p->ic_table = reinterpret_cast<float2*>(p->j3 + ic_head);
     p->geo.status = p->status;
     e = cudaMemset(p->status, 0, sizeof(int));
     if (e != cudaSuccess) { cudaFree(p->tw); cudaFree(p->j3); delete p; return cuda_fail(e, "status word"); }
     e = cudaMemcpy(p->tw, tw.data(), sizeof(float2) * tw.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(p->ic_angles, ict.data(), sizeof(float) * ict.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) { cudaFree(p->tw); cudaFree(p->j3); delete p; return cuda_fail(e, "twiddle upload"); }
     p->geo.tw = p->tw;
     *out = p;
@@ -405,7 +430,7 @@ gridspt_status gridspt_workspace_size(gridspt_plan p, size_t* bytes) {
 
 gridspt_status gridspt_linear_amplitude(const gridspt_cosmo* c, double* A) {
     if (!c || !A) return fail(GRIDSPT_E_INVALID, "cosmo/A is NULL");
-    if (!(c->sigma8 > 0) || !(gamma_of(c) > 0)) return fail(GRIDSPT_E_INVALID, "sigma8 and Gamma must be > 0");
+    if (gridspt_status st = check_spectrum(c)) return st;
     *A = c->sigma8 * c->sigma8 / sigma8_sq_unit(c);
     return GRIDSPT_OK;
 }
@@ -417,10 +442,12 @@ gridspt_status gridspt_make_linear_field(gridspt_plan p, const gridspt_cosmo* c,
     if (!c || !seeds || !delta1_k) return fail(GRIDSPT_E_INVALID, "NULL argument");
     if (!aligned16(delta1_k)) return fail(GRIDSPT_E_INVALID, "delta1_k not 16-byte aligned");
     if (gridspt_status st = set_device(p)) return st;
-    double A = 0.0;
-    if (gridspt_status st = gridspt_linear_amplitude(c, &A)) return st;
+    if (gridspt_status st = check_spectrum(c)) return st;
     IcArgs a{};
-    a.amp = A;
+    a.sigma8 = c->sigma8;
+    a.angles = p->ic_angles;
+    a.logs = reinterpret_cast<const float2*>(p->ic_angles + kIcAngles);
+    a.parts = p->ic_parts;
     a.n_s = c->n_s;
     a.gamma = gamma_of(c);
     a.inv_vol = 1.0 / (p->d.box * p->d.box * p->d.box);

@@ -126,15 +126,24 @@ struct YZExpArgs {
                            //      (only those are read); every real output is formed
 };
 
+// Tables and scratch of the initial field, in the plan's device block
+constexpr int kIcAngles = 512;          // (cos, sin)(2 pi j / 512) as FP32 values and their errors
+constexpr int kIcLogs = 129;            // -ln(r / 512) likewise, r = 131072 / i rounded, i = 128 .. 256
+constexpr float kIcAngleUnitHi = 7.31459059988282e-10f, kIcAngleUnitLo = -2.035470133961082e-17f;   // 2 pi 2^-33
+constexpr int kIcParts = 256;           // partial sums of the sigma_8 integral
 struct IcArgs {
     float2* out;           // one realisation
     uint64_t seed;
-    double amp;            // A of P(k) = A k^ns T^2
+    double sigma8;         // P(k) = A k^ns T^2, A = sigma8^2 over the unit spectrum's sigma_8^2
+    const float4* angles;
+    const float2* logs;
+    double* parts;         // [kIcParts], written and read by launch_ic_table
     double n_s;
     double gamma;
     double inv_vol;        // 1 / L^3
     long long s2_cut;      // keep 0 < |s|^2 <= s2_cut
-    double* table;         // [s2_cut + 1]: sqrt(P(k_F sqrt(s2)) / L^3) / sqrt(2), made by launch_ic_table
+    float2* table;         // [s2_cut + 1]: sqrt(P(k_F sqrt(s2)) / L^3) / sqrt(2) as FP32 value and error,
+                           // made by launch_ic_table
     double kF;
 };
 
