@@ -618,4 +618,259 @@ __device__ __forceinline__ void fft_col_pair(float2 (&x)[2][fft_elems(L)], int p
     if constexpr (NB == 2 && (fft_nstages(L) - 1) % 2 == 1) __syncthreads();
 }
 
+
+// --------------------------------------------- one-exchange column transform (col2)
+// The column transform of the power-of-two lengths L = 128 .. 1024 with its stages
+// grouped so that an element crosses shared memory once:
+//   L = 128, 256: radix 8, exchange, then 8 x 2 or 8 x 4 inside a thread (P = 8
+//     threads a column, E = 16 or 32 elements each);
+//   L = 512, 1024: 8 x 8 inside a pair of threads of a warp, exchange, then radix 8
+//     or 8 x 2 inside a thread (P = 16 or 32, E = 32). Half of a pair's values
+//     change threads by shuffles between its two stages.
+// Stages, butterflies and twiddle values are those of fft_column: the results are
+// bitwise equal (signs that the pair form moves around are exact).
+// The column passes are bound by shared-memory wavefronts, barriers and the warps
+// that 64 registers leave (512^3, one exchange per stage: 0.5 wavefronts and 50
+// instructions a point); here a thread carries 16 or 32 elements as independent
+// chains, most twiddles serve several butterflies, and a transform has two
+// barriers. 64 elements a thread (8, exchange, 8 x 8) spills and is slower.
+template <int L>
+struct Col2 {
+    static constexpr bool ok = L >= 128 && L <= 1024 && (L & (L - 1)) == 0;
+    static constexpr bool pair = L >= 512;
+    static constexpr int P = pair ? L / 32 : 8, E = L / P;
+    static constexpr int G = P / 2;                         // pairs of a column
+    static constexpr int R2 = pair ? (L == 512 ? 1 : 2) : L / 64;   // radix of the last stage (1: none)
+    // shared twiddles. P = 8: per thread p [8] stage 1, [8][R2] stage 2. Pair form: [2][4][8]
+    // of the second stage common to all pairs, then per thread 512: [4][8] stage 2;
+    // 1024: [2][8] stage 2, [2][8] stage 3. The pitch (two entries more) puts the
+    // threads of a warp on other banks.
+    static constexpr int PER = pair ? 32 : 8 + 8 * R2, PITCH = PER + 2;
+    static constexpr int TW = P * PITCH + (pair ? 64 : 0);        // float2, even
+    static constexpr int ROWS = L + L / 64;                       // exchange rows (row of n: n + n / 64)
+    static constexpr size_t bytes(int tz) { return sizeof(float2) * (TW + (size_t)ROWS * tz); }
+    // element held by thread p in x[i]: in_base(p) + in_step(i) before the transform, p + P i after
+    __host__ __device__ static constexpr int in_base(int p) { return pair ? (p >> 1) + 4 * G * (p & 1) : p; }
+    __host__ __device__ static constexpr int in_step(int i) { return pair ? G * ((i & 3) + 8 * (i >> 2)) : P * i; }
+};
+__device__ __forceinline__ int col2_row(int n) { return n + (n >> 6); }
+// sign that the pair form leaves on element m of the exchange: -1 where the index
+// inside the group of 64, r + 8 t, has r >= 4 and t odd
+__device__ __forceinline__ float col2_sign(int m) { return (m & 4) && (m & 8) ? -1.f : 1.f; }
+
+// Fill the table (whole block) from the L-th roots of unity in global memory; the
+// pair form ends with a block barrier (the others read it after an exchange's).
+template <int L>
+__device__ __forceinline__ void col2_table(float2* twl, const float2* __restrict__ twg) {
+    using C = Col2<L>;
+    if constexpr (!C::pair) {
+        for (int j = threadIdx.x; j < C::P * C::PER; j += blockDim.x) {
+            const int p = j / C::PER, r = j - p * C::PER, m = r - 8;
+            twl[p * C::PITCH + r] = r < 8 ? twg[r * p * (L / 64)] : twg[(m % C::R2) * (p + 8 * (m / C::R2))];
+        }
+    } else {
+        for (int j = threadIdx.x; j < 64; j += blockDim.x) {      // [h][s][own 4, received 4]: w64^(q r)
+            const int h = j / 32, r = (j / 8) % 4 + 4 * h, q = (j % 8) ^ (4 * h);
+            twl[j] = twg[q * r * (L / 64)];
+        }
+        for (int j = threadIdx.x; j < C::P * 32; j += blockDim.x) {
+            const int p = j / 32, r = j % 32, t = r % 8;
+            float2 w;
+            float g = 1.f;
+            if (L == 512) {                                       // butterfly p + 16 (r / 8)
+                const int k = p + 16 * (r / 8);
+                w = twg[t * k];
+                g = col2_sign(k);
+            } else if (r < 16) {                                  // k = p + 32 (r / 8), w512^(t k)
+                const int k = p + 32 * (r / 8);
+                w = twg[t * k * 2];
+                g = col2_sign(k);
+            } else {
+                w = twg[p + 32 * (r / 8 - 2) + 64 * t];           // w1024^(k + 64 t)
+            }
+            twl[64 + p * C::PITCH + r] = make_float2(g * w.x, g * w.y);
+        }
+        __syncthreads();                       // read before the first exchange's barrier
+    }
+}
+
+template <int DIR>
+__device__ __forceinline__ float2 col2_tw(float2 a, float wx, float wy) {   // a w (DIR > 0) or a conj w
+    const float y = DIR < 0 ? -wy : wy;
+    return make_float2(fmaf(a.x, wx, -a.y * y), fmaf(a.x, y, a.y * wx));
+}
+// v[t] *= w[t], T0 <= t < R, from consecutive table entries, two per 16-byte load;
+// with sign, v[0] is scaled by the real w[0] = +-1
+template <int R, int DIR, int T0 = 1, bool SIGN = false>
+__device__ __forceinline__ void col2_twiddle(float2* v, const float2* __restrict__ w) {
+#pragma unroll
+    for (int t = 0; t < R; t += 2) {
+        const float4 u = *reinterpret_cast<const float4*>(w + t);
+        if (t >= T0) v[t] = col2_tw<DIR>(v[t], u.x, u.y);
+        else if (SIGN) v[t] = cscale(v[t], u.x);
+        v[t + 1] = col2_tw<DIR>(v[t + 1], u.z, u.w);
+    }
+}
+// dft_small<8> with outputs s and s + 4 exchanged for g = -1. The products with
+// 1 / sqrt(2) and the sums after them are single roundings, as the compiler makes
+// them in dft_small.
+template <int DIR>
+__device__ __forceinline__ void dft8_half(float2* v, float g) {
+    const float r2 = g * 0.70710678118654752440f;
+    float2 e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
+    dft_small<4, DIR>(e);
+    dft_small<4, DIR>(o);
+    o[1] = cadd(o[1], cmul_i<DIR>(o[1]));
+    o[2] = cmul_i<DIR>(o[2]);
+    o[3] = csub(cmul_i<DIR>(o[3]), o[3]);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        const float w = t & 1 ? r2 : g;
+        v[t] = lfma(w, o[t], e[t]);
+        v[t + 4] = lfma(-w, o[t], e[t]);
+    }
+}
+
+// Thread p of a column holds elements in_base(p) + in_step(i) in x[i] before and
+// p + P i after. Every thread of the block calls it the same number of times; the
+// TZ columns of a thread index p are consecutive lanes (TZ = 8, 16 or 32). col: exchange
+// buffer of the column (element n at col[col2_row(n) * TZ]); the barrier before the
+// writes lets the readers of the previous transform finish.
+template <int L, int DIR, int TZ>
+__device__ __forceinline__ void fft_col2(float2 (&x)[Col2<L>::E], int p, float2* col,
+                                         const float2* __restrict__ twl) {
+    using C = Col2<L>;
+    constexpr int E = C::E, R2 = C::R2;
+    if constexpr (!C::pair) {
+        // stage 0: butterflies b = p + 8 q, outputs 8 b + t
+#pragma unroll
+        for (int q = 0; q < E / 8; ++q) {
+            float2 v[8];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) v[t] = x[q + t * (E / 8)];
+            dft_small<8, DIR>(v);
+#pragma unroll
+            for (int t = 0; t < 8; ++t) x[q + t * (E / 8)] = v[t];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < E / 8; ++q)
+#pragma unroll
+            for (int t = 0; t < 8; ++t) col[col2_row(8 * (p + 8 * q) + t) * TZ] = x[q + t * (E / 8)];
+        __syncthreads();
+        // stage 1: butterflies b = p + 8 s (k = p), inputs b + u L / 8; outputs of index
+        // u feed input s of the last stage's butterfly p + 8 u
+        const float2* tw = twl + p * C::PITCH;
+        float2 w1[8];
+#pragma unroll
+        for (int u = 0; u < 8; u += 2) {
+            const float4 w = *reinterpret_cast<const float4*>(tw + u);
+            w1[u] = make_float2(w.x, w.y);
+            w1[u + 1] = make_float2(w.z, w.w);
+        }
+#pragma unroll
+        for (int s = 0; s < R2; ++s) {
+            float2 v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = col[col2_row(p + 8 * s + u * (L / 8)) * TZ];
+#pragma unroll
+            for (int u = 1; u < 8; ++u) v[u] = col2_tw<DIR>(v[u], w1[u].x, w1[u].y);
+            dft_small<8, DIR>(v);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x[u + 8 * s] = v[u];
+        }
+        // last stage: butterflies p + 8 u, outputs p + 8 (u + 8 t)
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            float2 v[R2];
+#pragma unroll
+            for (int s = 0; s < R2; ++s) v[s] = x[u + 8 * s];
+            col2_twiddle<R2, DIR>(v, tw + 8 + u * R2);
+            dft_small<R2, DIR>(v);
+#pragma unroll
+            for (int t = 0; t < R2; ++t) x[u + 8 * t] = v[t];
+        }
+    } else {
+        // stage 0: butterflies g + G q of the pair, this thread q = 4 h + j; output r
+        // goes to slot r ^ 4 h, so slots 0 .. 3 are the ones this thread keeps
+        const int h = p & 1, g = p >> 1;
+        const float sg = h ? -1.f : 1.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float2 v[8];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) v[t] = x[j + 4 * t];
+            dft8_half<DIR>(v, sg);
+#pragma unroll
+            for (int t = 0; t < 8; ++t) x[j + 4 * t] = v[t];
+        }
+#pragma unroll
+        for (int i = 16; i < 32; ++i) {                           // slots 4 .. 7 change threads
+            x[i].x = __shfl_xor_sync(0xffffffffu, x[i].x, TZ);
+            x[i].y = __shfl_xor_sync(0xffffffffu, x[i].y, TZ);
+        }
+        // stage 1: for r = s + 4 h, inputs q: own 4 h + j, received 4 (1 - h) + j. For h = 1
+        // the two halves are exchanged, which leaves (-1)^t on output t (col2_sign)
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            float2 v[8];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                v[j] = x[j + 4 * s];
+                v[j + 4] = x[j + 4 * (s + 4)];
+            }
+            col2_twiddle<8, DIR, 0>(v, twl + 32 * h + 8 * s);
+            dft_small<8, DIR>(v);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                x[j + 4 * s] = v[j];
+                x[j + 4 * (s + 4)] = v[j + 4];
+            }
+        }
+        __syncthreads();
+        float2* wr = col + col2_row(64 * g + 4 * h) * TZ;         // (all rows of a group share the padding)
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+#pragma unroll
+            for (int t = 0; t < 8; ++t) wr[(s + 8 * t) * TZ] = t < 4 ? x[t + 4 * s] : x[t - 4 + 4 * (s + 4)];
+        __syncthreads();
+        const float2* tw = twl + 64 + p * C::PITCH;
+        if constexpr (L == 512) {
+            // stage 2: butterflies k = p + 16 m, outputs k + 64 t
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                float2 v[8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t) v[t] = col[(col2_row(64 * t) + p + 16 * m) * TZ];
+                col2_twiddle<8, DIR, 1, true>(v, tw + 8 * m);
+                dft_small<8, DIR>(v);
+#pragma unroll
+                for (int t = 0; t < 8; ++t) x[m + 4 * t] = v[t];
+            }
+        } else {
+            // stages 2 and 3 for k = p + 32 j: butterflies k and k + 64, then the pairs
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                float2 v[2][8];
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh) {
+#pragma unroll
+                    for (int t = 0; t < 8; ++t) v[hh][t] = col[(col2_row(64 * hh + 128 * t) + p + 32 * j) * TZ];
+                    col2_twiddle<8, DIR, 1, true>(v[hh], tw + 8 * j);
+                    dft_small<8, DIR>(v[hh]);
+                }
+#pragma unroll
+                for (int t = 0; t < 8; t += 2) {
+                    const float4 w = *reinterpret_cast<const float4*>(tw + 16 + 8 * j + t);
+                    const float2 a = col2_tw<DIR>(v[1][t], w.x, w.y), b = col2_tw<DIR>(v[1][t + 1], w.z, w.w);
+                    x[j + 2 * t] = cadd(v[0][t], a);
+                    x[j + 2 * t + 16] = csub(v[0][t], a);
+                    x[j + 2 * t + 2] = cadd(v[0][t + 1], b);
+                    x[j + 2 * t + 18] = csub(v[0][t + 1], b);
+                }
+            }
+        }
+    }
+}
+
 }  // namespace gridspt

@@ -59,11 +59,15 @@ struct QRow {
 
 // tile width of the column passes with 256 threads
 template <int N>
-__host__ __device__ constexpr int qtz() { return kQueueThreads / (N / fft_elems(N)); }
+__host__ __device__ constexpr int qtz() {
+    if constexpr (Col2<N>::ok) return kQueueThreads / Col2<N>::P;
+    else return kQueueThreads / (N / fft_elems(N));
+}
 
 template <int N>
 __host__ __device__ constexpr size_t col_smem() {
-    return ColSm<N, qtz<N>()>::bytes > colpass_smem<N, qtz<N>()>() ? ColSm<N, qtz<N>()>::bytes
+    if constexpr (Col2<N>::ok) return Col2<N>::bytes(qtz<N>());
+    else return ColSm<N, qtz<N>()>::bytes > colpass_smem<N, qtz<N>()>() ? ColSm<N, qtz<N>()>::bytes
                                                                     : colpass_smem<N, qtz<N>()>();
 }
 
@@ -257,12 +261,28 @@ __device__ void q_tile(const QStage& st, long long tile, float2* sm, bool tr) {
     const int by = (int)(rest % st.gy);
     const int bz = (int)(rest / st.gy);
     switch (st.kind) {
-        case Q_XEXP0: xexp_body<N, TZ, 0>(st.x, st.tw, st.kF, st.inv_kF2, bx, by, sm, tr); break;
-        case Q_XEXP1: xexp_body<N, TZ, 1>(st.x, st.tw, st.kF, st.inv_kF2, bx, by, sm, tr); break;
-        case Q_YEXP: yexp_body<N, TZ, false>(st.y, st.tw, st.kF, bx, by, sm, tr); break;
-        case Q_COLY: colpass_body<N, TZ, 1, false>(st.data, st.fstride, st.tw, -1, 0, 0, bx, by, bz, sm, tr); break;
+        case Q_XEXP0:
+            if constexpr (Col2<N>::ok) col2_xexp_body<N, TZ, 0>(st.x, st.tw, st.kF, bx, by, sm, tr);
+            else xexp_body<N, TZ, 0>(st.x, st.tw, st.kF, st.inv_kF2, bx, by, sm, tr);
+            break;
+        case Q_XEXP1:
+            if constexpr (Col2<N>::ok) col2_xexp_body<N, TZ, 1>(st.x, st.tw, st.kF, bx, by, sm, tr);
+            else xexp_body<N, TZ, 1>(st.x, st.tw, st.kF, st.inv_kF2, bx, by, sm, tr);
+            break;
+        case Q_YEXP:
+            if constexpr (Col2<N>::ok) col2_yexp_body<N, TZ>(st.y, st.tw, st.kF, bx, by, sm, tr);
+            else yexp_body<N, TZ, false>(st.y, st.tw, st.kF, bx, by, sm, tr);
+            break;
+        case Q_COLY:
+            if constexpr (Col2<N>::ok)
+                col2_pass_body<N, TZ, 1, false>(st.data, st.fstride, st.tw, -1, 0, 0, bx, by, bz, sm, tr);
+            else colpass_body<N, TZ, 1, false>(st.data, st.fstride, st.tw, -1, 0, 0, bx, by, bz, sm, tr);
+            break;
         case Q_COLX:
-            colpass_body<N, TZ, 0, true>(st.data, st.fstride, st.tw, st.s2, st.zero_k0, 0, bx, by, bz, sm, tr);
+            if constexpr (Col2<N>::ok)
+                col2_pass_body<N, TZ, 0, true>(st.data, st.fstride, st.tw, st.s2, st.zero_k0, 0, bx, by, bz, sm, tr);
+            else
+                colpass_body<N, TZ, 0, true>(st.data, st.fstride, st.tw, st.s2, st.zero_k0, 0, bx, by, bz, sm, tr);
             break;
         case Q_ZR2C: q_zr2c<N>(st, tile, sm, tr); break;
         case Q_Z: {

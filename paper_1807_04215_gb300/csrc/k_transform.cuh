@@ -692,6 +692,237 @@ k_yexp2(YZExpArgs args, const float2* __restrict__ twg, float kF) {
     }
 }
 
+// ------------------------------------ column passes on the one-exchange transform
+// The x, y and forward column passes of the power-of-two N >= 128 (fft_col2): TZ
+// adjacent kz columns (16: 128-byte rows) by P threads of E elements. Only one
+// column of registers is live: an output that shares its input with the previous
+// one reads it again (the block's own tile: L1 or L2), instead of keeping it beside
+// the working copy, which would halve the warps. Index arithmetic folds: the
+// element index is a thread's base plus a constant, and lies below N / 2 exactly
+// when i < E / 2. Kernel times against the one-exchange-per-stage tiles: 512^3 x
+// forward + expansion 1.69 -> 1.41 ms, y expansion 2.13 -> 1.90 (7 -> 12 fields), y
+// forward 0.385 -> 0.362, x forward 0.573 -> 0.393 (2 fields); 256^3 0.213 -> 0.158,
+// 0.273 -> 0.204; 1024^3 (one field) x 2.94 -> 2.80, y 2.69 -> 1.97.
+template <int N>
+struct Col2Tile {
+    static constexpr int TZ = N == 1024 ? 8 : 16;
+};
+
+template <int N, int TZ>
+struct Col2Cfg {
+    using C = Col2<N>;
+    static constexpr int THREADS = TZ * C::P;
+    // threads per SM by registers: 128 a thread for 32 elements, 80 for 16
+    static constexpr int MINB = cmax(1, (C::E == 32 ? 512 : 768) / THREADS);
+    static constexpr size_t smem = C::bytes(TZ);
+};
+
+// Keep a pointer opaque, so that a loop does not hold the addresses of all its
+// elements (which differ by more than an instruction's offset) in registers.
+template <typename T>
+__device__ __forceinline__ T* opaque(T* p) {
+    asm volatile("" : "+l"(p));
+    return p;
+}
+
+template <int N, int TZ, int AXIS, bool FIN>
+__device__ __forceinline__ void col2_pass_body(float2* __restrict__ data, long long fstride,
+                                               const float2* __restrict__ twg, long long s2_nl, int zero_k0,
+                                               int band, int bx, int by, int bz, float2* sm,
+                                               bool table_ready = false) {
+    using C = Col2<N>;
+    constexpr int M = N / 2, E = C::E, P = C::P;
+    const int tid = threadIdx.x, c = tid % TZ, p = tid / TZ;
+    if (!table_ready) col2_table<N>(sm, twg);
+    const int kz = bx * TZ + c;
+    const bool act = kz < M && (band <= 0 || kz < band);
+    constexpr long long estride = AXIS == 0 ? (long long)N * M : (long long)M;
+    constexpr long long astride = AXIS == 0 ? (long long)M : (long long)N * M;
+    float2* col = data + bz * fstride + by * astride + kz;
+    float2 x[E];
+    const float2* in = opaque(col + C::in_base(p) * estride);
+#pragma unroll
+    for (int i = 0; i < E; ++i) x[i] = act ? in[C::in_step(i) * estride] : make_float2(0.f, 0.f);
+    fft_col2<N, -1, TZ>(x, p, sm + C::TW + c, sm);
+    if (!act) return;                          // no block barrier follows
+    const int sy = signed_idx(by, N);
+    const float syz = (float)(sy * sy + kz * kz), fp = (float)p, cut = s2_nl >= 0 ? (float)s2_nl : 3.e38f;
+    float2* out = opaque(col + p * estride);
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+        const int sx = p + (i < E / 2 ? P * i : P * i - N);
+        if constexpr (FIN) {
+            const float fx = fp + (float)(i < E / 2 ? P * i : P * i - N), s2 = fmaf(fx, fx, syz);   // exact
+            if ((i == E / 2 && p == 0) || by == N / 2 || s2 > cut || (zero_k0 && s2 == 0.f)) x[i] = make_float2(0.f, 0.f);
+        }
+        if (band <= 0 || (sx < band && -sx < band)) out[P * i * estride] = x[i];
+    }
+}
+
+// The x expansion (see xexp_body): MODE 0 backward only, MODE 1 forward first,
+// MODE 2 backward of shell masks (bispectrum).
+template <int N, int TZ, int MODE>
+__device__ __forceinline__ void col2_xexp_body(const XExpArgs& args, const float2* __restrict__ twg, float kF,
+                                               int bx, int by, float2* sm, bool table_ready = false) {
+    using C = Col2<N>;
+    constexpr int M = N / 2, E = C::E, P = C::P;
+    const int tid = threadIdx.x, c = tid % TZ, p = tid / TZ;
+    if (!table_ready) col2_table<N>(sm, twg);
+    float2* buf = sm + C::TW + c;
+    const int kz = bx * TZ + c;
+    const int B = args.band;
+    const int ky = (B > 0 && by >= B) ? N - (2 * B - 1 - by) : by;   // band rows: [0, B) and (N - B, N)
+    const bool act = kz < M && (B <= 0 || kz < B);
+    constexpr long long plane = (long long)N * M;
+    const long long ofs = (long long)ky * M + kz;
+    const bool two = args.src1 != args.src0;
+    const int sy = signed_idx(ky, N);
+    const float syz = (float)(sy * sy + kz * kz), fin = (float)C::in_base(p), fout = (float)p;
+    // signed kx of input and output element i; |s|^2 = kx^2 + syz is exact in FP32
+    auto sx_in = [&](int i) { return fin + (float)(i < E / 2 ? C::in_step(i) : C::in_step(i) - N); };
+    float2 x[E];
+    auto load = [&](const float2* base, bool rd) {
+        const float2* q = opaque(base + ofs + C::in_base(p) * plane);
+#pragma unroll
+        for (int i = 0; i < E; ++i) x[i] = rd ? q[C::in_step(i) * plane] : make_float2(0.f, 0.f);
+    };
+    auto store = [&](float2* base) {
+        float2* q = opaque(base + ofs + p * plane);
+        if (act) {
+#pragma unroll
+            for (int i = 0; i < E; ++i) q[P * i * plane] = x[i];
+        }
+    };
+    if constexpr (MODE == 1) {
+        const float cut = args.s2_nl >= 0 ? (float)args.s2_nl : 3.e38f;
+        const float k0 = args.zero_k0 ? 0.f : -1.f;
+#pragma unroll 1
+        for (int w = 0; w < (two ? 2 : 1); ++w) {
+            float2* col = w ? args.src1 : args.src0;
+            load(col, act);
+            fft_col2<N, -1, TZ>(x, p, buf, sm);
+#pragma unroll
+            for (int i = 0; i < E; ++i) {
+                const float sx = fout + (float)(i < E / 2 ? P * i : P * i - N), s2 = fmaf(sx, sx, syz);
+                if ((i == E / 2 && p == 0) || ky == N / 2 || s2 > cut || s2 == k0) x[i] = make_float2(0.f, 0.f);
+            }
+            store(col);
+        }
+        __syncthreads();                       // the block's spectra are read back below, by other threads
+    }
+    const float cut_in = MODE == 0 && args.s2_in >= 0 ? (float)args.s2_in : 3.e38f;
+    // Outputs: the source column is read again for each (MODE 1: this block's
+    // stores above), scaled by its multiplier or shell mask, transformed, stored.
+#pragma unroll 1
+    for (int f = 0; f < args.nout; ++f) {
+        const int code = args.codes[f];
+        const int pa = (code >> 4) & 3, src = (code >> 8) & 3;
+        load(src != XS_DELTA && two ? args.src1 : args.src0, act && src != XS_ONE);
+        if constexpr (MODE == 2) {
+            const float lo = args.shell_lo > 1 ? (float)args.shell_lo : 1.f, hi = (float)args.shell_hi;
+#pragma unroll
+            for (int i = 0; i < E; ++i) {
+                const float sx = sx_in(i), s2 = fmaf(sx, sx, syz);
+                if (src == XS_ONE) x[i].x = 1.f;
+                if (!(s2 >= lo && s2 < hi)) x[i] = make_float2(0.f, 0.f);
+            }
+        } else {
+            if constexpr (MODE == 0) {
+#pragma unroll
+                for (int i = 0; i < E; ++i) {
+                    const float sx = sx_in(i);
+                    if (fmaf(sx, sx, syz) > cut_in) x[i] = make_float2(0.f, 0.f);
+                }
+            }
+            if (src == XS_PHI) {
+#pragma unroll
+                for (int i = 0; i < E; ++i) {
+                    const float sx = sx_in(i), s2 = fmaf(sx, sx, syz);
+                    x[i] = cscale(x[i], s2 > 0.f ? __frcp_rn(s2) : 0.f);   // 1 / k^2 (k_F = 1), 0 at k = 0
+                }
+            }
+            if (pa) {
+#pragma unroll
+                for (int i = 0; i < E; ++i) {
+                    const float kx = kF * sx_in(i);
+                    x[i] = cscale(x[i], pa == 1 ? kx : kx * kx);
+                }
+            }
+        }
+        fft_col2<N, +1, TZ>(x, p, buf, sm);
+        store(args.out + f * args.out_stride);
+    }
+}
+static_assert(kDerivUnit == 1.0f, "the column passes take 1 / k^2 as 1 / |s|^2");
+
+// The y expansion (see yexp_body).
+template <int N, int TZ>
+__device__ __forceinline__ void col2_yexp_body(const YZExpArgs& args, const float2* __restrict__ twg, float kF,
+                                               int bx, int by, float2* sm, bool table_ready = false) {
+    using C = Col2<N>;
+    constexpr int M = N / 2, E = C::E, P = C::P;
+    const int tid = threadIdx.x, c = tid % TZ, p = tid / TZ;
+    if (!table_ready) col2_table<N>(sm, twg);
+    float2* buf = sm + C::TW + c;
+    const int kz = bx * TZ + c;
+    const int B = args.band;
+    const bool act = kz < M && (B <= 0 || kz < B);
+    const long long ofs = (long long)by * N * M + kz;
+    const int ib = C::in_base(p);
+    auto live = [&](int i) {
+        const int sy = ib + (i < E / 2 ? C::in_step(i) : C::in_step(i) - N);
+        return act && (B <= 0 || (sy < B && -sy < B));
+    };
+#pragma unroll 1
+    for (int f = 0; f < args.nout; ++f) {
+        const int code = args.codes[f];
+        const int in = code & 255, pb = (code >> 8) & 3, slot = code >> 16;
+        const float2* col = args.in + in * args.in_stride + ofs + ib * M;
+        float2 x[E];
+#pragma unroll
+        for (int i = 0; i < E; ++i) x[i] = live(i) ? col[C::in_step(i) * M] : make_float2(0.f, 0.f);
+        if (f + 1 < args.nout && (args.codes[f + 1] & 255) != in) {   // the next input: into L2 meanwhile
+            const float2* nx = args.in + (args.codes[f + 1] & 255) * args.in_stride + ofs + ib * M;
+#pragma unroll
+            for (int i = 0; i < E; ++i)
+                if ((c & 15) == 0 && live(i)) prefetch_l2(nx + C::in_step(i) * M);
+        }
+        if (pb) {
+#pragma unroll
+            for (int i = 0; i < E; ++i) {
+                const float ky = kF * ((float)ib + (float)(i < E / 2 ? C::in_step(i) : C::in_step(i) - N));
+                x[i] = cscale(x[i], pb == 1 ? ky : ky * ky);
+            }
+        }
+        fft_col2<N, +1, TZ>(x, p, buf, sm);
+        if (act) {
+            float2* o = args.out + slot * args.out_stride + ofs + p * M;
+#pragma unroll
+            for (int i = 0; i < E; ++i) o[P * i * M] = x[i];
+        }
+    }
+}
+
+template <int N, int TZ, int AXIS, bool FIN>
+__global__ void __launch_bounds__(Col2Cfg<N, TZ>::THREADS, Col2Cfg<N, TZ>::MINB)
+k_fcol(float2* __restrict__ data, long long fstride, const float2* __restrict__ twg, long long s2_nl, int zero_k0,
+       int band) {
+    extern __shared__ __align__(16) float2 sm[];
+    col2_pass_body<N, TZ, AXIS, FIN>(data, fstride, twg, s2_nl, zero_k0, band, blockIdx.x, blockIdx.y, blockIdx.z, sm);
+}
+template <int N, int TZ, int MODE>
+__global__ void __launch_bounds__(Col2Cfg<N, TZ>::THREADS, Col2Cfg<N, TZ>::MINB)
+k_xcol(const __grid_constant__ XExpArgs args, const float2* __restrict__ twg, float kF) {
+    extern __shared__ __align__(16) float2 sm[];
+    col2_xexp_body<N, TZ, MODE>(args, twg, kF, blockIdx.x, blockIdx.y, sm);
+}
+template <int N, int TZ>
+__global__ void __launch_bounds__(Col2Cfg<N, TZ>::THREADS, Col2Cfg<N, TZ>::MINB)
+k_ycol(const __grid_constant__ YZExpArgs args, const float2* __restrict__ twg, float kF) {
+    extern __shared__ __align__(16) float2 sm[];
+    col2_yexp_body<N, TZ>(args, twg, kF, blockIdx.x, blockIdx.y, sm);
+}
+
 // ------------------------------------------------------------ z expansion
 // Output f = IFFT_z(c kz^g xy-field[in]) as a real row of N values, via the
 // half-length complex transform of the packed row (Nyquist term zero). The
@@ -1825,12 +2056,57 @@ struct Launch {
     }
 };
 
+// Launchers of the one-exchange column passes (power-of-two N >= 128).
+template <int N, int TZ>
+struct LaunchCol2 {
+    using F = Col2Cfg<N, TZ>;
+    static constexpr int M = N / 2;
+    static unsigned tiles(int B) { return (unsigned)(((B ? B : M) + TZ - 1) / TZ); }
+    static cudaError_t colpass(const Geo& g, float2* d, long long fs, int count, int axis, int fin, long long s2_nl,
+                               int band, cudaStream_t s) {
+        const int B = axis == 1 && band > 0 && band < M ? band : 0;
+        const dim3 grid(tiles(B), N, count);
+        cudaError_t e;
+#define GRIDSPT_FCOL(AX_, FIN_)                                                                      \
+    if ((e = set_smem(k_fcol<N, TZ, AX_, FIN_>, F::smem)) != cudaSuccess) return e;                  \
+    k_fcol<N, TZ, AX_, FIN_><<<grid, F::THREADS, F::smem, s>>>(d, fs, g.tw, s2_nl, fin == 2, B);     \
+    return cudaGetLastError();
+        if (axis == 0) {
+            if (fin) { GRIDSPT_FCOL(0, true) }
+            GRIDSPT_FCOL(0, false)
+        }
+        GRIDSPT_FCOL(1, false)
+#undef GRIDSPT_FCOL
+    }
+    template <int MODE>
+    static cudaError_t xexp_m(const Geo& g, const XExpArgs& a, cudaStream_t s) {
+        const int B = a.band > 0 && a.band < M ? a.band : 0;
+        cudaError_t e = set_smem(k_xcol<N, TZ, MODE>, F::smem);
+        if (e != cudaSuccess) return e;
+        k_xcol<N, TZ, MODE><<<dim3(tiles(B), B ? 2 * B - 1 : N), F::THREADS, F::smem, s>>>(a, g.tw, kDerivUnit);
+        return cudaGetLastError();
+    }
+    static cudaError_t xexp(const Geo& g, const XExpArgs& a, cudaStream_t s) {
+        const bool shell = a.nout > 0 && (a.codes[0] & 15) == XK_SHELL;   // (a call's outputs are all of one kind)
+        return a.fwd_first ? xexp_m<1>(g, a, s) : shell ? xexp_m<2>(g, a, s) : xexp_m<0>(g, a, s);
+    }
+    static cudaError_t yexp(const Geo& g, const YZExpArgs& a, cudaStream_t s) {
+        const int B = a.band > 0 && a.band < M ? a.band : 0;
+        cudaError_t e = set_smem(k_ycol<N, TZ>, F::smem);
+        if (e != cudaSuccess) return e;
+        k_ycol<N, TZ><<<dim3(tiles(B), N), F::THREADS, F::smem, s>>>(a, g.tw, kDerivUnit);
+        return cudaGetLastError();
+    }
+};
+
 // Per-size entry points (defined in the k_transform_*.cu units). The pass
 // variant v selects tile widths: v = 0 default, v = 1 alternative.
 #define GRIDSPT_TRANSFORM_SIZE(N)                                                                          \
     cudaError_t transform_colpass_##N(const Geo& g, float2* d, long long fs, int count, int axis, int fin, \
                                       long long s2, int band, int v, cudaStream_t s) {                     \
-        return v ? Launch<N, Cfg<N>::TZC1, Cfg<N>::TZZ0>::colpass(g, d, fs, count, axis, fin, s2, band, s) \
+        if constexpr (Col2<N>::ok)                                                                         \
+            return LaunchCol2<N, Col2Tile<N>::TZ>::colpass(g, d, fs, count, axis, fin, s2, band, s);       \
+        else return v ? Launch<N, Cfg<N>::TZC1, Cfg<N>::TZZ0>::colpass(g, d, fs, count, axis, fin, s2, band, s) \
                  : Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::colpass(g, d, fs, count, axis, fin, s2, band, s); \
     }                                                                                                      \
     cudaError_t transform_zr2c_##N(const Geo& g, const float2* in, float2* out, long long fs, int count,   \
@@ -1843,13 +2119,15 @@ struct Launch {
     cudaError_t transform_xexp_##N(const Geo& g, const XExpArgs& a, int v, cudaStream_t s) {               \
         if (a.fwd_first && a.div_in) /* four input columns in registers: the narrower tile */              \
             return Launch<N, Cfg<N>::TZC1, Cfg<N>::TZZ0>::template xexp<false>(g, a, s);                   \
-        if (v == 2) return Launch<N, Cfg<N>::TZC1, Cfg<N>::TZZ0>::template xexp<true>(g, a, s);            \
+        if constexpr (Col2<N>::ok) return LaunchCol2<N, Col2Tile<N>::TZ>::xexp(g, a, s);                   \
+        else if (v == 2) return Launch<N, Cfg<N>::TZC1, Cfg<N>::TZZ0>::template xexp<true>(g, a, s);            \
         if (v == 3) return Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::template xexp<true>(g, a, s);            \
         return v ? Launch<N, Cfg<N>::TZC1, Cfg<N>::TZZ0>::template xexp<false>(g, a, s)                    \
                  : Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::template xexp<false>(g, a, s);                   \
     }                                                                                                      \
     cudaError_t transform_yexp_##N(const Geo& g, const YZExpArgs& a, int v, cudaStream_t s) {              \
-        if (v == 2 && N >= 128 && a.band <= 0) return Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::yexp_tma(g, a, s); \
+        if constexpr (Col2<N>::ok) return LaunchCol2<N, Col2Tile<N>::TZ>::yexp(g, a, s);                   \
+        else if (v == 2 && N >= 128 && a.band <= 0) return Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::yexp_tma(g, a, s); \
         if (v == 3) return Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::yexp2(g, a, s);                          \
         if (v == 4) return Launch<N, Cfg<N>::TZC1, Cfg<N>::TZZ0>::template yexp<true, false>(g, a, s);      \
         if (v == 5) return Launch<N, Cfg<N>::TZC1, Cfg<N>::TZZ0>::template yexp<false, true>(g, a, s);      \
