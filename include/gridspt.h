@@ -350,15 +350,10 @@ gridspt_status gridspt_multi_destroy(gridspt_multi multi);
 /* Autotuner for the transform passes (not part of the paper's method). Each
  * pass (0 forward column pass, 1 x expansion, 2 y expansion, 3 z expansion,
  * 4 contiguous-axis forward pass) has two variants for N >= 128 (identical for
- * smaller N). The x expansion has two more (2, 3) that transform two outputs
- * (and the two forward inputs) at a time in a shared exchange. The y
- * expansion has a third, TMA-staged one (N >= 128), a fourth with two
- * adjacent columns per thread (16-byte accesses), a fifth that copies the
- * next input's columns by cp.async during the current input's transforms, and
- * a sixth and seventh (5, 6) that transform two outputs of one input at a
- * time. The z
- * expansion and the contiguous-axis forward pass have a third that runs one z
- * row per group of warp lanes without block-wide barriers (every N but 12,
+ * smaller N), except that the passes 0, 1 and 2 of the power-of-two N >= 128 have
+ * one form. The x expansion also accepts 2 and 3 (they run as 1 and 0), the y
+ * expansion 2 .. 6 (they run as 0, 0, 1, 1, 0). The z expansion and the
+ * contiguous-axis forward pass have a third that runs one z row per group of warp lanes without block-wide barriers (every N but 12,
  * which runs variant 0 when it is chosen); the z expansion's
  * choice also applies to the pair products fused into it and to the z pass of
  * the bispectrum shells. gridspt_autotune times the
@@ -435,9 +430,8 @@ gridspt_status gridspt_profile_end(gridspt_kernel_stat* stats, int32_t capacity,
 
 /* Device-side status: synchronises `stream` and reads the plan's status word,
  * which the plan's kernels set since the last check:
- * - GRIDSPT_E_TIMEOUT if a bounded device-side wait (the mbarrier waits of the
- *   TMA-staged passes, or the self-test's) gave up; the results of those calls
- *   are invalid;
+ * - GRIDSPT_E_TIMEOUT if a bounded device-side wait (the work queue's, or the
+ *   self-test's) gave up; the results of those calls are invalid;
  * - else GRIDSPT_E_NUMERIC if a power, cross-correlation or bispectrum result
  *   was NaN or infinite (a non-finite value in an input spectrum inside the
  *   bins reaches the result; values outside every bin are not seen);
@@ -445,10 +439,9 @@ gridspt_status gridspt_profile_end(gridspt_kernel_stat* stats, int32_t capacity,
 gridspt_status gridspt_check(gridspt_plan plan, gridspt_stream stream);
 
 /* Failure-detection self-test (not part of the paper's method): launches one
- * block that waits, with the same bounded wait as the TMA-staged passes, on a
- * barrier that is never completed. The wait gives up (about 1 ms), the kernel
- * records the timeout and returns; the next gridspt_check reports
- * GRIDSPT_E_TIMEOUT. Nothing faults or hangs. */
+ * block that waits, with a bounded wait, on a barrier that is never completed.
+ * The wait gives up (about 1 ms), the kernel records the timeout and returns;
+ * the next gridspt_check reports GRIDSPT_E_TIMEOUT. Nothing faults or hangs. */
 gridspt_status gridspt_selftest_bounded_wait(gridspt_plan plan, gridspt_stream stream);
 
 /* Message for the last non-OK status returned on this thread ("" if none). */

@@ -346,6 +346,11 @@ gridspt_status gridspt_plan_create(const gridspt_desc* d, gridspt_plan* out) {
     // 192^3, 6.38 / 3.90 at 256^3, 41.6 / 29.8 at 512^3. The z forward pass from
     // N = 256 on: r2c 0.048 / 0.052 ms at 192^3, 0.089 / 0.085 at 256^3, 0.70 /
     // 0.64 at 512^3.
+    // The tiles of the 3 * 2^a grids: narrow x and y tiles where the wide ones leave
+    // a block of 256 threads (192^3: x 2.62 -> 2.56, y 2.62 -> 2.50 ms in all) or of
+    // 1024 at 64 registers (768^3: x 72.3 -> 68.5, y 72.3 -> 67.3), the wide ones at
+    // 384^3 (16.5 against 16.8 and 17.1).
+    p->geo.var[TV_XEXP] = p->geo.var[TV_YEXP] = N % 3 == 0 && N >= 128 && N != 384;
     p->geo.var[TV_ZEXP] = N >= 64 ? 2 : 0;
     p->geo.var[TV_ZR2C] = N >= 256 ? 2 : 0;
     cudaError_t e = cudaGetDevice(&p->device);
@@ -1427,13 +1432,10 @@ gridspt_status gridspt_autotune(gridspt_plan p, void* scratch, size_t scratch_by
         float tbest = 0.f;
         best[pass] = 0;
         for (int v = 0; v < kTuneVariants[pass] && e == cudaSuccess; ++v) {
+            if (tune_variant(p->geo.N, pass, v) != v) continue;   // runs as another one
             Geo g = p->geo;
             g.var[pass] = v;
             e = run(g, pass);   // warm-up
-            if (e == cudaErrorNotSupported) {   // variant not built for this size
-                e = cudaSuccess;
-                continue;
-            }
             if (e == cudaSuccess) e = cudaEventRecord(a, s);
             for (int r = 0; r < 3 && e == cudaSuccess; ++r) e = run(g, pass);
             if (e == cudaSuccess) e = cudaEventRecord(b, s);
@@ -1464,7 +1466,7 @@ gridspt_status gridspt_check(gridspt_plan p, gridspt_stream stream) {
     CK(cudaMemcpy(&st, p->status, sizeof(int), cudaMemcpyDeviceToHost), "check: read status");
     if (st) {
         CK(cudaMemset(p->status, 0, sizeof(int)), "check: reset status");
-        if (st & (kStatusWaitTma | kStatusWaitSelftest | kStatusWaitQueue))
+        if (st & (kStatusWaitSelftest | kStatusWaitQueue))
             return fail(GRIDSPT_E_TIMEOUT, "a bounded device-side wait gave up (status %d); results of the calls "
                                            "since the last check are invalid", st);
         return fail(GRIDSPT_E_NUMERIC, "an estimator produced a NaN or infinite result since the last check "

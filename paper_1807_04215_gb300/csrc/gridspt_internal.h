@@ -14,7 +14,6 @@ constexpr int kMaxOrder = 8;
 constexpr int kPowerMaxBlocks = 1216;
 
 // Bits of the plan's device status word (read and cleared by gridspt_check).
-constexpr int kStatusWaitTma = 1;       // a bounded mbarrier wait of a TMA-staged pass gave up
 constexpr int kStatusWaitSelftest = 2;  // the bounded-wait self-test's wait gave up
 constexpr int kStatusNonFinite = 4;     // an estimator produced a NaN or infinite result
 
@@ -38,18 +37,25 @@ struct Geo {
     int accum;              // estimator shell sums: kAccumCompensated or kAccumFp64
 };
 
-// number of tile variants per pass (the autotuner times each; results are
-// bitwise equal across them):
+// Variant numbers accepted per pass (results are bitwise equal across them):
 //   column pass: 0 wide tile, 1 narrow tile;
-//   x expansion: 0 wide tile, 1 narrow tile, 2 narrow and 3 wide tile with
-//                two outputs per transform (fft_column_pair);
-//   y expansion: 0, 1 tiles, 2 TMA-staged tiles, 3 two columns per thread,
-//                4 narrow tile with cp.async prefetch of the next input,
-//                5 narrow and 6 wide tile with two outputs per transform;
+//   x expansion: 0 wide tile, 1 narrow tile (2 and 3 run 1 and 0);
+//   y expansion: 0 wide tile, 1 narrow tile (2, 3, 6 run 0; 4, 5 run 1);
 //   z expansion (and the fused pair products, bispectrum z pass): 0 tile,
 //                1 tile with cp.async prefetch, 2 warp rows;
 //   z forward pass: 0, 1 tiles, 2 warp rows.
+// The column, x and y passes of the power-of-two N >= 128 have one form, whatever
+// the variant.
 constexpr int kTuneVariants[TV_COUNT] = {2, 4, 7, 3, 3};
+// The variant that variant v of a pass runs as (the autotuner times only those
+// that run as themselves).
+constexpr int tune_variant(int N, int pass, int v) {
+    if (pass <= TV_YEXP) {
+        if (N < 128 || (N & (N - 1)) == 0) return 0;
+        return pass == TV_YEXP ? (v == 1 || v == 4 || v == 5) : pass == TV_XEXP ? (v == 1 || v == 2) : v;
+    }
+    return v == 2 && N == 12 ? 0 : v;
+}
 
 // Unit of the wavevector in the derivative multipliers of the expansion
 // passes: k_F, i.e. integer wavevectors s. Every source term of Eq.

@@ -271,7 +271,7 @@ __device__ void q_tile(const QStage& st, long long tile, float2* sm, bool tr) {
             break;
         case Q_YEXP:
             if constexpr (Col2<N>::ok) col2_yexp_body<N, TZ>(st.y, st.tw, st.kF, bx, by, sm, tr);
-            else yexp_body<N, TZ, false>(st.y, st.tw, st.kF, bx, by, sm, tr);
+            else yexp_body<N, TZ>(st.y, st.tw, st.kF, bx, by, sm, tr);
             break;
         case Q_COLY:
             if constexpr (Col2<N>::ok)

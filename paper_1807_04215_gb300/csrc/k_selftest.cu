@@ -1,5 +1,5 @@
-// Self-test of the bounded device-side wait used by the TMA-staged passes: one
-// block waits on an mbarrier whose phase never completes (no arrival is ever
+// Self-test of a bounded device-side wait and its status path: one block waits
+// on an mbarrier whose phase never completes (no arrival is ever
 // made). The wait gives up after its iteration limit, the kernel records the
 // timeout in the status word and returns. Used only by the failure-detection
 // test; no GPU fault, trap or unbounded spin is involved.

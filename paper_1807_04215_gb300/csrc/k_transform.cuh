@@ -18,8 +18,6 @@
 // packed sequence z[m] = x[2m] + i x[2m+1]; the Nyquist coefficient X[N/2] is
 // zero in every spectrum of this library and is not stored.
 #pragma once
-#include <cuda.h>
-
 #include "fft_core.cuh"
 #include "gridspt_internal.h"
 
@@ -28,12 +26,11 @@ namespace gridspt {
 __host__ __device__ constexpr int cmin(int a, int b) { return a < b ? a : b; }
 __host__ __device__ constexpr int cmax(int a, int b) { return a > b ? a : b; }
 
-// Tile widths. Variant 0 is the default; variant 1 is the alternative width
+// Tile widths. Variant 0 is the wide tile; variant 1 is the alternative width
 // the autotuner also times (only instantiated separately for N >= 128). For
 // the z expansion variant 1 keeps the tile width and instead prefetches the
-// next input tile with cp.async. Further variants per pass are listed with
-// kTuneVariants (TMA-staged, column-pair and prefetching y passes; warp-row z
-// passes).
+// next input tile with cp.async; variant 2 of the z passes runs warp rows. The
+// column passes of the power-of-two N >= 128 have one form (Col2Tile).
 template <int N>
 struct Cfg {
     static constexpr int M = N / 2;
@@ -58,20 +55,17 @@ struct Cfg {
     static_assert(pair_smem(TZP) <= 232448, "fused z pass tiles exceed shared memory");
 };
 
-// Shared memory of the column passes (colpass, x and y expansion): the
-// lane-major stage-twiddle table of fft_col, then NB exchange buffers of
-// col_rows(N) rows of TZ columns (W = 2: column pairs, 16-byte elements), then
-// EXTRA float2 (the y pass's prefetch tile). Two buffers (one barrier per
-// exchange) whenever they fit the 227 KB a block may hold; a variant whose
-// tiles do not fit even with one buffer (the wide column-pair tile of N = 768)
-// is not built for that size.
-template <int N, int TZ, int W = 1, int EXTRA = 0>
+// Shared memory of the column passes (x and y expansion): the lane-major
+// stage-twiddle table of fft_col, then NB exchange buffers of col_rows(N) rows of
+// TZ columns. Two buffers (one barrier per exchange) whenever they fit the 227 KB
+// a block may hold.
+template <int N, int TZ>
 struct ColSm {
     static constexpr int P = N / fft_elems(N);
     static constexpr int TW = (fft_row_tw_total<N>() * P + 1) / 2 * 2;   // 16-byte multiple
-    static constexpr int BUF = col_rows(N) * TZ * W;
-    static constexpr size_t bytes_nb(int nb) { return sizeof(float2) * (TW + (size_t)nb * BUF + EXTRA); }
-    static constexpr bool fits = bytes_nb(1) <= 232448;
+    static constexpr int BUF = col_rows(N) * TZ;
+    static constexpr size_t bytes_nb(int nb) { return sizeof(float2) * (TW + (size_t)nb * BUF); }
+    static_assert(bytes_nb(1) <= 232448, "column tile exceeds shared memory");
     static constexpr int NB = bytes_nb(2) <= 232448 ? 2 : 1;
     static constexpr size_t bytes = bytes_nb(NB);
 };
@@ -289,22 +283,16 @@ __host__ __device__ constexpr int xexp_min_blocks() {
 // fields V_x, V_y, V_z, S are transformed forward along x and combined into
 // A = i k . V, B = -(k^2 / 2) S, delta = cdA A + cdB B, theta = ctA A + ctB B
 // (written to src0, src1 and finalised like MODE 1).
-// PAIR: consecutive outputs (and the two forward inputs) are transformed two
-// at a time by fft_column_pair (shared twiddle loads and barriers, 16-byte
-// exchanges of both transforms' elements; the exchange buffer is twice as
-// large). Per output the arithmetic is that of fft_column, bit for bit.
-template <int N, int TZ, int MODE, bool PAIR = false>
+template <int N, int TZ, int MODE>
 __device__ __forceinline__ void xexp_body(const XExpArgs& args, const float2* __restrict__ twg, float kF,
                                           float inv_kF2, int bx, int by, float2* sm, bool table_ready = false) {
     constexpr int M = N / 2, E = fft_elems(N), P = N / E;
-    using CS = ColSm<N, TZ, PAIR ? 2 : 1>;
+    using CS = ColSm<N, TZ>;
     constexpr int NB = CS::NB;
     float2* twl = sm;
     float2* bufA = sm + CS::TW;
     float2* bufB = bufA + CS::BUF;
     const int tid = threadIdx.x, c = tid % TZ, p = tid / TZ;
-    float4* pairA = reinterpret_cast<float4*>(bufA) + c;
-    float4* pairB = reinterpret_cast<float4*>(bufB) + c;
     if (!table_ready) col_twiddles<N, N>(twl, twg);
     const int kz = bx * TZ + c;
     const int B = args.band;
@@ -365,23 +353,8 @@ __device__ __forceinline__ void xexp_body(const XExpArgs& args, const float2* __
     }
     if constexpr (MODE >= 1) {
         if constexpr (MODE == 1) {
-            if (PAIR && two) {
-                float2 w[2][E];
-#pragma unroll
-                for (int i = 0; i < E; ++i) {
-                    w[0][i] = xd[i];
-                    w[1][i] = xt[i];
-                }
-                fft_col_pair<N, -1, NB>(w, p, pairA, pairB, TZ, twl);
-#pragma unroll
-                for (int i = 0; i < E; ++i) {
-                    xd[i] = w[0][i];
-                    xt[i] = w[1][i];
-                }
-            } else {
-                fft_col<N, -1, NB>(xd, p, bufA + c, bufB + c, TZ, twl);
-                if (two) fft_col<N, -1, NB>(xt, p, bufA + c, bufB + c, TZ, twl);
-            }
+            fft_col<N, -1, NB>(xd, p, bufA + c, bufB + c, TZ, twl);
+            if (two) fft_col<N, -1, NB>(xt, p, bufA + c, bufB + c, TZ, twl);
         }
 #pragma unroll
         for (int i = 0; i < E; ++i) {
@@ -440,39 +413,25 @@ __device__ __forceinline__ void xexp_body(const XExpArgs& args, const float2* __
     };
     auto src_of = [&](int f) { return (args.codes[f] >> 8) & 3; };
     auto is_delta = [&](int f) { return src_of(f) == XS_DELTA; };
-    // transform and store outputs f (and f + 1 when paired) from column sc
-    auto emit = [&](int f, bool pair, const float2 (&sc)[E]) {
-        if (PAIR && pair) {
-            float2 y[2][E];
-            input(f, sc, y[0]);
-            input(f + 1, sc, y[1]);
-            fft_col_pair<N, +1, NB>(y, p, pairA, pairB, TZ, twl);
-            store(f, y[0]);
-            store(f + 1, y[1]);
-        } else {
-            float2 y[E];
-            input(f, sc, y);
-            fft_col<N, +1, NB>(y, p, bufA + c, bufB + c, TZ, twl);
-            store(f, y);
-        }
+    // transform and store output f from column sc
+    auto emit = [&](int f, const float2 (&sc)[E]) {
+        float2 y[E];
+        input(f, sc, y);
+        fft_col<N, +1, NB>(y, p, bufA + c, bufB + c, TZ, twl);
+        store(f, y);
     };
     int f = 0;
-    while (f < args.nout && is_delta(f)) {
-        const bool pair = PAIR && f + 1 < args.nout && is_delta(f + 1);
-        emit(f, pair, xd);
-        f += pair ? 2 : 1;
-    }
+    for (; f < args.nout && is_delta(f); ++f) emit(f, xd);
     if (f < args.nout) {
         float2 xs[E];
         load_col(two ? args.src1 : args.src0, xs);
         bool phi = false;                                 // xs holds theta / k^2
-        while (f < args.nout) {
+        for (; f < args.nout; ++f) {
             const int src = src_of(f);
             if (src == XS_DELTA) {                        // a later delta output: re-read delta
                 float2 d[E];
                 load_col(args.src0, d);
-                emit(f, false, d);
-                f += 1;
+                emit(f, d);
                 continue;
             }
             if (src == XS_PHI && !phi) {
@@ -488,18 +447,16 @@ __device__ __forceinline__ void xexp_body(const XExpArgs& args, const float2* __
                 load_col(two ? args.src1 : args.src0, xs);
                 phi = false;
             }
-            const bool pair = PAIR && f + 1 < args.nout && src_of(f + 1) == src;
-            emit(f, pair, xs);
-            f += pair ? 2 : 1;
+            emit(f, xs);
         }
     }
 }
 
-template <int N, int TZ, int MODE, bool PAIR>
-__global__ void __launch_bounds__(TZ * Cfg<N>::PC, PAIR ? 1 : xexp_min_blocks<N, TZ, MODE>())
+template <int N, int TZ, int MODE>
+__global__ void __launch_bounds__(TZ * Cfg<N>::PC, xexp_min_blocks<N, TZ, MODE>())
 k_xexp(const __grid_constant__ XExpArgs args, const float2* __restrict__ twg, float kF, float inv_kF2) {
     extern __shared__ __align__(16) float2 sm[];
-    xexp_body<N, TZ, MODE, PAIR>(args, twg, kF, inv_kF2, blockIdx.x, blockIdx.y, sm);
+    xexp_body<N, TZ, MODE>(args, twg, kF, inv_kF2, blockIdx.x, blockIdx.y, sm);
 }
 
 // ------------------------------------------------------------ y expansion
@@ -508,22 +465,17 @@ k_xexp(const __grid_constant__ XExpArgs args, const float2* __restrict__ twg, fl
 // registers. In-place use (out == in, one output per input, same index) is
 // safe: a block owns its columns.
 //
-// PF: the next input's column tile is copied into a second shared buffer by
-// cp.async (8-byte, zero-filled where the band excludes it) while the outputs
-// of the current input are transformed. Otherwise the next input's column is
-// prefetched into L2 (prefetch.global.L2), so its loads wait for L2, not HBM.
-// PAIR: two consecutive outputs of the same input are transformed together by
-// fft_column_pair (as in xexp_body; bit for bit the same outputs).
-template <int N, int TZ, bool PF, bool PAIR = false>
+// The next input's column is prefetched into L2 (prefetch.global.L2), so its
+// loads wait for L2, not HBM.
+template <int N, int TZ>
 __device__ __forceinline__ void yexp_body(const YZExpArgs& args, const float2* __restrict__ twg, float kF, int bx,
                                           int by, float2* sm, bool table_ready = false) {
     constexpr int M = N / 2, E = fft_elems(N), P = N / E;
-    using CS = ColSm<N, TZ, PAIR ? 2 : 1, PF ? N * TZ : 0>;
+    using CS = ColSm<N, TZ>;
     constexpr int NB = CS::NB;
     float2* twl = sm;
     float2* bufA = sm + CS::TW;
     float2* bufB = bufA + CS::BUF;
-    float2* pre = bufA + NB * CS::BUF;           // PF: next input tile, element (n, c) at n * TZ + c
     const int tid = threadIdx.x, c = tid % TZ, p = tid / TZ;
     if (!table_ready) col_twiddles<N, N>(twl, twg);
     const int kz = bx * TZ + c;
@@ -534,80 +486,29 @@ __device__ __forceinline__ void yexp_body(const YZExpArgs& args, const float2* _
     const long long colofs = (long long)xr * N * M + kz;
     float2 xin[E];
     int cur = -1;
-    bool have_next = false;
     for (int f = 0; f < args.nout; ++f) {
         const int code = args.codes[f];
         const int in = code & 255, pb = (code >> 8) & 3, slot = code >> 16;
         if (in != cur) {
-            if (PF && have_next) {
-                cp_async_wait_all();
-                __syncthreads();                 // every thread's copies have landed
+            const float2* col = args.in + in * args.in_stride + colofs;
 #pragma unroll
-                for (int i = 0; i < E; ++i) xin[i] = pre[(p + P * i) * TZ + c];
-            } else {
-                const float2* col = args.in + in * args.in_stride + colofs;
+            for (int i = 0; i < E; ++i) {
+                const int sy = signed_idx(p + P * i, N);
+                const bool live = act && (B <= 0 || (sy < B && -sy < B));
+                xin[i] = live ? col[(p + P * i) * estride] : make_float2(0.f, 0.f);
+            }
+            cur = in;
+            int g2 = f + 1;                      // the next distinct input: prefetched into L2 meanwhile
+            while (g2 < args.nout && (args.codes[g2] & 255) == in) ++g2;
+            if (g2 < args.nout) {
+                const float2* nx = args.in + (args.codes[g2] & 255) * args.in_stride + colofs;
 #pragma unroll
                 for (int i = 0; i < E; ++i) {
                     const int sy = signed_idx(p + P * i, N);
                     const bool live = act && (B <= 0 || (sy < B && -sy < B));
-                    xin[i] = live ? col[(p + P * i) * estride] : make_float2(0.f, 0.f);
+                    if (live) prefetch_l2(nx + (p + P * i) * estride);
                 }
             }
-            cur = in;
-            have_next = false;
-            if constexpr (!PF) {                 // the next distinct input: prefetched into L2 meanwhile
-                int g2 = f + 1;
-                while (g2 < args.nout && (args.codes[g2] & 255) == in) ++g2;
-                if (g2 < args.nout) {
-                    const float2* col = args.in + (args.codes[g2] & 255) * args.in_stride + colofs;
-#pragma unroll
-                    for (int i = 0; i < E; ++i) {
-                        const int sy = signed_idx(p + P * i, N);
-                        const bool live = act && (B <= 0 || (sy < B && -sy < B));
-                        if (live) prefetch_l2(col + (p + P * i) * estride);
-                    }
-                }
-            }
-            if constexpr (PF) {                  // the next distinct input, if any
-                int g2 = f + 1;
-                while (g2 < args.nout && (args.codes[g2] & 255) == in) ++g2;
-                if (g2 < args.nout) {
-                    __syncthreads();             // everyone has read the previous prefetch
-                    const float2* col = args.in + (args.codes[g2] & 255) * args.in_stride + colofs;
-#pragma unroll
-                    for (int i = 0; i < E; ++i) {
-                        const int sy = signed_idx(p + P * i, N);
-                        const bool live = act && (B <= 0 || (sy < B && -sy < B));
-                        cp_async8(pre + (p + P * i) * TZ + c, live ? col + (p + P * i) * estride : col, live ? 8 : 0);
-                    }
-                    cp_async_commit();
-                    have_next = true;
-                }
-            }
-        }
-        if (PAIR && f + 1 < args.nout && (args.codes[f + 1] & 255) == in) {
-            const int code1 = args.codes[f + 1];
-            const int pb1 = (code1 >> 8) & 3, slot1 = code1 >> 16;
-            float2 y[2][E];
-#pragma unroll
-            for (int i = 0; i < E; ++i) {
-                const float ky = kF * (float)signed_idx(p + P * i, N);
-                y[0][i] = pb == 0 ? xin[i] : cscale(xin[i], pb == 1 ? ky : ky * ky);
-                y[1][i] = pb1 == 0 ? xin[i] : cscale(xin[i], pb1 == 1 ? ky : ky * ky);
-            }
-            fft_col_pair<N, +1, NB>(y, p, reinterpret_cast<float4*>(bufA) + c, reinterpret_cast<float4*>(bufB) + c,
-                                    TZ, twl);
-            if (act) {
-                float2* o0 = args.out + slot * args.out_stride + colofs;
-                float2* o1 = args.out + slot1 * args.out_stride + colofs;
-#pragma unroll
-                for (int i = 0; i < E; ++i) {
-                    o0[(p + P * i) * estride] = y[0][i];
-                    o1[(p + P * i) * estride] = y[1][i];
-                }
-            }
-            ++f;                                  // the pair's second output is done too
-            continue;
         }
         float2 y[E];
 #pragma unroll
@@ -624,72 +525,11 @@ __device__ __forceinline__ void yexp_body(const YZExpArgs& args, const float2* _
     }
 }
 
-template <int N, int TZ, bool PF, bool PAIR>
-__global__ void __launch_bounds__(TZ * Cfg<N>::PC, (PF || PAIR) ? 1 : col_min_blocks<N, TZ>())
+template <int N, int TZ>
+__global__ void __launch_bounds__(TZ * Cfg<N>::PC, col_min_blocks<N, TZ>())
 k_yexp(const __grid_constant__ YZExpArgs args, const float2* __restrict__ twg, float kF) {
     extern __shared__ __align__(16) float2 sm[];
-    yexp_body<N, TZ, PF, PAIR>(args, twg, kF, blockIdx.x, blockIdx.y, sm);
-}
-
-// Column-pair form of k_yexp: each thread holds two adjacent kz columns, so
-// global and shared accesses move 16 bytes (both columns) and every twiddle
-// load and index computation serves two columns (fft_column_pair); TZ columns
-// (TZ / 2 pairs) per block. Same outputs bit for bit.
-template <int N, int TZ>
-__global__ void __launch_bounds__(TZ / 2 * Cfg<N>::PC)
-k_yexp2(YZExpArgs args, const float2* __restrict__ twg, float kF) {
-    constexpr int M = N / 2, E = fft_elems(N), P = N / E, TP = TZ / 2;
-    static_assert(TZ % 2 == 0 && M % 2 == 0, "column pairs");
-    extern __shared__ __align__(16) float2 sm[];
-    float2* tw = sm;
-    float4* buf = reinterpret_cast<float4*>(sm + N + (N & 1));
-    const int tid = threadIdx.x, c2 = tid % TP, p = tid / TP;
-    load_table(tw, twg, N);
-    const int kz0 = blockIdx.x * TZ + 2 * c2;
-    const int xr = blockIdx.y;
-    const int B = args.band;
-    const bool act0 = kz0 < M && (B <= 0 || kz0 < B);
-    const bool act1 = kz0 + 1 < M && (B <= 0 || kz0 + 1 < B);
-    constexpr long long estride = (long long)M;
-    const long long colofs = (long long)xr * N * M + kz0;
-    float2 xin[2][E];
-    int cur = -1;
-    __syncthreads();
-    for (int f = 0; f < args.nout; ++f) {
-        const int code = args.codes[f];
-        const int in = code & 255, pb = (code >> 8) & 3, slot = code >> 16;
-        if (in != cur) {
-            const float2* col = args.in + in * args.in_stride + colofs;
-#pragma unroll
-            for (int i = 0; i < E; ++i) {
-                const int sy = signed_idx(p + P * i, N);
-                const bool live = act0 && (B <= 0 || (sy < B && -sy < B));
-                const float4 v = live ? *reinterpret_cast<const float4*>(col + (p + P * i) * estride)
-                                      : make_float4(0.f, 0.f, 0.f, 0.f);
-                xin[0][i] = make_float2(v.x, v.y);
-                xin[1][i] = act1 ? make_float2(v.z, v.w) : make_float2(0.f, 0.f);
-            }
-            cur = in;
-        }
-        float2 y[2][E];
-#pragma unroll
-        for (int i = 0; i < E; ++i) {
-            const float ky = kF * (float)signed_idx(p + P * i, N);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) y[h][i] = pb == 0 ? xin[h][i] : cscale(xin[h][i], pb == 1 ? ky : ky * ky);
-        }
-        fft_column_pair<N, +1, N>(y, p, buf + c2, TP, tw);
-        if (act0) {
-            float2* o = args.out + slot * args.out_stride + colofs;
-#pragma unroll
-            for (int i = 0; i < E; ++i) {
-                if (act1)
-                    *reinterpret_cast<float4*>(o + (p + P * i) * estride) = make_float4(y[0][i].x, y[0][i].y, y[1][i].x, y[1][i].y);
-                else
-                    o[(p + P * i) * estride] = y[0][i];
-            }
-        }
-    }
+    yexp_body<N, TZ>(args, twg, kF, blockIdx.x, blockIdx.y, sm);
 }
 
 // ------------------------------------ column passes on the one-exchange transform
@@ -1421,126 +1261,6 @@ k_zrow(const __grid_constant__ ZPairArgs args, const float2* __restrict__ twg, f
                            maxp);
 }
 
-// ------------------------------------------------- TMA-staged y expansion
-// Same computation as k_yexp, but each input column tile (all N rows of TZ
-// adjacent kz columns of one x plane) is copied into shared memory by the
-// tensor-memory accelerator (cp.async.bulk.tensor, 4D map over kz, ky, x and
-// field), completion tracked by an mbarrier, while the previous input's
-// outputs are transformed. The tile being consumed is read into registers and
-// then serves as the transform's exchange buffer. Every wait is bounded: on
-// timeout the kernel sets *status and continues (results are then invalid and
-// gridspt_check reports GRIDSPT_E_TIMEOUT); it never traps or spins forever.
-constexpr unsigned kWaitLimit = 1u << 22;
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"((unsigned)__cvta_generic_to_shared(bar)),
-                 "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(
-                     (unsigned)__cvta_generic_to_shared(bar)), "r"(bytes) : "memory");
-}
-// true when the phase with the given parity has completed; bounded
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity) {
-    const unsigned a = (unsigned)__cvta_generic_to_shared(bar);
-    for (unsigned it = 0; it < kWaitLimit; ++it) {
-        unsigned done;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done) : "r"(a), "r"(parity) : "memory");
-        if (done) return true;
-        if (it > 64) __nanosleep(64);
-    }
-    return false;
-}
-__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
-                                            uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
-        "%5}], [%6];\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
-        "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"((unsigned)__cvta_generic_to_shared(bar))
-        : "memory");
-}
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
-
-// rows per TMA box: the largest divisor of N not above 256 (a box dimension is at most 256)
-__host__ __device__ constexpr int tma_rows(int N) { return N <= 256 ? N : (N % 256 == 0 ? 256 : N / 2 <= 256 ? N / 2 : 192); }
-
-template <int N, int TZ>
-__global__ void __launch_bounds__(TZ * Cfg<N>::PC, (TZ * Cfg<N>::PC <= 512) ? 2 : 1)
-k_yexp_tma(YZExpArgs args, const __grid_constant__ CUtensorMap tmap, const float2* __restrict__ twg, float kF,
-           int* __restrict__ status) {
-    constexpr int M = N / 2, E = fft_elems(N), P = N / E;
-    constexpr int BR = tma_rows(N);
-    static_assert(N % BR == 0 && BR <= 256, "TMA box rows must divide N");
-    constexpr unsigned TILE_BYTES = (unsigned)N * TZ * sizeof(float2);
-    extern __shared__ unsigned char smraw[];
-    // tiles start on a 1024-byte boundary (TMA destinations need at least 128)
-    const unsigned base_off = (1024u - ((unsigned)__cvta_generic_to_shared(smraw) & 1023u)) & 1023u;
-    unsigned char* smb = smraw + base_off;
-    float2* tile[2] = {reinterpret_cast<float2*>(smb), reinterpret_cast<float2*>(smb + TILE_BYTES)};
-    float2* tw = reinterpret_cast<float2*>(smb + 2 * TILE_BYTES);
-    __shared__ uint64_t bar[2];
-    const int tid = threadIdx.x, c = tid % TZ, p = tid / TZ;
-    const int kz0 = blockIdx.x * TZ;
-    const int xr = blockIdx.y;
-    load_table(tw, twg, N);
-    if (tid == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
-        fence_proxy_async();
-    }
-    __syncthreads();
-    auto issue = [&](int b, int in) {   // thread 0 only
-        mbar_expect_tx(&bar[b], TILE_BYTES);
-#pragma unroll
-        for (int r = 0; r < N / BR; ++r) tma_load_4d(tile[b] + r * BR * TZ, &tmap, kz0, r * BR, xr, in, &bar[b]);
-    };
-    if (tid == 0) issue(0, args.codes[0] & 255);
-    unsigned phase[2] = {0u, 0u};
-    int pending[2] = {1, 0};
-    int buf = 0, cur = -1;
-    bool ok = true;
-    constexpr long long estride = (long long)M;
-    const long long colofs = (long long)xr * N * M + kz0 + c;
-    float2 xin[E];
-    for (int f = 0; f < args.nout; ++f) {
-        const int code = args.codes[f];
-        const int in = code & 255, pb = (code >> 8) & 3, slot = code >> 16;
-        if (in != cur) {
-            if (cur >= 0) buf ^= 1;
-            ok = mbar_wait(&bar[buf], phase[buf]) && ok;
-            phase[buf] ^= 1u;
-            pending[buf] = 0;
-#pragma unroll
-            for (int i = 0; i < E; ++i) xin[i] = tile[buf][(p + P * i) * TZ + c];
-            fence_proxy_async();     // generic-proxy use of the other tile ends before the TMA refills it
-            __syncthreads();
-            int nf = f + 1;
-            while (nf < args.nout && (args.codes[nf] & 255) == in) ++nf;
-            if (nf < args.nout) {
-                if (tid == 0) issue(buf ^ 1, args.codes[nf] & 255);
-                pending[buf ^ 1] = 1;
-            }
-            cur = in;
-        }
-        float2 y[E];
-#pragma unroll
-        for (int i = 0; i < E; ++i) {
-            const float ky = kF * (float)signed_idx(p + P * i, N);
-            y[i] = pb == 0 ? xin[i] : cscale(xin[i], pb == 1 ? ky : ky * ky);
-        }
-        fft_column<N, +1, N>(y, p, tile[buf] + c, TZ, tw);
-        float2* o = args.out + slot * args.out_stride + colofs;
-#pragma unroll
-        for (int i = 0; i < E; ++i) o[(p + P * i) * estride] = y[i];
-    }
-    // never leave with a copy in flight into this block's shared memory
-    for (int b = 0; b < 2; ++b)
-        if (pending[b]) ok = mbar_wait(&bar[b], phase[b]) && ok;
-    if (!ok && tid == 0) atomicOr(status, kStatusWaitTma);
-}
-
 // ------------------------------------------- z pass fused with the shell sums
 // Bispectrum estimator, one shell (Sec. III.B.1, Eq. bk_tree, FFT shell
 // estimator): the three xy-fields I_a, I_b, J (nonzero only for kz < band)
@@ -1794,10 +1514,6 @@ k_zrow_r2c(const float2* in, float2* out, long long fstride, int count, const fl
 }
 
 // ------------------------------------------------------------- launchers
-// cuTensorMapEncodeTiled through the runtime's driver entry point (k_tma_host.cpp)
-cudaError_t encode_tensor_map(CUtensorMap* map, void* base, const cuuint64_t* dims, const cuuint64_t* strides,
-                              const cuuint32_t* box, const cuuint32_t* elem_strides);
-
 template <typename K>
 static cudaError_t set_smem(K kernel, size_t bytes) {
     if (bytes > 48 * 1024)
@@ -1861,56 +1577,26 @@ struct Launch {
         k_zr2c<N, TZZ><<<grid, TZZ * PZ, smem, s>>>(in, out, fs, g.tw, scale, band > 0 && band < M ? band : 0);
         return cudaGetLastError();
     }
-    template <bool PAIR = false>
     static cudaError_t xexp(const Geo& g, const XExpArgs& a, cudaStream_t s) {
-        if constexpr (!ColSm<N, TZC, PAIR ? 2 : 1>::fits) return cudaErrorNotSupported;
-        else return xexp_fit<PAIR>(g, a, s);
+        return a.fwd_first && a.div_in ? xexp_m<2>(g, a, s) : a.fwd_first ? xexp_m<1>(g, a, s) : xexp_m<0>(g, a, s);
     }
-    template <bool PAIR>
-    static cudaError_t xexp_fit(const Geo& g, const XExpArgs& a, cudaStream_t s) {
+    template <int MODE>
+    static cudaError_t xexp_m(const Geo& g, const XExpArgs& a, cudaStream_t s) {
         const int B = a.band > 0 && a.band < M ? a.band : 0;
         dim3 grid(((B ? B : M) + TZC - 1) / TZC, B ? 2 * B - 1 : N);
-        const size_t smem = ColSm<N, TZC, PAIR ? 2 : 1>::bytes;
-        const float kF = kDerivUnit, ikF2 = 1.0f / (kDerivUnit * kDerivUnit);
-        cudaError_t e;
-        if (a.fwd_first && a.div_in) {
-            e = set_smem(k_xexp<N, TZC, 2, false>, ColSm<N, TZC>::bytes);
-            if (e != cudaSuccess) return e;
-            k_xexp<N, TZC, 2, false><<<grid, TZC * PC, ColSm<N, TZC>::bytes, s>>>(a, g.tw, kF, ikF2);
-        } else if (a.fwd_first) {
-            e = set_smem(k_xexp<N, TZC, 1, PAIR>, smem);
-            if (e != cudaSuccess) return e;
-            k_xexp<N, TZC, 1, PAIR><<<grid, TZC * PC, smem, s>>>(a, g.tw, kF, ikF2);
-        } else {
-            e = set_smem(k_xexp<N, TZC, 0, PAIR>, smem);
-            if (e != cudaSuccess) return e;
-            k_xexp<N, TZC, 0, PAIR><<<grid, TZC * PC, smem, s>>>(a, g.tw, kF, ikF2);
-        }
-        return cudaGetLastError();
-    }
-    static cudaError_t yexp2(const Geo& g, const YZExpArgs& a, cudaStream_t s) {
-        const int B = a.band > 0 && a.band < M ? a.band : 0;
-        dim3 grid(((B ? B : M) + TZC - 1) / TZC, N);
-        const size_t smem = sizeof(float2) * (N + (N & 1) + (size_t)N * TZC);
-        cudaError_t e = set_smem(k_yexp2<N, TZC>, smem);
+        const size_t smem = ColSm<N, TZC>::bytes;
+        cudaError_t e = set_smem(k_xexp<N, TZC, MODE>, smem);
         if (e != cudaSuccess) return e;
-        k_yexp2<N, TZC><<<grid, TZC / 2 * PC, smem, s>>>(a, g.tw, kDerivUnit);
+        k_xexp<N, TZC, MODE><<<grid, TZC * PC, smem, s>>>(a, g.tw, kDerivUnit, 1.0f / (kDerivUnit * kDerivUnit));
         return cudaGetLastError();
     }
-    template <bool PF = false, bool PAIR = false>
     static cudaError_t yexp(const Geo& g, const YZExpArgs& a, cudaStream_t s) {
-        static_assert(!(PF && PAIR), "prefetching and paired outputs are separate variants");
-        if constexpr (!ColSm<N, TZC, PAIR ? 2 : 1, PF ? N * TZC : 0>::fits) return cudaErrorNotSupported;
-        else return yexp_fit<PF, PAIR>(g, a, s);
-    }
-    template <bool PF, bool PAIR>
-    static cudaError_t yexp_fit(const Geo& g, const YZExpArgs& a, cudaStream_t s) {
         const int B = a.band > 0 && a.band < M ? a.band : 0;
         dim3 grid(((B ? B : M) + TZC - 1) / TZC, N);
-        const size_t smem = ColSm<N, TZC, PAIR ? 2 : 1, PF ? N * TZC : 0>::bytes;
-        cudaError_t e = set_smem(k_yexp<N, TZC, PF, PAIR>, smem);
+        const size_t smem = ColSm<N, TZC>::bytes;
+        cudaError_t e = set_smem(k_yexp<N, TZC>, smem);
         if (e != cudaSuccess) return e;
-        k_yexp<N, TZC, PF, PAIR><<<grid, TZC * PC, smem, s>>>(a, g.tw, kDerivUnit);
+        k_yexp<N, TZC><<<grid, TZC * PC, smem, s>>>(a, g.tw, kDerivUnit);
         return cudaGetLastError();
     }
     template <bool PF>
@@ -1921,32 +1607,6 @@ struct Launch {
         cudaError_t e = set_smem(k_zexp<N, TZZ, PF>, smem);
         if (e != cudaSuccess) return e;
         k_zexp<N, TZZ, PF><<<grid, TZZ * PZ, smem, s>>>(a, g.tw, kDerivUnit);
-        return cudaGetLastError();
-    }
-    // TMA-staged y expansion: 8-column tiles, two tile buffers per block
-    static cudaError_t yexp_tma(const Geo& g, const YZExpArgs& a, cudaStream_t s) {
-        constexpr int TZ = 8;
-        constexpr int BR = tma_rows(N);
-        if (N < 128 || M % TZ != 0) return cudaErrorNotSupported;
-        int nin = 0;
-        for (int f = 0; f < a.nout; ++f) nin = (a.codes[f] & 255) + 1 > nin ? (a.codes[f] & 255) + 1 : nin;
-        CUtensorMap map;
-        // dims: kz (M), ky (N), x (N), field (nin); element = 8 bytes (one float2)
-        const cuuint64_t dims[4] = {(cuuint64_t)M, (cuuint64_t)N, (cuuint64_t)N, (cuuint64_t)nin};
-        const cuuint64_t strides[3] = {(cuuint64_t)M * 8, (cuuint64_t)N * M * 8, (cuuint64_t)a.in_stride * 8};
-        const cuuint32_t box[4] = {(cuuint32_t)TZ, (cuuint32_t)BR, 1, 1};
-        const cuuint32_t estr[4] = {1, 1, 1, 1};
-        // host-side checks of the TMA rules: 16-byte aligned base and strides, inner box
-        // extent a multiple of 16 bytes, box rows <= 256; every kz offset used is a
-        // multiple of TZ = 8 columns (64 bytes)
-        if ((reinterpret_cast<uintptr_t>(a.in) & 15) || (strides[2] & 15) || (TZ * 8) % 16 || BR > 256)
-            return cudaErrorInvalidValue;
-        cudaError_t e = encode_tensor_map(&map, const_cast<float2*>(a.in), dims, strides, box, estr);
-        if (e != cudaSuccess) return e;
-        const size_t smem = 2 * (size_t)N * TZ * sizeof(float2) + sizeof(float2) * N + 1024;   // + alignment slack
-        if ((e = set_smem(k_yexp_tma<N, TZ>, smem)) != cudaSuccess) return e;
-        dim3 grid(M / TZ, N);
-        k_yexp_tma<N, TZ><<<grid, TZ * PC, smem, s>>>(a, map, g.tw, kDerivUnit, g.status);
         return cudaGetLastError();
     }
     static cudaError_t zexp_pairs(const Geo& g, const ZPairArgs& a, cudaStream_t s) {
@@ -2099,15 +1759,37 @@ struct LaunchCol2 {
     }
 };
 
-// Per-size entry points (defined in the k_transform_*.cu units). The pass
-// variant v selects tile widths: v = 0 default, v = 1 alternative.
+// The column passes of one size: the one-exchange form where it exists, else the
+// tile of variant v (0 wide, 1 narrow). The divergence form's x pass holds four
+// columns: always the narrow tile of xexp_body.
+template <int N>
+struct Columns {
+    using Wide = Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>;
+    using Narrow = Launch<N, Cfg<N>::TZC1, Cfg<N>::TZZ0>;
+    using One = LaunchCol2<N, Col2Tile<N>::TZ>;
+    static cudaError_t colpass(const Geo& g, float2* d, long long fs, int count, int axis, int fin, long long s2,
+                               int band, int v, cudaStream_t s) {
+        if constexpr (Col2<N>::ok) return One::colpass(g, d, fs, count, axis, fin, s2, band, s);
+        else return v ? Narrow::colpass(g, d, fs, count, axis, fin, s2, band, s)
+                      : Wide::colpass(g, d, fs, count, axis, fin, s2, band, s);
+    }
+    static cudaError_t xexp(const Geo& g, const XExpArgs& a, int v, cudaStream_t s) {
+        if (a.fwd_first && a.div_in) return Narrow::template xexp_m<2>(g, a, s);
+        if constexpr (Col2<N>::ok) return One::xexp(g, a, s);
+        else return v ? Narrow::xexp(g, a, s) : Wide::xexp(g, a, s);
+    }
+    static cudaError_t yexp(const Geo& g, const YZExpArgs& a, int v, cudaStream_t s) {
+        if constexpr (Col2<N>::ok) return One::yexp(g, a, s);
+        else return v ? Narrow::yexp(g, a, s) : Wide::yexp(g, a, s);
+    }
+};
+
+// Per-size entry points (defined in the k_transform_*.cu units); v: the pass's
+// variant (tune_variant).
 #define GRIDSPT_TRANSFORM_SIZE(N)                                                                          \
     cudaError_t transform_colpass_##N(const Geo& g, float2* d, long long fs, int count, int axis, int fin, \
                                       long long s2, int band, int v, cudaStream_t s) {                     \
-        if constexpr (Col2<N>::ok)                                                                         \
-            return LaunchCol2<N, Col2Tile<N>::TZ>::colpass(g, d, fs, count, axis, fin, s2, band, s);       \
-        else return v ? Launch<N, Cfg<N>::TZC1, Cfg<N>::TZZ0>::colpass(g, d, fs, count, axis, fin, s2, band, s) \
-                 : Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::colpass(g, d, fs, count, axis, fin, s2, band, s); \
+        return Columns<N>::colpass(g, d, fs, count, axis, fin, s2, band, v, s);                            \
     }                                                                                                      \
     cudaError_t transform_zr2c_##N(const Geo& g, const float2* in, float2* out, long long fs, int count,   \
                                    float scale, int band, int v, cudaStream_t s) {                         \
@@ -2117,23 +1799,10 @@ struct LaunchCol2 {
                  : Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::zr2c(g, in, out, fs, count, scale, band, s);     \
     }                                                                                                      \
     cudaError_t transform_xexp_##N(const Geo& g, const XExpArgs& a, int v, cudaStream_t s) {               \
-        if (a.fwd_first && a.div_in) /* four input columns in registers: the narrower tile */              \
-            return Launch<N, Cfg<N>::TZC1, Cfg<N>::TZZ0>::template xexp<false>(g, a, s);                   \
-        if constexpr (Col2<N>::ok) return LaunchCol2<N, Col2Tile<N>::TZ>::xexp(g, a, s);                   \
-        else if (v == 2) return Launch<N, Cfg<N>::TZC1, Cfg<N>::TZZ0>::template xexp<true>(g, a, s);            \
-        if (v == 3) return Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::template xexp<true>(g, a, s);            \
-        return v ? Launch<N, Cfg<N>::TZC1, Cfg<N>::TZZ0>::template xexp<false>(g, a, s)                    \
-                 : Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::template xexp<false>(g, a, s);                   \
+        return Columns<N>::xexp(g, a, v, s);                                                               \
     }                                                                                                      \
     cudaError_t transform_yexp_##N(const Geo& g, const YZExpArgs& a, int v, cudaStream_t s) {              \
-        if constexpr (Col2<N>::ok) return LaunchCol2<N, Col2Tile<N>::TZ>::yexp(g, a, s);                   \
-        else if (v == 2 && N >= 128 && a.band <= 0) return Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::yexp_tma(g, a, s); \
-        if (v == 3) return Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::yexp2(g, a, s);                          \
-        if (v == 4) return Launch<N, Cfg<N>::TZC1, Cfg<N>::TZZ0>::template yexp<true, false>(g, a, s);      \
-        if (v == 5) return Launch<N, Cfg<N>::TZC1, Cfg<N>::TZZ0>::template yexp<false, true>(g, a, s);      \
-        if (v == 6) return Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::template yexp<false, true>(g, a, s);      \
-        return v == 1 ? Launch<N, Cfg<N>::TZC1, Cfg<N>::TZZ0>::template yexp<false, false>(g, a, s)        \
-                      : Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::template yexp<false, false>(g, a, s);       \
+        return Columns<N>::yexp(g, a, v, s);                                                               \
     }                                                                                                      \
     cudaError_t transform_zexp_##N(const Geo& g, const YZExpArgs& a, int v, cudaStream_t s) {              \
         if (a.band & 1) return cudaErrorInvalidValue; /* row copies move kz pairs */                       \

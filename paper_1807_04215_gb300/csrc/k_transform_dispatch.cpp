@@ -36,7 +36,7 @@ cudaError_t launch_colpass_fwd(const Geo& g, float2* data, long long fstride, in
     switch (g.N) {
 #define GRIDSPT_CASE(n)                                                                                       \
     case n:                                                                                                   \
-        return transform_colpass_##n(g, data, fstride, count, axis, finalize, s2_nl, band, g.var[TV_COLPASS], s);
+        return transform_colpass_##n(g, data, fstride, count, axis, finalize, s2_nl, band, tune_variant(g.N, TV_COLPASS, g.var[TV_COLPASS]), s);
         GRIDSPT_ALL_N(GRIDSPT_CASE)
 #undef GRIDSPT_CASE
         default: return cudaErrorInvalidValue;
@@ -47,7 +47,7 @@ cudaError_t launch_zr2c(const Geo& g, const float2* in, float2* out, long long f
                         int band, cudaStream_t s) {
     switch (g.N) {
 #define GRIDSPT_CASE(n) \
-    case n: return transform_zr2c_##n(g, in, out, fstride, count, scale, band, g.var[TV_ZR2C], s);
+    case n: return transform_zr2c_##n(g, in, out, fstride, count, scale, band, tune_variant(g.N, TV_ZR2C, g.var[TV_ZR2C]), s);
         GRIDSPT_ALL_N(GRIDSPT_CASE)
 #undef GRIDSPT_CASE
         default: return cudaErrorInvalidValue;
@@ -56,7 +56,7 @@ cudaError_t launch_zr2c(const Geo& g, const float2* in, float2* out, long long f
 
 cudaError_t launch_xexp(const Geo& g, const XExpArgs& a, cudaStream_t s) {
     switch (g.N) {
-#define GRIDSPT_CASE(n) case n: return transform_xexp_##n(g, a, g.var[TV_XEXP], s);
+#define GRIDSPT_CASE(n) case n: return transform_xexp_##n(g, a, tune_variant(g.N, TV_XEXP, g.var[TV_XEXP]), s);
         GRIDSPT_ALL_N(GRIDSPT_CASE)
 #undef GRIDSPT_CASE
         default: return cudaErrorInvalidValue;
@@ -65,7 +65,7 @@ cudaError_t launch_xexp(const Geo& g, const XExpArgs& a, cudaStream_t s) {
 
 cudaError_t launch_yexp(const Geo& g, const YZExpArgs& a, cudaStream_t s) {
     switch (g.N) {
-#define GRIDSPT_CASE(n) case n: return transform_yexp_##n(g, a, g.var[TV_YEXP], s);
+#define GRIDSPT_CASE(n) case n: return transform_yexp_##n(g, a, tune_variant(g.N, TV_YEXP, g.var[TV_YEXP]), s);
         GRIDSPT_ALL_N(GRIDSPT_CASE)
 #undef GRIDSPT_CASE
         default: return cudaErrorInvalidValue;
@@ -74,7 +74,7 @@ cudaError_t launch_yexp(const Geo& g, const YZExpArgs& a, cudaStream_t s) {
 
 cudaError_t launch_zexp(const Geo& g, const YZExpArgs& a, cudaStream_t s) {
     switch (g.N) {
-#define GRIDSPT_CASE(n) case n: return transform_zexp_##n(g, a, g.var[TV_ZEXP], s);
+#define GRIDSPT_CASE(n) case n: return transform_zexp_##n(g, a, tune_variant(g.N, TV_ZEXP, g.var[TV_ZEXP]), s);
         GRIDSPT_ALL_N(GRIDSPT_CASE)
 #undef GRIDSPT_CASE
         default: return cudaErrorInvalidValue;
