@@ -585,6 +585,20 @@ void diag1_table(const YZExpArgs& za, PairTarget& T) {
     for (int t = 0; t < 3; ++t) term(10 + t, 10 + t, 0.f, 2.f);  // 2 (d_a u_b)^2, a < b
 }
 
+int order_band(const gridspt_plan_s* p, int m, int start);
+
+// Columns kz of an order m >= 2 below n_max that its forward passes write (0: all):
+// its x pass reads only the band columns and its spectra are zeroed outside them.
+int forward_band(const gridspt_plan_s* p, int m, int start) {
+    if (m >= p->d.n_max) return 0;
+    const int b = order_band(p, m, start);
+    return b > 0 && b + (b & 1) < p->geo.M ? b + (b & 1) : 0;
+}
+
+// The z passes of a run transform an order's finished rows forward themselves
+// (PairTarget::r2c); not in the work queue, whose stages do it separately.
+bool fused_r2c(const gridspt_plan_s* p) { return !t_queue && zexp_pairs_r2c(p->geo); }
+
 // z pass of order m fused with the pair products (m, j), j < m, m + j <= n_max,
 // for the targets n' = m + j >= start. Stores the order's real fields when a
 // later order needs them (2m <= n_max). More than two targets are split over
@@ -611,6 +625,12 @@ gridspt_status zexp_pairs(const gridspt_plan_s* p, int m, const YZExpArgs& za, f
         // fields per output over all its targets (order 1 supplies at most one
         // partner per output, higher orders two)
         int partners = 0;
+        // a finished order's rows: 2 fields written, of which the r2c form keeps kz < band
+        auto finish = [&](PairTarget& T, int n) {
+            T.r2c = fused_r2c(p) ? 1 : 0;
+            T.r2c_band = T.r2c ? forward_band(p, n, start) : 0;
+            return fb * 2 * (T.r2c_band ? (double)T.r2c_band / p->geo.M : 1.0);
+        };
         if (m == 1 && n_max >= 2 && start <= 2 && a.store) {   // the diagonal pair (1, 1): all of order 2
             PairTarget& T = a.t[a.ntargets++];
             T.partner = a.store;
@@ -619,7 +639,7 @@ gridspt_status zexp_pairs(const gridspt_plan_s* p, int m, const YZExpArgs& za, f
             T.out_b = reinterpret_cast<float*>(spec_delta[2] + field_c(p));
             recursion_coefs(p, 2, &T.ca0, &T.ca1, &T.cb0, &T.cb1);
             partners = 1;
-            bytes += fb * 2;   // delta_2, theta_2 written; the partners are this launch's own stores
+            bytes += finish(T, 2);   // delta_2, theta_2 written; the partners are this launch's own stores
         }
         for (size_t q = first; q < js.size() && a.ntargets < kMaxPairTargets; ++q, ++first) {
             const int j = js[q], n = m + j;
@@ -640,7 +660,9 @@ gridspt_status zexp_pairs(const gridspt_plan_s* p, int m, const YZExpArgs& za, f
                 T.out_a = reinterpret_cast<float*>(spec_delta[n]);
                 T.out_b = reinterpret_cast<float*>(spec_delta[n] + field_c(p));
                 recursion_coefs(p, n, &T.ca0, &T.ca1, &T.cb0, &T.cb1);
+                bytes += finish(T, n);
             } else {
+                bytes += fb * 2;
                 T.out_a = acc;
                 T.out_b = acc + cells;
                 T.ca0 = 1.f;
@@ -648,7 +670,7 @@ gridspt_status zexp_pairs(const gridspt_plan_s* p, int m, const YZExpArgs& za, f
                 T.cb0 = 0.f;
                 T.cb1 = 1.f;
             }
-            bytes += fb * (j == 1 ? 13 : 17) + fb * 2 + (T.acc_in_a ? fb * 2 : 0);
+            bytes += fb * (j == 1 ? 13 : 17) + (T.acc_in_a ? fb * 2 : 0);
         }
         for (int sl = 0; sl < 17; ++sl) {   // the kernels stage at most kMaxPartners partner tiles
             int c = 0;
@@ -992,15 +1014,12 @@ gridspt_status run_orders_impl(gridspt_plan p, const void* delta1_k, int32_t sta
                 // columns (|ky|, kz < band) and its spectra are zeroed outside them
                 // after it, so the z pass writes only kz < band and the y pass
                 // transforms only those columns and writes only their band rows.
-                int fband = 0;
-                if (m < n_max) {
-                    const int b = order_band(p, m, start_order);
-                    if (b > 0 && b + (b & 1) < p->geo.M) fband = b + (b & 1);
-                }
+                const int fband = forward_band(p, m, start_order);
                 const double fo = fband ? (double)fband / p->geo.M : 1.0;
                 const double fr = fband ? (2.0 * fband - 1.0) / p->geo.N : 1.0;
-                CKQ(PK_ZR2C, (2 + 2 * fo) * fb, s, launch_zr2c(p->geo, dk, dk, F, 2, 1.0f, fband, s), "z r2c",
-                    col(Q_ZR2C));
+                if (!fused_r2c(p))   // else the rows were transformed by the z pass that finished them
+                    CKQ(PK_ZR2C, (2 + 2 * fo) * fb, s, launch_zr2c(p->geo, dk, dk, F, 2, 1.0f, fband, s), "z r2c",
+                        col(Q_ZR2C));
                 CKQ(PK_Y_FWD, 2 * fo * (1 + fr) * fb, s, launch_colpass_fwd(p->geo, dk, F, 2, 1, 0, -1, fband, s),
                     "y pass fwd", col(Q_COLY));
                 if (m == n_max) {

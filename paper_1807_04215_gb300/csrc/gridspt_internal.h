@@ -167,6 +167,9 @@ struct PairTarget {
     float* out_a;               // out_a = ca0 A + ca1 B, out_b = cb0 A + cb1 B
     float* out_b;
     float ca0, ca1, cb0, cb1;
+    int r2c;                    // 1: out_a, out_b receive the rows' forward z transform (half
+                                // spectra rows; the last pair of a target) instead of the rows
+    int r2c_band;               // with r2c, > 0: only kz < r2c_band is written
     int pcount[17];             // per produced slot: number of partner fields (0..2)
     int pfield[17][2];          // partner field index in the stored order; -1: the produced field
                                 // itself (a square), no partner rows are read
@@ -181,6 +184,8 @@ struct ZPairArgs {
     PairTarget t[kMaxPairTargets];
 };
 cudaError_t launch_zexp_pairs(const Geo& g, const ZPairArgs& a, cudaStream_t s);
+// Whether launch_zexp_pairs of this geometry honours PairTarget::r2c (warp rows).
+bool zexp_pairs_r2c(const Geo& g);
 
 struct ProductArgs {
     const float* ws;       // derived fields; order m field j at ws + (base[m] + j) * cells

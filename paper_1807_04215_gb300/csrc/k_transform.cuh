@@ -1271,12 +1271,37 @@ __device__ __forceinline__ void zrow_body(const ZPairArgs& args, const float2* _
                         accB[t][i] = cadd(accB[t][i], vb);
                     }
                 }
-                float2* oa = reinterpret_cast<float2*>(T.out_a) + row * M;
-                float2* ob = reinterpret_cast<float2*>(T.out_b) + row * M;
+                // The two rows of the target, written as they are, or (r2c: the last pair
+                // of an order) transformed forward along z first, as k_zrow_r2c does it,
+                // while they are in registers: that kernel's read and write of two
+                // fields (0.41 ms an order at 512^3) become work of a pass that waits
+                // for memory. 512^3 recursion 26.8 -> 26.2 ms.
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h) {
+                    const float c0 = h ? T.cb0 : T.ca0, c1 = h ? T.cb1 : T.ca1;
+                    float2* o = reinterpret_cast<float2*>(h ? T.out_b : T.out_a) + row * M;
+                    float2 x[E];
 #pragma unroll
-                for (int i = 0; i < E; ++i) {
-                    oa[p + P * i] = lfma(T.ca0, accA[t][i], cscale(accB[t][i], T.ca1));
-                    ob[p + P * i] = lfma(T.cb0, accA[t][i], cscale(accB[t][i], T.cb1));
+                    for (int i = 0; i < E; ++i) x[i] = lfma(c0, accA[t][i], cscale(accB[t][i], c1));
+                    if (T.r2c) {
+                        fft_row<M, -1>(x, p, xrow, twl, bar);
+#pragma unroll
+                        for (int i = 0; i < E; ++i) xrow[xpad(p + P * i)] = x[i];
+                        row_sync<P>(bar);
+#pragma unroll
+                        for (int i = 0; i < E; ++i) {
+                            const int k = p + P * i;
+                            const float2 Z = xrow[xpad(k)];
+                            const float2 Zr = cconj(xrow[xpad(k ? M - k : 0)]);
+                            const float2 S = cadd(Z, Zr);                                // 2 E[k]
+                            const float2 v = cmul(cconj(twp[i * P + p]), csub(Z, Zr));   // e^{-2 pi i k/N} 2i O[k]
+                            if (T.r2c_band <= 0 || k < T.r2c_band) o[k] = make_float2(0.5f * (S.x + v.y), 0.5f * (S.y - v.x));
+                        }
+                        row_sync<P>(bar);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < E; ++i) o[p + P * i] = x[i];
+                    }
                 }
             }
         }

@@ -90,6 +90,8 @@ cudaError_t launch_zexp_pairs(const Geo& g, const ZPairArgs& a, cudaStream_t s) 
     }
 }
 
+bool zexp_pairs_r2c(const Geo& g) { return tune_variant(g.N, TV_ZEXP, g.var[TV_ZEXP]) == 2; }
+
 int shell_blocks(const Geo& g) {
     switch (g.N) {
 #define GRIDSPT_CASE(n) case n: return transform_shell_blocks_##n();
