@@ -12,7 +12,7 @@
 // lane (kz) first, then bins the sums. Only sets inside the top edge are
 // visited. A scan per row, over all N^2 rows with a 64-bit division each, took
 // 121 us per spectrum at 512^3 (top edge |s| = 127, 69 MB of modes); a set-wise
-// one 34 us.
+// one 32 us.
 // Determinism: one warp per set, chunks of 32 consecutive kz (two chunks per
 // step, scanned side by side). Along a row the bin index is
 // non-decreasing in kz, so lanes with equal bins are contiguous: a segmented
@@ -35,7 +35,8 @@
 namespace gridspt {
 
 constexpr int kPowWarps = 8;
-constexpr int kPowBlocks = 456;         // blocks launched at most (the scratch holds power_blocks())
+constexpr int kPowBlocks = 304;         // blocks launched at most: two per SM, all resident (the scratch
+                                        // holds power_blocks(); 456 blocks: 34 us, 304: 32)
 
 int power_blocks(const Geo& g) {
     const long long rows = (long long)g.N * g.N;

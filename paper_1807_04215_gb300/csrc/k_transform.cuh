@@ -542,10 +542,13 @@ k_yexp(const __grid_constant__ YZExpArgs args, const float2* __restrict__ twg, f
 // when i < E / 2. Kernel times against the one-exchange-per-stage tiles: 512^3 x
 // forward + expansion 1.69 -> 1.41 ms, y expansion 2.13 -> 1.90 (7 -> 12 fields), y
 // forward 0.385 -> 0.362, x forward 0.573 -> 0.393 (2 fields); 256^3 0.213 -> 0.158,
-// 0.273 -> 0.204; 1024^3 (one field) x 2.94 -> 2.80, y 2.69 -> 1.97.
+// 0.273 -> 0.204; 1024^3 (one field) x 2.94 -> 1.96, y 2.69 -> 1.99.
+// (1024^3: 8 columns, two 256-thread blocks per SM, take 2.80 / 1.97 / 1.87 / 2.72 ms
+// for x, y, y forward, x forward of one field; 16 columns, one block, 1.96 / 1.99 /
+// 1.93 / 2.03: whole 128-byte lines a megabyte apart count for more.)
 template <int N>
 struct Col2Tile {
-    static constexpr int TZ = N == 1024 ? 8 : 16;
+    static constexpr int TZ = 16;
 };
 
 template <int N, int TZ>
