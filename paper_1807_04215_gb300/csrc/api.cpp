@@ -475,8 +475,8 @@ namespace {
 void expansion_codes(int m, XExpArgs& xa, YZExpArgs& ya, YZExpArgs& za) {
     const int I = 1, NI = 2;  // z-pass constants i and -i
     if (m == 1) {
-        const int xc[5] = {x_code(XK_POW, 0, XS_DELTA), x_code(XK_POW, 1, XS_DELTA), x_code(XK_POW, 0, XS_PHI),
-                           x_code(XK_POW, 1, XS_PHI), x_code(XK_POW, 2, XS_PHI)};
+        const int xc[5] = {x_code(0, XS_DELTA), x_code(1, XS_DELTA), x_code(0, XS_PHI),
+                           x_code(1, XS_PHI), x_code(2, XS_PHI)};
         const int yc[9] = {y_code(0, 0, 0), y_code(0, 1, 1), y_code(1, 0, 2), y_code(2, 0, 3), y_code(2, 1, 4),
                            y_code(2, 2, 5), y_code(3, 0, 6), y_code(3, 1, 7), y_code(4, 0, 8)};
         const int zc[13] = {z_code(0, 0, 0, 0), z_code(0, 1, I, 3), z_code(1, 0, I, 2), z_code(2, 0, I, 1),
@@ -490,9 +490,9 @@ void expansion_codes(int m, XExpArgs& xa, YZExpArgs& ya, YZExpArgs& za) {
         for (int i = 0; i < 9; ++i) ya.codes[i] = yc[i];
         for (int i = 0; i < 13; ++i) za.codes[i] = zc[i];
     } else {
-        const int xc[7] = {x_code(XK_POW, 0, XS_DELTA), x_code(XK_POW, 1, XS_DELTA), x_code(XK_POW, 0, XS_THETA),
-                           x_code(XK_POW, 1, XS_THETA), x_code(XK_POW, 0, XS_PHI), x_code(XK_POW, 1, XS_PHI),
-                           x_code(XK_POW, 2, XS_PHI)};
+        const int xc[7] = {x_code(0, XS_DELTA), x_code(1, XS_DELTA), x_code(0, XS_THETA),
+                           x_code(1, XS_THETA), x_code(0, XS_PHI), x_code(1, XS_PHI),
+                           x_code(2, XS_PHI)};
         const int yc[12] = {y_code(0, 0, 0), y_code(0, 1, 1), y_code(1, 0, 2), y_code(2, 0, 3),
                             y_code(2, 1, 4), y_code(3, 0, 5), y_code(4, 0, 6), y_code(4, 1, 7),
                             y_code(4, 2, 8), y_code(5, 0, 9), y_code(5, 1, 10), y_code(6, 0, 11)};
@@ -819,44 +819,25 @@ gridspt_status derive_order(const gridspt_plan_s* p, int m, float2* dk, float2* 
     return zexp_pairs(p, m, za, ws, start, spec_delta, s);
 }
 
-// Backward transform of `count` fields in place (or in -> out): x, y, z passes
-// with one output per input, optionally with a shell mask (bispectrum).
-gridspt_status backward_fields(const gridspt_plan_s* p, const float2* in0, const float2* in1, float2* out,
-                               long long out_stride, int count, bool shell, long long lo, long long hi,
-                               int band, bool skip_z, cudaStream_t s) {
+// Backward transform of one field, in -> out (which may be in place): x, y, z passes.
+gridspt_status backward_field(const gridspt_plan_s* p, const float2* in, float2* out, cudaStream_t s) {
     const double fb = 4.0 * (double)field_floats(p);
     XExpArgs xa{};
-    xa.src0 = const_cast<float2*>(in0);
-    xa.src1 = const_cast<float2*>(in1);
+    xa.src0 = xa.src1 = const_cast<float2*>(in);
     xa.out = out;
-    xa.out_stride = out_stride;
     xa.s2_nl = -1;
-    xa.shell_lo = lo;
-    xa.shell_hi = hi;
-    xa.band = band;
-    xa.nout = count;
-    const int srcs[3] = {XS_DELTA, in1 == in0 ? XS_DELTA : XS_THETA, XS_ONE};
-    for (int f = 0; f < count; ++f) xa.codes[f] = x_code(shell ? XK_SHELL : XK_POW, 0, srcs[f]);
+    xa.nout = 1;
+    xa.codes[0] = x_code(0, XS_DELTA);
     YZExpArgs ya{};
     ya.in = out;
-    ya.in_stride = out_stride;
     ya.out = out;
-    ya.out_stride = out_stride;
-    ya.nout = count;
-    ya.band = band;
-    for (int f = 0; f < count; ++f) ya.codes[f] = y_code(f, 0, f);
+    ya.nout = 1;
+    ya.codes[0] = y_code(0, 0, 0);
     YZExpArgs za = ya;
-    za.band = 0;
-    for (int f = 0; f < count; ++f) za.codes[f] = z_code(f, 0, 0, f);
-    const int nin = in1 == in0 ? 1 : 2;
-    // algorithmic bytes: with a band B only the band columns move
-    const double N = p->geo.N, M = p->geo.M;
-    const double fx = band > 0 ? (2.0 * band - 1.0) * band / (N * M) : 1.0;   // x columns
-    const double fy_in = band > 0 ? (2.0 * band - 1.0) / N * band / M : 1.0;   // y inputs
-    const double fy_out = band > 0 ? band / M : 1.0;                         // y outputs
-    CKP(shell ? PK_BX : PK_XEXP, fb * fx * (nin + count), s, launch_xexp(p->geo, xa, s), "x pass");
-    CKP(shell ? PK_BY : PK_YEXP, fb * count * (fy_in + fy_out), s, launch_yexp(p->geo, ya, s), "y pass");
-    if (!skip_z) CKP(shell ? PK_BZ : PK_ZEXP, 2 * fb * count, s, launch_zexp(p->geo, za, s), "z pass");
+    za.codes[0] = z_code(0, 0, 0, 0);
+    CKP(PK_XEXP, 2 * fb, s, launch_xexp(p->geo, xa, s), "x pass");
+    CKP(PK_YEXP, 2 * fb, s, launch_yexp(p->geo, ya, s), "y pass");
+    CKP(PK_ZEXP, 2 * fb, s, launch_zexp(p->geo, za, s), "z pass");
     return GRIDSPT_OK;
 }
 
@@ -897,9 +878,9 @@ gridspt_status derive_order_div(const gridspt_plan_s* p, int m, float2* dk, floa
     }
     if (m < n_max) {
         xa.nout = 3;
-        xa.codes[0] = x_code(XK_POW, 0, XS_DELTA);
-        xa.codes[1] = x_code(XK_POW, 0, XS_PHI);
-        xa.codes[2] = x_code(XK_POW, 1, XS_PHI);
+        xa.codes[0] = x_code(0, XS_DELTA);
+        xa.codes[1] = x_code(0, XS_PHI);
+        xa.codes[2] = x_code(1, XS_PHI);
     }
     xa.s2_in = -1;
     YZExpArgs ya{}, za{};
@@ -1591,9 +1572,7 @@ gridspt_status gridspt_c2r(gridspt_plan p, const void* in_k, float* out_x, int32
     const long long F = field_c(p);
     for (int f = 0; f < count; ++f) {
         const float2* in = static_cast<const float2*>(in_k) + f * F;
-        if (gridspt_status st = backward_fields(p, in, in, reinterpret_cast<float2*>(out_x) + f * F, F, 1, false, 0, 0,
-                                                0, false, s))
-            return st;
+        if (gridspt_status st = backward_field(p, in, reinterpret_cast<float2*>(out_x) + f * F, s)) return st;
     }
     return GRIDSPT_OK;
 }
@@ -1832,56 +1811,6 @@ int shell_grid(int N, int band) {
     return N;
 }
 
-// Shell fields of one bispectrum shell on grid g: I_a, I_b (, I_c) and,
-// without a cached sum J^3, J, transformed along x (pruned to |ky|, kz < band)
-// and y into out[f] (stride fstride); the z pass follows fused with the sums.
-// a, b, c are half spectra of grid g.
-gridspt_status shell_fields(const Geo& geo, const float2* a, const float2* b, const float2* c, bool has_j,
-                            long long lo, long long hi, int band, float2* out, long long fstride, cudaStream_t s) {
-    const double N = geo.N, M = geo.M;
-    const double fb = 4.0 * N * N * N;
-    const double fx = band > 0 ? (2.0 * band - 1.0) * band / (N * M) : 1.0;   // x columns
-    const double fy_in = band > 0 ? (2.0 * band - 1.0) / N * band / M : 1.0;   // y inputs
-    const double fy_out = band > 0 ? band / M : 1.0;                         // y outputs
-    auto xpass = [&](const float2* s0, const float2* s1, int first, int count, const int* srcs) -> gridspt_status {
-        XExpArgs xa{};
-        xa.src0 = const_cast<float2*>(s0);
-        xa.src1 = const_cast<float2*>(s1);
-        xa.out = out + first * fstride;
-        xa.out_stride = fstride;
-        xa.s2_nl = -1;
-        xa.shell_lo = lo;
-        xa.shell_hi = hi;
-        xa.band = band;
-        xa.nout = count;
-        for (int f = 0; f < count; ++f) xa.codes[f] = x_code(XK_SHELL, 0, srcs[f]);
-        CKP(PK_BX, fb * fx * ((s0 == s1 ? 1 : 2) + count), s, launch_xexp(geo, xa, s), "x pass");
-        return GRIDSPT_OK;
-    };
-    int nf = 0;
-    if (!c) {
-        const int srcs[3] = {XS_DELTA, b == a ? XS_DELTA : XS_THETA, XS_ONE};
-        if (gridspt_status st = xpass(a, b, 0, has_j ? 3 : 2, srcs)) return st;
-        nf = has_j ? 3 : 2;
-    } else {
-        const int s_ab[2] = {XS_DELTA, b == a ? XS_DELTA : XS_THETA};
-        const int s_cj[2] = {XS_DELTA, XS_ONE};
-        if (gridspt_status st = xpass(a, b, 0, 2, s_ab)) return st;
-        if (gridspt_status st = xpass(c, c, 2, has_j ? 2 : 1, s_cj)) return st;
-        nf = has_j ? 4 : 3;
-    }
-    YZExpArgs ya{};
-    ya.in = out;
-    ya.in_stride = fstride;
-    ya.out = out;
-    ya.out_stride = fstride;
-    ya.nout = nf;
-    ya.band = band;
-    for (int f = 0; f < nf; ++f) ya.codes[f] = y_code(f, 0, f);
-    CKP(PK_BY, fb * nf * (fy_in + fy_out), s, launch_yexp(geo, ya, s), "y pass");
-    return GRIDSPT_OK;
-}
-
 // E = L^6 sum I_a^2 I_b / sum J^3 (c == NULL) or L^6 sum I_a I_b I_c / sum J^3.
 // Each shell is evaluated on the smallest grid that holds its products
 // without aliasing (shell_grid): the inputs are copied onto that grid once per
@@ -1927,53 +1856,97 @@ gridspt_status bispectrum_impl(gridspt_plan p, const void* a_k, const void* b_k,
         if (j == nin) uniq[nin++] = in0[f];
         slot[f] = j;
     }
+    // Consecutive shells on one grid go through the passes together, as many as the
+    // field area and the partial sums hold; the final sums of all shells whose
+    // partials fit are one launch.
+    ShellArgs sa{};
+    ShellFinalArgs fin{};
+    fin.has_j = cached ? 0 : 1;
+    int used = 0;                       // blocks of partial sums in use
     int have = 0;                       // grid size the workspace's inputs are on (0: none)
-    for (int i = 0; i < nbins; ++i) {
+    auto flush = [&]() -> gridspt_status {
+        if (fin.n)
+            CKP(PK_BISPEC, 16.0 * used, s,
+                launch_bispec_final(fin, partial, p->j3, e_out, ntri_out, L * L * L * L * L * L, p->status, s),
+                "bispectrum final sum");
+        fin.n = 0;
+        used = 0;
+        return GRIDSPT_OK;
+    };
+    int i = 0;
+    while (i < nbins) {
         if (bs.thr[i + 1] <= 1) {   // shell holds no mode with k > 0
             CK(cudaMemsetAsync(e_out + i, 0, sizeof(double), s), "bispectrum empty shell");
             CK(cudaMemsetAsync(ntri_out + i, 0, sizeof(double), s), "bispectrum empty shell");
             if (!cached) CK(cudaMemsetAsync(p->j3 + i, 0, sizeof(double), s), "bispectrum empty shell");
+            ++i;
             continue;
         }
-        // every mode of the shell has |s_a| < band in each component
-        const int band = (int)std::floor(std::sqrt((double)(bs.thr[i + 1] - 1))) + 1;
-        int S = shell_grid(N, band);
+        // every mode of shell j has |s_a| < band in each component; its grid
+        auto band_of = [&](int j) { return (int)std::floor(std::sqrt((double)(bs.thr[j + 1] - 1))) + 1; };
         Geo geo{};
-        if (!sub_geo(p, S, &geo)) return fail(GRIDSPT_E_INVALID, "internal: no transform table for grid %d", S);
-        const size_t fs = align256((size_t)S * S * S * sizeof(float));
-        if (S < N && (7 * fs > 4 * fb || shell_blocks(geo) > G)) {
-            S = N;
-            sub_geo(p, S, &geo);
-        }
-        const float2* in[3] = {in0[0], in0[1], in0[2]};
-        float2* fields = reinterpret_cast<float2*>(base);
-        long long fstride = (long long)(fb / sizeof(float2));
+        size_t fs = 0;
+        auto grid_of = [&](int j) {
+            int S = shell_grid(N, band_of(j));
+            if (!sub_geo(p, S, &geo)) return 0;
+            fs = align256((size_t)S * S * S * sizeof(float));
+            if (S < N && (7 * fs > 4 * fb || shell_blocks(geo) > G)) {
+                S = N;
+                sub_geo(p, S, &geo);
+                fs = fb;
+            }
+            return S;
+        };
+        int last = i + 1;               // shells [i, last) share the grid S
+        const int S = grid_of(i);
+        if (!S) return fail(GRIDSPT_E_INVALID, "internal: no transform table for grid %d", shell_grid(N, band_of(i)));
+        while (last < nbins && grid_of(last) == S) ++last;
+        grid_of(i);                     // geo, fs of this grid again
+        const int Gs = shell_blocks(geo);
+        const size_t area = (4 * fb - (S < N ? 3 * fs : 0)) / fs / nf;   // shells the field area holds
+        const int most = (int)std::min<size_t>(area, (size_t)std::max(1, G / Gs));
+        last = std::min(last, i + most);
+        sa.n = last - i;
+        sa.nf = nf;
+        sa.fstride = (long long)(fs / sizeof(float2));
+        float2* small = reinterpret_cast<float2*>(base);
+        sa.out = small + (S < N ? 3 : 0) * sa.fstride;
         if (S < N) {
-            float2* small = reinterpret_cast<float2*>(base);
-            const long long sstride = (long long)(fs / sizeof(float2));
             if (S != have) {
                 CKP(PK_BGATHER, 2.0 * nin * (double)S * S * S * 4.0, s,
-                    launch_subgrid(N, S, uniq, nin, small, sstride, s), "bispectrum sub-grid copy");
+                    launch_subgrid(N, S, uniq, nin, small, sa.fstride, s), "bispectrum sub-grid copy");
                 have = S;
             }
-            for (int f = 0; f < (c_k ? 3 : 2); ++f) in[f] = small + slot[f] * sstride;
-            fields = small + 3 * sstride;
-            fstride = sstride;
         } else {
             have = 0;                   // the full-size shell fields overwrite the copies
         }
-        if (gridspt_status st = shell_fields(geo, in[0], in[1], c_k ? in[2] : nullptr, !cached, bs.thr[i],
-                                             bs.thr[i + 1], band, fields, fstride, s))
-            return st;
-        const double fbytes = 4.0 * (double)S * S * S;
-        const int Gs = shell_blocks(geo);
-        CKP(PK_BZ, fbytes * nf * ((double)band / geo.M), s,
-            launch_zshell(geo, fields, fstride, band, nf, triple, partial, s), "bispectrum z pass and sums");
-        CKP(PK_BISPEC, 16.0 * Gs, s,
-            launch_bispec_final(geo, partial, Gs, cached ? 2 : 3, p->j3 + i, e_out + i, ntri_out + i,
-                                L * L * L * L * L * L, s),
-            "bispectrum final sum");
+        for (int f = 0; f < 4; ++f) sa.in[f] = nullptr;
+        for (int f = 0; f < 2 + triple; ++f) sa.in[f] = S < N ? small + slot[f] * sa.fstride : in0[f];
+        if (used + sa.n * Gs > G)
+            if (gridspt_status st = flush()) return st;
+        double bx = 0.0, by = 0.0, bz = 0.0;                 // algorithmic bytes
+        const double fbytes = 4.0 * (double)S * S * S, M = geo.M;
+        for (int q = 0; q < sa.n; ++q) {
+            const int band = band_of(i + q);
+            sa.lo[q] = bs.thr[i + q];
+            sa.hi[q] = bs.thr[i + q + 1];
+            sa.band[q] = band;
+            const double fx = band < geo.M ? (2.0 * band - 1.0) * band / (S * M) : 1.0;
+            bx += fbytes * fx * (2 + triple + nf);
+            by += fbytes * nf * (band < geo.M ? (2.0 * band - 1.0) / S * band / M + band / M : 2.0);
+            bz += fbytes * nf * std::min(1.0, band / M);
+            fin.off[fin.n] = used + q * Gs;
+            fin.blocks[fin.n] = Gs;
+            fin.bin[fin.n] = i + q;
+            fin.cells[fin.n++] = (double)S * S * S;
+        }
+        CKP(PK_BX, bx, s, launch_xshell(geo, sa, s), "shells: x pass");
+        CKP(PK_BY, by, s, launch_yshell(geo, sa, s), "shells: y pass");
+        CKP(PK_BZ, bz, s, launch_zshell(geo, sa, triple, partial + 2 * used, s), "shells: z pass and sums");
+        used += sa.n * Gs;
+        i = last;
     }
+    if (gridspt_status st = flush()) return st;
     if (!cached) {
         p->j3_nb = nbins;
         for (int i = 0; i <= nbins; ++i) p->j3_thr[i] = bs.thr[i];

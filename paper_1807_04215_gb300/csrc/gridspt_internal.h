@@ -75,15 +75,14 @@ constexpr float kDerivUnit = 1.0f;
 // phi = theta / k^2} and c in {1, i, -i}. Factors of (ky, kz) commute with the
 // transform along x and factors of kz with the transform along y, so the
 // backward transform is split into three expansion passes:
-//   x pass: kx^a * src (or a shell mask), transformed along x    ("x-fields")
+//   x pass: kx^a * src, transformed along x                       ("x-fields")
 //   y pass: ky^b * x-field, transformed along y                    ("xy-fields")
 //   z pass: c * kz^g * xy-field, half-complex -> real along z      (real fields)
 // Each pass reads every input once and writes every output once.
 constexpr int kMaxExpOut = 17;
-enum XKind : int { XK_POW = 0, XK_SHELL = 1 };
-enum XSrc : int { XS_DELTA = 0, XS_THETA = 1, XS_PHI = 2, XS_ONE = 3 };
-// x pass code: kind | a << 4 | src << 8
-constexpr int x_code(int kind, int a, int src) { return kind | (a << 4) | (src << 8); }
+enum XSrc : int { XS_DELTA = 0, XS_THETA = 1, XS_PHI = 2 };
+// x pass code: a << 4 | src << 8
+constexpr int x_code(int a, int src) { return (a << 4) | (src << 8); }
 // y pass code: input index | b << 8 | output slot << 16
 constexpr int y_code(int in, int b, int slot) { return in | (b << 8) | (slot << 16); }
 // z pass code: input index | g << 8 | c << 12 | output slot << 16  (c: 0 -> 1, 1 -> i, 2 -> -i)
@@ -101,8 +100,6 @@ struct XExpArgs {
     long long s2_nl;       // finalise: zero modes with |s|^2 > s2_nl (< 0: no cut)
     int zero_k0;           // finalise: also write the k = 0 mode as zero (orders n >= 2,
                            //    whose k = 0 mode vanishes exactly: mass conservation)
-    long long shell_lo;    // XK_SHELL: 0 < |s|^2, lo <= |s|^2 < hi
-    long long shell_hi;
     int band;              // > 0: only columns with |ky| < band and kz < band are
                            //      read, transformed and written; the others are left
                            //      untouched (their exact values are zero: the
@@ -261,17 +258,35 @@ int power_blocks(const Geo& g);
 cudaError_t launch_power(const Geo& g, const float2* a, const float2* b, const BinSpec& bins,
                          double* partial, double* p_out, int64_t* nk_out, double volume,
                          cudaStream_t s);
-// Bispectrum, one shell: z transform of the xy-fields I_a, I_b (and I_c when
-// triple; then J when present; kz < band) fused with the sums of I_a^2 I_b or
-// I_a I_b I_c (and J^3), per-block partials, then the fixed-order final
-// reduction. nfields counts the data fields and J. sum J^3 does not depend on
-// the data: with has_j (nfields 3 in the final kernel's convention) the final
-// kernel stores it in *j3_cache, otherwise it reads it from there.
+// Bispectrum shells evaluated on one grid: shell i holds the modes with 0 < |s|^2,
+// lo[i] <= |s|^2 < hi[i], whose components are below band[i]. Field f of shell i is
+// at out + (i nf + f) fstride: the masked input in[f], or the mask itself for
+// in[f] == NULL (J, the last field when sum J^3 is not known yet).
+struct ShellArgs {
+    const float2* in[4];
+    float2* out;
+    long long fstride;     // float2 elements between fields
+    int nf;                // fields of a shell (data fields, then J when present)
+    int n;                 // shells
+    int lo[kMaxBins], hi[kMaxBins], band[kMaxBins];
+};
+// x pass, y pass (in place; both move only the columns |ky|, kz < band) and the z
+// pass fused with the sums of I_a^2 I_b, or I_a I_b I_c with triple, and of J^3:
+// FP64 partials of shell i at partial + 2 i shell_blocks().
 int shell_blocks(const Geo& g);
-cudaError_t launch_zshell(const Geo& g, const float2* in, long long in_stride, int band, int nfields, int triple,
-                          double* partial, cudaStream_t s);
-cudaError_t launch_bispec_final(const Geo& g, const double* partial, int blocks, int nfields, double* j3_cache,
-                                double* e_out, double* ntri_out, double vol2, cudaStream_t s);
+cudaError_t launch_xshell(const Geo& g, const ShellArgs& a, cudaStream_t s);
+cudaError_t launch_yshell(const Geo& g, const ShellArgs& a, cudaStream_t s);
+cudaError_t launch_zshell(const Geo& g, const ShellArgs& a, int triple, double* partial, cudaStream_t s);
+// Final reduction of n shells: `blocks[i]` partial pairs from pair off[i] on, grid of
+// cells[i] points; results to entry bin[i] of e_out, ntri_out. sum J^3 does not
+// depend on the data: with has_j it is stored in j3_cache, else read from there.
+struct ShellFinalArgs {
+    int n, has_j;
+    int off[kMaxBins], blocks[kMaxBins], bin[kMaxBins];
+    double cells[kMaxBins];
+};
+cudaError_t launch_bispec_final(const ShellFinalArgs& a, const double* partial, double* j3_cache, double* e_out,
+                                double* ntri_out, double vol2, int* status, cudaStream_t s);
 // Copy the modes of nin half spectra of size N (in[f]) onto a smaller grid of
 // size S (out + f * out_stride, half-spectrum layout of size S): mode s with
 // every component in (-S/2, S/2) keeps its value, the Nyquist planes of the

@@ -240,12 +240,15 @@ cudaError_t launch_power(const Geo& g, const float2* a, const float2* b, const B
 }
 
 // ------------------------------------------------------------ bispectrum
-// Final reduction of the per-block partials written by k_zshell (one shell):
-// E = L^6 sum I_a^2 I_b / sum J^3, N_tri = sum J^3 / N^3; one block, fixed order.
+// Final reduction of the per-block partials written by the shells' z passes, one
+// block per shell, fixed order: E = L^6 sum I_a^2 I_b / sum J^3, N_tri = sum J^3 / N^3.
 __global__ void __launch_bounds__(256)
-k_bispec_final(const double* __restrict__ partial, int G, int nfields, double* __restrict__ j3_cache, double vol2,
-               double cells, double* __restrict__ e_out, double* __restrict__ ntri_out, int* __restrict__ status) {
+k_bispec_final(const __grid_constant__ ShellFinalArgs a, const double* __restrict__ partials,
+               double* __restrict__ j3_cache, double vol2, double* __restrict__ e_out,
+               double* __restrict__ ntri_out, int* __restrict__ status) {
     __shared__ double r1[256], r2[256];
+    const double* partial = partials + 2LL * a.off[blockIdx.x];
+    const int G = a.blocks[blockIdx.x], bin = a.bin[blockIdx.x];
     double s1 = 0.0, s2 = 0.0;
     for (int g = threadIdx.x; g < G; g += 256) {
         s1 += partial[2 * g];
@@ -263,20 +266,19 @@ k_bispec_final(const double* __restrict__ partial, int G, int nfields, double* _
     }
     if (threadIdx.x == 0) {
         double j3 = r2[0];
-        if (nfields == 3) *j3_cache = j3;
-        else j3 = *j3_cache;
-        const double nt = j3 / cells;
+        if (a.has_j) j3_cache[bin] = j3;
+        else j3 = j3_cache[bin];
+        const double nt = j3 / a.cells[blockIdx.x];
         const double ev = nt > 0.5 ? vol2 * r1[0] / j3 : 0.0;
-        *ntri_out = nt;
-        *e_out = ev;
+        ntri_out[bin] = nt;
+        e_out[bin] = ev;
         if (!isfinite(ev) || !isfinite(nt) || !isfinite(r1[0])) atomicOr(status, kStatusNonFinite);
     }
 }
 
-cudaError_t launch_bispec_final(const Geo& g, const double* partial, int blocks, int nfields, double* j3_cache,
-                                double* e_out, double* ntri_out, double vol2, cudaStream_t s) {
-    k_bispec_final<<<1, 256, 0, s>>>(partial, blocks, nfields, j3_cache, vol2, (double)g.N * g.N * g.N, e_out,
-                                     ntri_out, g.status);
+cudaError_t launch_bispec_final(const ShellFinalArgs& a, const double* partial, double* j3_cache, double* e_out,
+                                double* ntri_out, double vol2, int* status, cudaStream_t s) {
+    k_bispec_final<<<a.n, 256, 0, s>>>(a, partial, j3_cache, vol2, e_out, ntri_out, status);
     return cudaGetLastError();
 }
 

@@ -272,8 +272,7 @@ __host__ __device__ constexpr int xexp_min_blocks() {
 }
 
 // Inputs: delta(k) and theta(k) columns along kx. Each output f is
-// kx^a * src (src = delta, theta, phi = theta / k^2 or 1) or a shell mask times
-// src, transformed backward along x. With FWD the inputs first hold the
+// kx^a * src (src = delta, theta or phi = theta / k^2), transformed backward along x. With FWD the inputs first hold the
 // y-transformed product output: they are transformed forward along x and
 // finalised (delta_n(k), theta_n(k) complete, stored back in place), so the
 // spectra are read from HBM once for both directions.
@@ -381,27 +380,14 @@ __device__ __forceinline__ void xexp_body(const XExpArgs& args, const float2* __
     // when its outputs start: MODE 0 reads the input, MODES 1 and 2 re-read the
     // finalised column this thread stored above (its own stores, so the values
     // are those it held).
-    // output f before its transform: kx^a * src (or a shell mask times src),
-    // src (delta, theta or phi) taken from the column sc
+    // output f before its transform: kx^a * src, src (delta, theta or phi) taken
+    // from the column sc
     auto input = [&](int f, const float2 (&sc)[E], float2 (&y)[E]) {
-        const int code = args.codes[f];
-        const int kind = code & 15, pa = (code >> 4) & 3, src = (code >> 8) & 3;
+        const int pa = (args.codes[f] >> 4) & 3;
 #pragma unroll
         for (int i = 0; i < E; ++i) {
-            const int n = p + P * i;
-            const int sx = signed_idx(n, N);
-            const int s2 = sx * sx + syz;
-            const float2 v0 = src == XS_ONE ? make_float2(1.f, 0.f) : sc[i];
-            float2 v = v0;
-            if (kind == XK_POW) {
-                const float kx = kF * (float)sx;
-                if (pa == 1) v = cscale(v, kx);
-                else if (pa == 2) v = cscale(v, kx * kx);
-            } else {
-                const bool in = s2 > 0 && (long long)s2 >= args.shell_lo && (long long)s2 < args.shell_hi;
-                if (!in) v = make_float2(0.f, 0.f);
-            }
-            y[i] = v;
+            const float kx = kF * (float)signed_idx(p + P * i, N);
+            y[i] = pa == 0 ? sc[i] : cscale(sc[i], pa == 1 ? kx : kx * kx);
         }
     };
     auto store = [&](int f, const float2 (&y)[E]) {
@@ -602,8 +588,7 @@ __device__ __forceinline__ void col2_pass_body(float2* __restrict__ data, long l
     }
 }
 
-// The x expansion (see xexp_body): MODE 0 backward only, MODE 1 forward first,
-// MODE 2 backward of shell masks (bispectrum).
+// The x expansion (see xexp_body): MODE 0 backward only, MODE 1 forward first.
 template <int N, int TZ, int MODE>
 __device__ __forceinline__ void col2_xexp_body(const XExpArgs& args, const float2* __restrict__ twg, float kF,
                                                int bx, int by, float2* sm, bool table_ready = false) {
@@ -655,41 +640,31 @@ __device__ __forceinline__ void col2_xexp_body(const XExpArgs& args, const float
     }
     const float cut_in = MODE == 0 && args.s2_in >= 0 ? (float)args.s2_in : 3.e38f;
     // Outputs: the source column is read again for each (MODE 1: this block's
-    // stores above), scaled by its multiplier or shell mask, transformed, stored.
+    // stores above), scaled by its multiplier, transformed, stored.
 #pragma unroll 1
     for (int f = 0; f < args.nout; ++f) {
         const int code = args.codes[f];
         const int pa = (code >> 4) & 3, src = (code >> 8) & 3;
-        load(src != XS_DELTA && two ? args.src1 : args.src0, act && src != XS_ONE);
-        if constexpr (MODE == 2) {
-            const float lo = args.shell_lo > 1 ? (float)args.shell_lo : 1.f, hi = (float)args.shell_hi;
+        load(src != XS_DELTA && two ? args.src1 : args.src0, act);
+        if constexpr (MODE == 0) {
+#pragma unroll
+            for (int i = 0; i < E; ++i) {
+                const float sx = sx_in(i);
+                if (fmaf(sx, sx, syz) > cut_in) x[i] = make_float2(0.f, 0.f);
+            }
+        }
+        if (src == XS_PHI) {
 #pragma unroll
             for (int i = 0; i < E; ++i) {
                 const float sx = sx_in(i), s2 = fmaf(sx, sx, syz);
-                if (src == XS_ONE) x[i].x = 1.f;
-                if (!(s2 >= lo && s2 < hi)) x[i] = make_float2(0.f, 0.f);
+                x[i] = cscale(x[i], s2 > 0.f ? __frcp_rn(s2) : 0.f);   // 1 / k^2 (k_F = 1), 0 at k = 0
             }
-        } else {
-            if constexpr (MODE == 0) {
+        }
+        if (pa) {
 #pragma unroll
-                for (int i = 0; i < E; ++i) {
-                    const float sx = sx_in(i);
-                    if (fmaf(sx, sx, syz) > cut_in) x[i] = make_float2(0.f, 0.f);
-                }
-            }
-            if (src == XS_PHI) {
-#pragma unroll
-                for (int i = 0; i < E; ++i) {
-                    const float sx = sx_in(i), s2 = fmaf(sx, sx, syz);
-                    x[i] = cscale(x[i], s2 > 0.f ? __frcp_rn(s2) : 0.f);   // 1 / k^2 (k_F = 1), 0 at k = 0
-                }
-            }
-            if (pa) {
-#pragma unroll
-                for (int i = 0; i < E; ++i) {
-                    const float kx = kF * sx_in(i);
-                    x[i] = cscale(x[i], pa == 1 ? kx : kx * kx);
-                }
+            for (int i = 0; i < E; ++i) {
+                const float kx = kF * sx_in(i);
+                x[i] = cscale(x[i], pa == 1 ? kx : kx * kx);
             }
         }
         fft_col2<N, +1, TZ>(x, p, buf, sm);
@@ -1320,6 +1295,57 @@ k_zrow(const __grid_constant__ ZPairArgs args, const float2* __restrict__ twg, f
                            maxp);
 }
 
+// ------------------------------------------------ bispectrum shells: x and y
+// The masked fields of several shells on one grid, backward along x, then y (in
+// place): blockIdx.z is the shell, its columns outside |ky|, kz < band are zero and
+// not touched. One launch for all shells of a grid: at the sizes that shells have
+// (8^3 to 128^3 for 256^3 fields) a launch is mostly latency, 16 shells of three
+// to four launches each took 490 us, 275 in groups.
+template <int N, int TZ, bool Y>
+__device__ __forceinline__ void shell_pass(const ShellArgs& args, const float2* __restrict__ twg, float2* sm) {
+    constexpr int M = N / 2;
+    constexpr bool ONE = Col2<N>::ok;
+    constexpr int E = ONE ? Col2<N>::E : fft_elems(N), P = N / E;
+    const int sh = blockIdx.z, band = args.band[sh], B = band < M ? band : 0;   // 0: every column
+    const int rows = Y ? N : B ? 2 * B - 1 : N;
+    if ((int)blockIdx.x * TZ >= (B ? B : M) || (int)blockIdx.y >= rows) return;   // a wider shell's block
+    const int tid = threadIdx.x, c = tid % TZ, p = tid / TZ;
+    float2* buf = sm + (ONE ? Col2<N>::TW : ColSm<N, TZ>::TW);
+    if constexpr (ONE) col2_table<N>(sm, twg);
+    else col_twiddles<N, N>(sm, twg);
+    const int kz = blockIdx.x * TZ + c;
+    const bool act = kz < M && (B <= 0 || kz < B);
+    const int by = blockIdx.y, ky = !Y && B > 0 && by >= B ? N - (2 * B - 1 - by) : by;
+    constexpr long long estride = Y ? M : (long long)N * M;
+    const long long ofs = (long long)ky * (Y ? (long long)N * M : (long long)M) + kz;
+    const int sy = signed_idx(ky, N), syz = sy * sy + kz * kz, lo = args.lo[sh], hi = args.hi[sh];
+    float2* out = args.out + (long long)sh * args.nf * args.fstride + ofs;
+#pragma unroll 1
+    for (int f = 0; f < args.nf; ++f, out += args.fstride) {
+        const float2* in = Y ? out : args.in[f] ? args.in[f] + ofs : nullptr;
+        float2 x[E];
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+            const int n = ONE ? Col2<N>::in_base(p) + Col2<N>::in_step(i) : p + P * i;
+            const int s1 = signed_idx(n, N), s2 = s1 * s1 + syz;
+            const bool live = act && (Y ? B <= 0 || (s1 < B && -s1 < B) : s2 > 0 && s2 >= lo && s2 < hi);
+            x[i] = !live ? make_float2(0.f, 0.f) : in ? in[n * estride] : make_float2(1.f, 0.f);
+        }
+        if constexpr (ONE) fft_col2<N, +1, TZ>(x, p, buf + c, sm);
+        else fft_col<N, +1, ColSm<N, TZ>::NB>(x, p, buf + c, buf + ColSm<N, TZ>::BUF + c, TZ, sm);
+        if (act) {
+#pragma unroll
+            for (int i = 0; i < E; ++i) out[(p + P * i) * estride] = x[i];
+        }
+    }
+}
+template <int N, int TZ, bool Y>
+__global__ void __launch_bounds__(TZ * (Col2<N>::ok ? Col2<N>::P : Cfg<N>::PC))
+k_shell(const __grid_constant__ ShellArgs args, const float2* __restrict__ twg) {
+    extern __shared__ __align__(16) float2 sm[];
+    shell_pass<N, TZ, Y>(args, twg, sm);
+}
+
 // ------------------------------------------- z pass fused with the shell sums
 // Bispectrum estimator, one shell (Sec. III.B.1, Eq. bk_tree, FFT shell
 // estimator): the three xy-fields I_a, I_b, J (nonzero only for kz < band)
@@ -1346,8 +1372,8 @@ __device__ __forceinline__ float cell_mul3(float2 a, float2 b, float2 c) {
 // I_a^2 I_b. NF counts the data fields plus J when present.
 template <int N, int TZ, int NF, bool TRI>
 __global__ void __launch_bounds__(TZ * Cfg<N>::PZ, (TZ * Cfg<N>::PZ <= 512) ? 2 : 1)
-k_zshell(const float2* __restrict__ in, long long in_stride, int band, const float2* __restrict__ twg,
-         double* __restrict__ partial, int f64) {
+k_zshell(const __grid_constant__ ShellArgs args, const float2* __restrict__ twg, double* __restrict__ partial,
+         int f64) {
     constexpr int M = N / 2, E = fft_elems(M), P = M / E, PITCH = Cfg<N>::PITCH, NT = TZ * P;
     extern __shared__ float2 sm[];
     float2* tw = sm;
@@ -1357,7 +1383,10 @@ k_zshell(const float2* __restrict__ in, long long in_stride, int band, const flo
     load_table(tw, twg, N);
     const long long rows = (long long)N * N;
     const long long row0 = (long long)blockIdx.x * TZ;
-    const int B = band < M ? band : M;
+    const int sh = blockIdx.y, B = args.band[sh] < M ? args.band[sh] : M;
+    const long long in_stride = args.fstride;
+    const float2* in = args.out + (long long)sh * args.nf * in_stride;
+    partial += 2LL * sh * gridDim.x;
     // kz < B of each field (asynchronous copies), zeros elsewhere
     for (int f = 0; f < NF; ++f) {
         const float2* src = in + f * in_stride;
@@ -1455,8 +1484,8 @@ k_zshell(const float2* __restrict__ in, long long in_stride, int band, const flo
 // kernel, so the partials are bitwise equal.
 template <int N, int NF, bool TRI>
 __global__ void __launch_bounds__(kRowWarps * 32, 2)
-k_zrow_shell(const float2* __restrict__ in, long long in_stride, int band, const float2* __restrict__ twg,
-             double* __restrict__ partial, int f64) {
+k_zrow_shell(const __grid_constant__ ShellArgs args, const float2* __restrict__ twg, double* __restrict__ partial,
+             int f64) {
     using C = RowCfg<N>;
     constexpr int M = C::M, E = C::E, P = C::P, RW = C::RW;
     constexpr int G = Cfg<N>::TZZ0;
@@ -1468,8 +1497,11 @@ k_zrow_shell(const float2* __restrict__ in, long long in_stride, int band, const
     const int r = lane / P, p = lane - r * P;
     zrow_tables<N>(twl, twp, twg);
     float2* xrow = sm + C::HDR + (warp * RW + r) * C::XROW;
-    const int B = band < M ? band : M;
+    const int sh = blockIdx.y, B = args.band[sh] < M ? args.band[sh] : M;
+    const long long in_stride = args.fstride;
+    const float2* in = args.out + (long long)sh * args.nf * in_stride;
     const long long groups = (long long)N * N / G;
+    partial += 2LL * sh * groups;
     for (long long grp = (long long)blockIdx.x * kRowWarps + warp; grp < groups;
          grp += (long long)gridDim.x * kRowWarps) {
         float s1 = 0.f, c1 = 0.f, s2 = 0.f, c2 = 0.f;   // this lane's chains over its rows
@@ -1726,52 +1758,51 @@ struct Launch {
                                       Cfg<N>::TZZ0 % RowCfg<N>::RW == 0 && (N * N) % Cfg<N>::TZZ0 == 0;
     static int shell_blocks() { return (int)(((long long)N * N + TZZ - 1) / TZZ); }
     template <int NF, bool TRI>
-    static cudaError_t zrow_shell(const Geo& g, const float2* in, long long st, int band, double* partial,
-                                  cudaStream_t s) {
-        using C = RowCfg<N>;
-        if constexpr (!row_shell) {
-            return cudaErrorNotSupported;
-        } else {
-            const size_t smem = sizeof(float2) * (C::HDR + (size_t)kRowWarps * C::RW * C::XROW);
-            cudaError_t e = set_smem(k_zrow_shell<N, NF, TRI>, smem);
-            if (e != cudaSuccess) return e;
-            int dev = 0, sms = 0, per = 0;
-            if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-            if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_zrow_shell<N, NF, TRI>, kRowWarps * 32,
-                                                                     smem)) != cudaSuccess)
-                return e;
-            const long long groups = (long long)N * N / Cfg<N>::TZZ0;
-            const long long need = (groups + kRowWarps - 1) / kRowWarps;
-            const long long resident = (long long)(per > 0 ? per : 1) * sms;
-            k_zrow_shell<N, NF, TRI><<<(unsigned)(need < resident ? need : resident), kRowWarps * 32, smem, s>>>(
-                in, st, band, g.tw, partial, g.accum == kAccumFp64);
-            return cudaGetLastError();
+    static cudaError_t zshell_nf(const Geo& g, const ShellArgs& a, double* partial, cudaStream_t s) {
+        const int f64 = g.accum == kAccumFp64;
+        cudaError_t e;
+        if constexpr (row_shell) {
+            if (g.var[TV_ZEXP] == 2) {
+                using C = RowCfg<N>;
+                const size_t smem = sizeof(float2) * (C::HDR + (size_t)kRowWarps * C::RW * C::XROW);
+                if ((e = set_smem(k_zrow_shell<N, NF, TRI>, smem)) != cudaSuccess) return e;
+                int dev = 0, sms = 0, per = 0;
+                if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+                if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+                if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_zrow_shell<N, NF, TRI>, kRowWarps * 32,
+                                                                         smem)) != cudaSuccess)
+                    return e;
+                const long long need = ((long long)N * N / Cfg<N>::TZZ0 + kRowWarps - 1) / kRowWarps;
+                const long long resident = (long long)(per > 0 ? per : 1) * sms;
+                k_zrow_shell<N, NF, TRI><<<dim3((unsigned)(need < resident ? need : resident), a.n), kRowWarps * 32,
+                                           smem, s>>>(a, g.tw, partial, f64);
+                return cudaGetLastError();
+            }
         }
-    }
-    template <int NF, bool TRI>
-    static cudaError_t zshell_tile(const Geo& g, const float2* in, long long st, int band, double* partial,
-                                   cudaStream_t s) {
         const size_t smem = sizeof(float2) * (N + (size_t)NF * TZZ * PITCH);
-        cudaError_t e = set_smem(k_zshell<N, TZZ, NF, TRI>, smem);
-        if (e != cudaSuccess) return e;
-        k_zshell<N, TZZ, NF, TRI><<<shell_blocks(), TZZ * PZ, smem, s>>>(in, st, band, g.tw, partial,
-                                                                          g.accum == kAccumFp64);
+        if ((e = set_smem(k_zshell<N, TZZ, NF, TRI>, smem)) != cudaSuccess) return e;
+        k_zshell<N, TZZ, NF, TRI><<<dim3(shell_blocks(), a.n), TZZ * PZ, smem, s>>>(a, g.tw, partial, f64);
         return cudaGetLastError();
     }
     // nf: data fields (2: a, b; 3 with tri: a, b, c) plus J when present
-    static cudaError_t zshell(const Geo& g, const float2* in, long long st, int band, int nf, int tri,
-                              double* partial, cudaStream_t s) {
-        if (g.var[TV_ZEXP] == 2 && row_shell && TZZ == Cfg<N>::TZZ0) {
-            if (tri) return nf == 4 ? zrow_shell<4, true>(g, in, st, band, partial, s)
-                                    : zrow_shell<3, true>(g, in, st, band, partial, s);
-            return nf == 3 ? zrow_shell<3, false>(g, in, st, band, partial, s)
-                           : zrow_shell<2, false>(g, in, st, band, partial, s);
-        }
-        if (tri) return nf == 4 ? zshell_tile<4, true>(g, in, st, band, partial, s)
-                                : zshell_tile<3, true>(g, in, st, band, partial, s);
-        return nf == 3 ? zshell_tile<3, false>(g, in, st, band, partial, s)
-                       : zshell_tile<2, false>(g, in, st, band, partial, s);
+    static cudaError_t zshell(const Geo& g, const ShellArgs& a, int tri, double* partial, cudaStream_t s) {
+        if (tri) return a.nf == 4 ? zshell_nf<4, true>(g, a, partial, s) : zshell_nf<3, true>(g, a, partial, s);
+        return a.nf == 3 ? zshell_nf<3, false>(g, a, partial, s) : zshell_nf<2, false>(g, a, partial, s);
+    }
+    // x (Y = false) or y pass of the shells: columns up to the widest band
+    template <bool Y>
+    static cudaError_t shell(const Geo& g, const ShellArgs& a, cudaStream_t s) {
+        constexpr bool ONE = Col2<N>::ok;
+        constexpr int TZ = ONE ? Col2Tile<N>::TZ : TZC;
+        constexpr size_t smem = ONE ? Col2<N>::bytes(TZ) : ColSm<N, TZ>::bytes;
+        int B = 0;                                       // 0: some shell needs every column
+        for (int i = 0; i < a.n; ++i) B = a.band[i] > B ? a.band[i] : B;
+        if (B >= M) B = 0;
+        cudaError_t e = set_smem(k_shell<N, TZ, Y>, smem);
+        if (e != cudaSuccess) return e;
+        const dim3 grid(((B ? B : M) + TZ - 1) / TZ, Y ? N : B ? 2 * B - 1 : N, a.n);
+        k_shell<N, TZ, Y><<<grid, TZ * (ONE ? Col2<N>::P : PC), smem, s>>>(a, g.tw);
+        return cudaGetLastError();
     }
 };
 
@@ -1806,8 +1837,7 @@ struct LaunchCol2 {
         return cudaGetLastError();
     }
     static cudaError_t xexp(const Geo& g, const XExpArgs& a, cudaStream_t s) {
-        const bool shell = a.nout > 0 && (a.codes[0] & 15) == XK_SHELL;   // (a call's outputs are all of one kind)
-        return a.fwd_first ? xexp_m<1>(g, a, s) : shell ? xexp_m<2>(g, a, s) : xexp_m<0>(g, a, s);
+        return a.fwd_first ? xexp_m<1>(g, a, s) : xexp_m<0>(g, a, s);
     }
     static cudaError_t yexp(const Geo& g, const YZExpArgs& a, cudaStream_t s) {
         const int B = a.band > 0 && a.band < M ? a.band : 0;
@@ -1881,9 +1911,15 @@ struct Columns {
                                    : Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::template zrow<2>(g, a, s);       \
         return Launch<N, Cfg<N>::TZC0, Cfg<N>::TZP>::zexp_pairs(g, a, s);                                 \
     }                                                                                                      \
-    cudaError_t transform_zshell_##N(const Geo& g, const float2* in, long long st, int band, int nf,       \
-                                     int tri, double* partial, cudaStream_t s) {                           \
-        return Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::zshell(g, in, st, band, nf, tri, partial, s);        \
+    cudaError_t transform_xshell_##N(const Geo& g, const ShellArgs& a, cudaStream_t s) {                   \
+        return Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::template shell<false>(g, a, s);                      \
+    }                                                                                                      \
+    cudaError_t transform_yshell_##N(const Geo& g, const ShellArgs& a, cudaStream_t s) {                   \
+        return Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::template shell<true>(g, a, s);                       \
+    }                                                                                                      \
+    cudaError_t transform_zshell_##N(const Geo& g, const ShellArgs& a, int tri, double* partial,           \
+                                     cudaStream_t s) {                                                     \
+        return Launch<N, Cfg<N>::TZC0, Cfg<N>::TZZ0>::zshell(g, a, tri, partial, s);                       \
     }
 
 }  // namespace gridspt
