@@ -264,11 +264,12 @@ k_zr2c(const float2* in, float2* out, long long fstride, const float2* __restric
 }
 
 // ------------------------------------------------------------ x expansion
-// Blocks per SM: col_min_blocks (a small spill at 64 registers), except for
-// the divergence form, which keeps four input columns in registers.
+// Blocks per SM: col_min_blocks (a small spill at 64 registers); the divergence
+// form holds three columns at its widest, 128 registers a thread: two blocks of
+// 256 threads (384^3: 0.76 ms, one block at 255 registers 1.09).
 template <int N, int TZ, int MODE>
 __host__ __device__ constexpr int xexp_min_blocks() {
-    return MODE != 2 ? col_min_blocks<N, TZ>() : 1;
+    return MODE != 2 ? col_min_blocks<N, TZ>() : TZ * (N / fft_elems(N)) <= 256 ? 2 : 1;
 }
 
 // Inputs: delta(k) and theta(k) columns along kx. Each output f is
@@ -315,9 +316,11 @@ __device__ __forceinline__ void xexp_body(const XExpArgs& args, const float2* __
         }
     };
     if constexpr (MODE == 2) {
-        float2 A[E], Bs[E];
+        // V_x, V_y, V_z into A, then S: at most A, the column and the transform's
+        // temporaries are live
+        float2 A[E];
 #pragma unroll 1
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < 3; ++q) {
             const float2* col = args.div_in + q * args.div_stride + colofs;
             float2 v[E];
 #pragma unroll
@@ -326,20 +329,23 @@ __device__ __forceinline__ void xexp_body(const XExpArgs& args, const float2* __
 #pragma unroll
             for (int i = 0; i < E; ++i) {
                 const int sx = signed_idx(p + P * i, N);
-                if (q < 3) {
-                    const float kq = kF * (float)(q == 0 ? sx : (q == 1 ? sy : sz));
-                    const float2 t = cmul_i<+1>(cscale(v[i], kq));            // i k_q V_q
-                    A[i] = q == 0 ? t : cadd(A[i], t);
-                } else {
-                    const float k2 = kF * kF * (float)(sx * sx + syz);
-                    Bs[i] = cscale(v[i], -0.5f * k2);                        // -(k^2 / 2) S
-                }
+                const float kq = kF * (float)(q == 0 ? sx : (q == 1 ? sy : sz));
+                const float2 t = cmul_i<+1>(cscale(v[i], kq));                // i k_q V_q
+                A[i] = q == 0 ? t : cadd(A[i], t);
             }
         }
+        const float2* col = args.div_in + 3 * args.div_stride + colofs;
+        float2 v[E];
+#pragma unroll
+        for (int i = 0; i < E; ++i) v[i] = act ? col[(p + P * i) * estride] : make_float2(0.f, 0.f);
+        fft_col<N, -1, NB>(v, p, bufA + c, bufB + c, TZ, twl);
 #pragma unroll
         for (int i = 0; i < E; ++i) {
-            xd[i] = make_float2(fmaf(args.cdA, A[i].x, args.cdB * Bs[i].x), fmaf(args.cdA, A[i].y, args.cdB * Bs[i].y));
-            xt[i] = make_float2(fmaf(args.ctA, A[i].x, args.ctB * Bs[i].x), fmaf(args.ctA, A[i].y, args.ctB * Bs[i].y));
+            const int sx = signed_idx(p + P * i, N);
+            const float k2 = kF * kF * (float)(sx * sx + syz);
+            const float2 B2 = cscale(v[i], -0.5f * k2);                       // -(k^2 / 2) S
+            xd[i] = make_float2(fmaf(args.cdA, A[i].x, args.cdB * B2.x), fmaf(args.cdA, A[i].y, args.cdB * B2.y));
+            xt[i] = make_float2(fmaf(args.ctA, A[i].x, args.ctB * B2.x), fmaf(args.ctA, A[i].y, args.ctB * B2.y));
         }
     } else if constexpr (MODE == 1) {
 #pragma unroll
@@ -407,6 +413,7 @@ __device__ __forceinline__ void xexp_body(const XExpArgs& args, const float2* __
         store(f, y);
     };
     int f = 0;
+    if (MODE == 2 && args.nout > 0) load_col(args.src0, xd);   // the stored column: not held across the store
     for (; f < args.nout && is_delta(f); ++f) emit(f, xd);
     if (f < args.nout) {
         float2 xs[E];
@@ -1669,7 +1676,7 @@ struct Launch {
         return cudaGetLastError();
     }
     static cudaError_t xexp(const Geo& g, const XExpArgs& a, cudaStream_t s) {
-        return a.fwd_first && a.div_in ? xexp_m<2>(g, a, s) : a.fwd_first ? xexp_m<1>(g, a, s) : xexp_m<0>(g, a, s);
+        return a.fwd_first ? xexp_m<1>(g, a, s) : xexp_m<0>(g, a, s);   // the divergence form: xexp_m<2>
     }
     template <int MODE>
     static cudaError_t xexp_m(const Geo& g, const XExpArgs& a, cudaStream_t s) {
