@@ -505,10 +505,13 @@ __global__ void k_convert(const float* __restrict__ src, T* __restrict__ dst, lo
 long long mlp_params(int I, int H, int O) { return (long long)I * H + H + (long long)H * H + H + (long long)H * O + O; }
 int mlp_bwd_blocks(int B) { return (B + kGradRows - 1) / kGradRows; }
 
-template <typename K>
-static cudaError_t smem_attr(K k, size_t bytes) {
-    return bytes > 48 * 1024 ? cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)
-                             : cudaSuccess;
+// The limit of the widest network (256) for every call: two threads with networks
+// of different widths must not lower it under one another's launch.
+template <int R, typename K>
+static cudaError_t smem_attr(K k) {
+    constexpr size_t most = 2 * (size_t)kWBytes + sizeof(float) * (size_t)(row_pitch<R>() * 2 * 256 + 3 * 256);
+    static_assert(most <= 232448, "rows of the widest network exceed shared memory");
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 
 // Rows per block: two while that gives at most two blocks per SM (304), eight
@@ -520,7 +523,7 @@ static cudaError_t mlp_forward_r(const float* x, int B, int I, int H, int O, con
                                  cudaStream_t s) {
     const size_t sm = 2 * (size_t)kWBytes +
                       sizeof(float) * ((size_t)row_pitch<R>() * ((H > I ? H : I) + H) + 2 * H + O);
-    cudaError_t e = smem_attr(k_mlp_forward<T, R>, sm);
+    cudaError_t e = smem_attr<R>(k_mlp_forward<T, R>);
     if (e != cudaSuccess) return e;
     const int wide = H > O ? H : O, ct = FwdTile<R>::CT;
     int nt = (((wide + ct - 1) / ct) * (R / FwdTile<R>::RT) + 31) / 32 * 32;
@@ -546,7 +549,7 @@ template <typename T, int R>
 static cudaError_t mlp_delta_r(int row0, int row1, int I, int H, int O, const void* theta, const float* act,
                                const float* dy, float* d2, float* d1, cudaStream_t s) {
     const size_t sm = 2 * (size_t)kWBytes + sizeof(float) * (size_t)row_pitch<R>() * ((O > H ? O : H) + H);
-    cudaError_t e = smem_attr(k_mlp_delta<T, R>, sm);
+    cudaError_t e = smem_attr<R>(k_mlp_delta<T, R>);
     if (e != cudaSuccess) return e;
     const int need = (H * (R == 2 ? 1 : 2) + 31) / 32 * 32, nt = need < 256 ? 256 : need;
     k_mlp_delta<T, R><<<(unsigned)((row1 - row0 + R - 1) / R), nt, sm, s>>>(

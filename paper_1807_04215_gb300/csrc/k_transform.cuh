@@ -1740,8 +1740,12 @@ struct Launch {
                     for (int q = 0; q < a.t[t].pcount[sl]; ++q) c += a.t[t].pfield[sl][q] >= 0 ? 1 : 0;
                 maxp = c > maxp ? c : maxp;
             }
+            // the limit is that of the largest call: a smaller one set by another
+            // thread between this call and its launch would refuse the launch
+            constexpr size_t most = C::smem(NT > 0 ? kMaxPartners : 0, WARPS);
+            static_assert(most <= 232448, "warp-row z pass exceeds shared memory");
             const size_t smem = C::smem(maxp, WARPS);
-            cudaError_t e = set_smem(k_zrow<N, NT, BAND>, smem);
+            cudaError_t e = set_smem(k_zrow<N, NT, BAND>, most);
             if (e != cudaSuccess) return e;
             int dev = 0, sms = 0, per = 0;
             if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

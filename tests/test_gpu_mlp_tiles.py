@@ -55,3 +55,19 @@ def test_mse_sums_every_element(n):
     L, d = om.masked_mse(y.astype(np.float64), t.astype(np.float64), m.astype(np.float64)) if m.sum() else (0.0, 0 * m)
     assert abs(loss.item() - L) <= 1e-5 * L
     assert np.abs(dy.cpu().numpy() - d).max() <= 1e-5 * max(np.abs(d).max(), 1e-30)
+
+
+def test_networks_of_different_widths_run_from_two_threads():
+    """The kernels' shared memory differs with the width: a thread's launch must
+    not depend on the width of the network that another thread launches."""
+    from concurrent.futures import ThreadPoolExecutor
+
+    def run(H):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            net = g.MLP(3, H, 20, bf16=False, seed=H)
+            x = torch.from_numpy(inputs.rng(H).standard_normal((40, 3)).astype(np.float32)).cuda()
+            ref = net.forward(x)
+            return all(bool(torch.equal(net.forward(x), ref)) for _ in range(200))
+
+    with ThreadPoolExecutor(2) as pool:
+        assert all(pool.map(run, (8, 256)))

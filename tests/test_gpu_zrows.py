@@ -46,3 +46,19 @@ def test_warp_row_shell_sums_equal_the_tile_kernel(N):
                    [t.clone() for t in g.bispectrum_one_loop(plan, d1[0], sp[0, 0, 0], sp[0, 1, 0], sp[0, 2, 0], edges)])
     for a, b in zip(*out):
         assert torch.equal(a, b)
+
+
+def test_recursions_of_different_orders_run_from_two_threads():
+    """The z pass stages as many partner rows as its order has, so its shared
+    memory differs between launches: no launch may depend on another thread's."""
+    from concurrent.futures import ThreadPoolExecutor
+
+    def run(n_max):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            plan = g.Plan(64, n_max, 256.0)
+            d1 = g.make_linear_field(plan, [n_max])
+            ref = g.run_orders(plan, d1).clone()
+            return all(bool(torch.equal(g.run_orders(plan, d1), ref)) for _ in range(100))
+
+    with ThreadPoolExecutor(2) as pool:
+        assert all(pool.map(run, (2, 6)))
