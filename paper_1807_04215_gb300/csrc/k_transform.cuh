@@ -1297,7 +1297,7 @@ template <int N, int NT, bool BAND>
 __global__ void __launch_bounds__(ZRowLaunch<N, NT>::WARPS * 32, ZRowLaunch<N, NT>::MINB)
 k_zrow(const __grid_constant__ ZPairArgs args, const float2* __restrict__ twg, float kF, int maxp) {
     extern __shared__ __align__(16) float2 sm[];
-    constexpr int teams = ZRowLaunch<N, NT>::WARPS * 32 / RowCfg<N>::TL;
+    const int teams = blockDim.x / RowCfg<N>::TL;
     zrow_body<N, NT, BAND>(args, twg, kF, (long long)blockIdx.x * teams, (long long)gridDim.x * teams, sm, false,
                            maxp);
 }
@@ -1732,7 +1732,7 @@ struct Launch {
         if constexpr (!C::ok) {
             return cudaErrorNotSupported;
         } else {
-            constexpr int WARPS = ZRowLaunch<N, NT>::WARPS, TEAMS = WARPS * 32 / C::TL;
+            constexpr int WARPS = ZRowLaunch<N, NT>::WARPS;
             int maxp = 0;                                // partner rows staged for one output
             for (int sl = 0; sl < 17; ++sl) {
                 int c = 0;
@@ -1744,19 +1744,25 @@ struct Launch {
             // thread between this call and its launch would refuse the launch
             constexpr size_t most = C::smem(NT > 0 ? kMaxPartners : 0, WARPS);
             static_assert(most <= 232448, "warp-row z pass exceeds shared memory");
-            const size_t smem = C::smem(maxp, WARPS);
             cudaError_t e = set_smem(k_zrow<N, NT, BAND>, most);
             if (e != cudaSuccess) return e;
             int dev = 0, sms = 0, per = 0;
             if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
             if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_zrow<N, NT, BAND>, WARPS * 32,
-                                                                     smem)) != cudaSuccess)
-                return e;
+            // halve the block while its blocks would not reach every SM: on a small grid
+            // one warp's chain of rows and outputs is the time, and fewer warps share an SM
+            // (recursion 64^3, 64 blocks of 8 warps -> 256 of 2: 95.6 -> 85.5 us)
             const long long groups = (long long)N * N / C::RW;
-            const long long need = (groups + TEAMS - 1) / TEAMS;
+            int warps = WARPS;
+            while (warps > 2 && warps % 2 == 0 && groups * (C::TL / 32) / warps < sms) warps /= 2;
+            const int teams = warps * 32 / C::TL;
+            const size_t smem = C::smem(maxp, warps);
+            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_zrow<N, NT, BAND>, warps * 32, smem)) !=
+                cudaSuccess)
+                return e;
+            const long long need = (groups + teams - 1) / teams;
             const long long resident = (long long)(per > 0 ? per : 1) * sms;
-            k_zrow<N, NT, BAND><<<(unsigned)(need < resident ? need : resident), WARPS * 32, smem, s>>>(
+            k_zrow<N, NT, BAND><<<(unsigned)(need < resident ? need : resident), warps * 32, smem, s>>>(
                 a, g.tw, kDerivUnit, maxp);
             return cudaGetLastError();
         }
