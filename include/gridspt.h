@@ -138,8 +138,9 @@ gridspt_status gridspt_linear_amplitude(const gridspt_cosmo* cosmo, double* ampl
  * c_z = c_y = 0 and c_x > 0) is packed as three 21-bit two's-complement
  * fields; u = (r + 1/2) 2^-32, g1 + i g2 = sqrt(-2 ln u1) e^{2 pi i u2},
  * delta(c) = sqrt(P(|k|) / L^3) (g1 + i g2) / sqrt(2), delta(-c) = conj.
- * Zero: k = 0, Nyquist modes and |s|^2 > (kcut_lin / k_F)^2. FP64 arithmetic,
- * stored as FP32. */
+ * Zero: k = 0, Nyquist modes and |s|^2 > (kcut_lin / k_F)^2. Formed in pairs of
+ * FP32 numbers (relative error 2e-13; the amplitudes' table and sigma_8
+ * in FP64, on the device), stored as FP32. */
 gridspt_status gridspt_make_linear_field(gridspt_plan plan, const gridspt_cosmo* cosmo,
                                          const uint64_t* seeds, void* delta1_k,
                                          gridspt_stream stream);
@@ -190,9 +191,10 @@ gridspt_status gridspt_r2c(gridspt_plan plan, const float* in_x, void* out_k, in
  *   a_k, b_k: device half spectra (one realisation each; b_k may equal a_k).
  *   edges:    HOST double[nbins+1], increasing, edges[nbins] <= k_Ny.
  *   p_out:    device double[nbins]; nk_out: device int64[nbins] (may be NULL).
- *   1 <= nbins <= 64. Products in FP32; runs of up to 32 consecutive modes
- *   of a bin summed in FP32 with each addition's rounding error carried
- *   (two-sum), the runs accumulated in FP64, all reduced in a fixed order
+ *   1 <= nbins <= 64. Products in FP32; the modes of up to eight rows with the
+ *   same |s|^2 at each kz, then up to 32 consecutive kz of a bin, summed in FP32
+ *   with each addition's rounding error carried (two-sum), the runs accumulated
+ *   in FP64, all reduced in a fixed order
  *   (bitwise repeatable); with accum = GRIDSPT_ACCUM_FP64 the products and
  *   every sum are FP64. A NaN or infinite result sets the plan's status
  *   (gridspt_check then returns GRIDSPT_E_NUMERIC). Cross terms of the paper carry a factor
@@ -385,8 +387,9 @@ gridspt_status gridspt_get_tuning(gridspt_plan plan, int32_t* choices);
  *   act: NULL, or FP32 [batch][4 * hidden] saved activations (z1, a1, z2, a2)
  *        for gridspt_mlp_backward.
  * gridspt_mlp_backward: grad = d(sum(dy * y)) / d params (FP32, parameter
- * layout), from x, the parameter copy, act and dy [batch][out]; per-block
- * partial gradients in ws are summed in a fixed order (bitwise repeatable).
+ * layout), from x, the parameter copy, act and dy [batch][out]; the layers'
+ * deltas lie in ws, every gradient element is one sum over the batch in a
+ * fixed order (bitwise repeatable).
  * gridspt_mlp_mse: dy = 2 mask (y - t) / sum(mask), loss = sum(mask (y - t)^2)
  * / sum(mask) over n elements (loss: device float, may be NULL).
  * gridspt_mlp_adam: increments the device step counter *step, then one Adam
