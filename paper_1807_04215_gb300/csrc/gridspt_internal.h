@@ -8,9 +8,8 @@ namespace gridspt {
 
 constexpr int kMaxBins = 64;
 constexpr int kMaxOrder = 8;
-// Blocks of the power estimator's first kernel (one warp per (kx, ky) row,
-// grid-stride): power_blocks() never exceeds this, and the allocation-free
-// entry point's static scratch is sized by it.
+// Blocks that the power estimator's scratch has room for: power_blocks() never
+// exceeds this, and the allocation-free entry point's static scratch is sized by it.
 constexpr int kPowerMaxBlocks = 1216;
 
 // Bits of the plan's device status word (read and cleared by gridspt_check).

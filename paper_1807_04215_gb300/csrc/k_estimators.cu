@@ -31,6 +31,7 @@
 // Bispectrum (Eq. bk_tree, FFT shell estimator): the per-shell sums are formed
 // in k_zshell (k_transform.cuh); the final fixed-order reduction is here.
 #include "gridspt_internal.h"
+#include "pdl.cuh"
 
 namespace gridspt {
 
@@ -99,6 +100,9 @@ k_power(const float2* __restrict__ a, const float2* __restrict__ b, BinSpec bins
     for (int i = threadIdx.x; i < kPowWarps * 2 * kMaxBins; i += blockDim.x) (&acc[0][0])[i] = 0.0;
     for (int i = threadIdx.x; i <= nb; i += blockDim.x) thr[i] = bins.thr[i];
     __syncthreads();
+    pdl_enter();
+    pdl_fresh(a);
+    pdl_fresh(b);
     const int top = thr[nb];
     const bool same = a == b;
     for (int t = blockIdx.x * kPowWarps + w; t < sets; t += gridDim.x * kPowWarps) {
@@ -196,6 +200,8 @@ __global__ void __launch_bounds__(256)
 k_power_final(const double* __restrict__ partial, int G, int nb, double vol,
               double* __restrict__ p_out, int64_t* __restrict__ nk_out, int* __restrict__ status) {
     __shared__ double rs[256], rc[256];
+    pdl_enter();
+    pdl_fresh(partial);
     const int t = blockIdx.x;
     double s = 0.0, c = 0.0;
     for (int g = threadIdx.x; g < G; g += 256) {
@@ -230,12 +236,12 @@ cudaError_t launch_power(const Geo& g, const float2* a, const float2* b, const B
     const int need = (sets + kPowWarps - 1) / kPowWarps, most = power_blocks(g) < kPowBlocks ? power_blocks(g) : kPowBlocks;
     const int G = need < 1 ? 1 : need < most ? need : most;
     if (g.accum == kAccumFp64)
-        k_power<double><<<G, kPowWarps * 32, 0, s>>>(a, b, bins, g.N, g.M, sets, partial);
+        pdl(k_power<double>, G, kPowWarps * 32, 0, s)(a, b, bins, g.N, g.M, sets, partial);
     else
-        k_power<float><<<G, kPowWarps * 32, 0, s>>>(a, b, bins, g.N, g.M, sets, partial);
+        pdl(k_power<float>, G, kPowWarps * 32, 0, s)(a, b, bins, g.N, g.M, sets, partial);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_power_final<<<bins.nbins, 256, 0, s>>>(partial, G, bins.nbins, volume, p_out, nk_out, g.status);
+    pdl(k_power_final, bins.nbins, 256, 0, s)(partial, G, bins.nbins, volume, p_out, nk_out, g.status);
     return cudaGetLastError();
 }
 
@@ -247,6 +253,9 @@ k_bispec_final(const __grid_constant__ ShellFinalArgs a, const double* __restric
                double* __restrict__ j3_cache, double vol2, double* __restrict__ e_out,
                double* __restrict__ ntri_out, int* __restrict__ status) {
     __shared__ double r1[256], r2[256];
+    pdl_enter();
+    pdl_fresh(partials);
+    pdl_fresh(j3_cache);
     const double* partial = partials + 2LL * a.off[blockIdx.x];
     const int G = a.blocks[blockIdx.x], bin = a.bin[blockIdx.x];
     double s1 = 0.0, s2 = 0.0;
@@ -278,7 +287,7 @@ k_bispec_final(const __grid_constant__ ShellFinalArgs a, const double* __restric
 
 cudaError_t launch_bispec_final(const ShellFinalArgs& a, const double* partial, double* j3_cache, double* e_out,
                                 double* ntri_out, double vol2, int* status, cudaStream_t s) {
-    k_bispec_final<<<a.n, 256, 0, s>>>(a, partial, j3_cache, vol2, e_out, ntri_out, status);
+    pdl(k_bispec_final, a.n, 256, 0, s)(a, partial, j3_cache, vol2, e_out, ntri_out, status);
     return cudaGetLastError();
 }
 

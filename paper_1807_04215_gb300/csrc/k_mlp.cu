@@ -23,6 +23,7 @@
 
 #include "fft_core.cuh"
 #include "gridspt_internal.h"
+#include "pdl.cuh"
 
 namespace gridspt {
 
@@ -121,6 +122,9 @@ template <typename T, int R>
 __global__ void __launch_bounds__(256 / FwdTile<R>::CT * (R / FwdTile<R>::RT))
 k_mlp_forward(const float* __restrict__ x, int B, int I, int H, int O, const T* __restrict__ theta,
               float* __restrict__ y, float* __restrict__ act) {
+    pdl_enter();
+    pdl_fresh(x);
+    pdl_fresh(theta);
     constexpr int RT = FwdTile<R>::RT, CT = FwdTile<R>::CT, RP = row_pitch<R>(), G = R / RT;
     extern __shared__ __align__(16) char smraw[];
     T* wb[2] = {reinterpret_cast<T*>(smraw), reinterpret_cast<T*>(smraw + kWBytes)};
@@ -254,6 +258,10 @@ template <typename T, int R>
 __global__ void __launch_bounds__(R == 2 ? 256 : 512)
 k_mlp_delta(int row0, int row1, int I, int H, int O, const T* __restrict__ theta, const float* __restrict__ act,
             const float* __restrict__ dy, float* __restrict__ d2, float* __restrict__ d1) {
+    pdl_enter();
+    pdl_fresh(theta);
+    pdl_fresh(act);
+    pdl_fresh(dy);
     constexpr int RT = R == 2 ? 2 : 4, G = R / RT, RP = row_pitch<R>();
     constexpr int W = 4 / (int)sizeof(T);
     extern __shared__ __align__(16) char smraw[];
@@ -353,6 +361,13 @@ __global__ void __launch_bounds__(kGT * kGT)
 k_mlp_grad(const float* __restrict__ x, int row0, int row1, int I, int H, int O, const float* __restrict__ act,
            const float* __restrict__ dy, const float* __restrict__ d2, const float* __restrict__ d1, int first,
            float* __restrict__ grad) {
+    pdl_enter();
+    pdl_fresh(x);
+    pdl_fresh(act);
+    pdl_fresh(dy);
+    pdl_fresh(d2);
+    pdl_fresh(d1);
+    pdl_fresh(grad);
     constexpr int PER = kGChunk / kGT;
     __shared__ float ls[2][kGChunk][kGT], rs[2][kGChunk][kGT];
     const int th = (H + kGT - 1) / kGT, to = (O + kGT - 1) / kGT;
@@ -528,7 +543,7 @@ static cudaError_t mlp_forward_r(const float* x, int B, int I, int H, int O, con
     const int wide = H > O ? H : O, ct = FwdTile<R>::CT;
     int nt = (((wide + ct - 1) / ct) * (R / FwdTile<R>::RT) + 31) / 32 * 32;
     if (nt < 256) nt = 256;                                        // the copies want threads too
-    k_mlp_forward<T, R><<<(unsigned)((B + R - 1) / R), nt, sm, s>>>(x, B, I, H, O, static_cast<const T*>(theta),
+    pdl(k_mlp_forward<T, R>, (unsigned)((B + R - 1) / R), nt, sm, s)(x, B, I, H, O, static_cast<const T*>(theta),
                                                                          y, act);
     return cudaGetLastError();
 }
@@ -552,7 +567,7 @@ static cudaError_t mlp_delta_r(int row0, int row1, int I, int H, int O, const vo
     cudaError_t e = smem_attr<R>(k_mlp_delta<T, R>);
     if (e != cudaSuccess) return e;
     const int need = (H * (R == 2 ? 1 : 2) + 31) / 32 * 32, nt = need < 256 ? 256 : need;
-    k_mlp_delta<T, R><<<(unsigned)((row1 - row0 + R - 1) / R), nt, sm, s>>>(
+    pdl(k_mlp_delta<T, R>, (unsigned)((row1 - row0 + R - 1) / R), nt, sm, s)(
         row0, row1, I, H, O, static_cast<const T*>(theta), act, dy, d2, d1);
     return cudaGetLastError();
 }
@@ -577,7 +592,7 @@ cudaError_t launch_mlp_backward(const float* x, int B, int I, int H, int O, cons
             e = bf16 ? mlp_delta_r<__nv_bfloat16, 8>(a, b, I, H, O, theta, act, dy, d2, d1, s)
                      : mlp_delta_r<float, 8>(a, b, I, H, O, theta, act, dy, d2, d1, s);
         if (e != cudaSuccess) return e;
-        k_mlp_grad<<<(unsigned)(th * (to + th + 1)), kGT * kGT, 0, s>>>(x, a, b, I, H, O, act, dy, d2, d1, r0 == 0, grad);
+        pdl(k_mlp_grad, (unsigned)(th * (to + th + 1)), kGT * kGT, 0, s)(x, a, b, I, H, O, act, dy, d2, d1, r0 == 0, grad);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;

@@ -20,25 +20,9 @@
 #pragma once
 #include "fft_core.cuh"
 #include "gridspt_internal.h"
+#include "pdl.cuh"
 
 namespace gridspt {
-
-// Programmatic dependent launch. Every block of these kernels first waits for the
-// whole previous kernel of the stream (its writes are then visible), so results and
-// order are as without it; only the launch itself and the block start overlap
-// the previous kernel's end. The next kernel is let in when all blocks have started (no
-// block of this one then waits for an SM that the next one holds); the persistent z
-// passes let it in only when they end, except where each team has one row group:
-// blocks that only wait would keep SMs from the kernels of other streams.
-// Recursion 64^3 85.5 -> 77.1 us, 16 bispectrum shells of 256^3 274 -> 225 us, 192^3
-// 2.29 -> 2.25 ms; from 256^3 on no difference.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_enter() {
-    pdl_wait();
-    pdl_release();
-}
-
 
 __host__ __device__ constexpr int cmin(int a, int b) { return a < b ? a : b; }
 __host__ __device__ constexpr int cmax(int a, int b) { return a > b ? a : b; }
@@ -231,7 +215,7 @@ __device__ __forceinline__ void colpass_body(float2* __restrict__ data, long lon
 
 template <int N, int TZ, int AXIS, bool FIN>
 __global__ void __launch_bounds__(TZ * Cfg<N>::PC)
-k_colpass(float2* __restrict__ data, long long fstride, const float2* __restrict__ twg,
+k_colpass(float2* data, long long fstride, const float2* __restrict__ twg,
           long long s2_nl, int zero_k0, int band) {
     pdl_enter();
     extern __shared__ float2 sm[];
@@ -751,7 +735,7 @@ __device__ __forceinline__ void col2_yexp_body(const YZExpArgs& args, const floa
 
 template <int N, int TZ, int AXIS, bool FIN>
 __global__ void __launch_bounds__(Col2Cfg<N, TZ>::THREADS, Col2Cfg<N, TZ>::MINB)
-k_fcol(float2* __restrict__ data, long long fstride, const float2* __restrict__ twg, long long s2_nl, int zero_k0,
+k_fcol(float2* data, long long fstride, const float2* __restrict__ twg, long long s2_nl, int zero_k0,
        int band) {
     pdl_enter();
     extern __shared__ __align__(16) float2 sm[];
@@ -1643,32 +1627,6 @@ k_zrow_r2c(const float2* in, float2* out, long long fstride, int count, const fl
 }
 
 // ------------------------------------------------------------- launchers
-// A launch that may be placed on the SMs while the stream's previous kernel ends
-// (a programmatic edge, also under capture); the kernel's pdl_wait() orders it.
-template <typename... P>
-struct PdlCall {
-    void (*k)(P...);
-    cudaLaunchConfig_t c;
-    template <typename... A>
-    void operator()(A&&... a) {
-        cudaLaunchAttribute at{};
-        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at.val.programmaticStreamSerializationAllowed = 1;
-        c.attrs = &at;
-        c.numAttrs = 1;
-        cudaLaunchKernelEx(&c, k, static_cast<P>(a)...);   // the caller reads cudaGetLastError()
-    }
-};
-template <typename... P>
-static PdlCall<P...> pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s) {
-    PdlCall<P...> r{k, {}};
-    r.c.gridDim = grid;
-    r.c.blockDim = block;
-    r.c.dynamicSmemBytes = smem;
-    r.c.stream = s;
-    return r;
-}
-
 template <typename K>
 static cudaError_t set_smem(K kernel, size_t bytes) {
     if (bytes > 48 * 1024)
