@@ -217,7 +217,7 @@ template <int N, int TZ, int AXIS, bool FIN>
 __global__ void __launch_bounds__(TZ * Cfg<N>::PC)
 k_colpass(float2* data, long long fstride, const float2* __restrict__ twg,
           long long s2_nl, int zero_k0, int band) {
-    pdl_enter();
+    pdl_wait();
     extern __shared__ float2 sm[];
     colpass_body<N, TZ, AXIS, FIN>(data, fstride, twg, s2_nl, zero_k0, band, blockIdx.x, blockIdx.y, blockIdx.z,
                                    sm);
@@ -227,7 +227,7 @@ k_colpass(float2* data, long long fstride, const float2* __restrict__ twg,
 template <int N, int TZ>
 __global__ void __launch_bounds__(TZ * Cfg<N>::PZ)
 k_zr2c(const float2* in, float2* out, long long fstride, const float2* __restrict__ twg, float scale, int band) {
-    pdl_enter();
+    pdl_wait();
     constexpr int M = N / 2, E = fft_elems(M), P = M / E, PITCH = Cfg<N>::PITCH;
     extern __shared__ float2 sm[];
     float2* tw = sm;
@@ -451,7 +451,7 @@ __device__ __forceinline__ void xexp_body(const XExpArgs& args, const float2* __
 template <int N, int TZ, int MODE>
 __global__ void __launch_bounds__(TZ * Cfg<N>::PC, xexp_min_blocks<N, TZ, MODE>())
 k_xexp(const __grid_constant__ XExpArgs args, const float2* __restrict__ twg, float kF, float inv_kF2) {
-    pdl_enter();
+    pdl_wait();
     extern __shared__ __align__(16) float2 sm[];
     xexp_body<N, TZ, MODE>(args, twg, kF, inv_kF2, blockIdx.x, blockIdx.y, sm);
 }
@@ -525,7 +525,7 @@ __device__ __forceinline__ void yexp_body(const YZExpArgs& args, const float2* _
 template <int N, int TZ>
 __global__ void __launch_bounds__(TZ * Cfg<N>::PC, col_min_blocks<N, TZ>())
 k_yexp(const __grid_constant__ YZExpArgs args, const float2* __restrict__ twg, float kF) {
-    pdl_enter();
+    pdl_wait();
     extern __shared__ __align__(16) float2 sm[];
     yexp_body<N, TZ>(args, twg, kF, blockIdx.x, blockIdx.y, sm);
 }
@@ -737,21 +737,21 @@ template <int N, int TZ, int AXIS, bool FIN>
 __global__ void __launch_bounds__(Col2Cfg<N, TZ>::THREADS, Col2Cfg<N, TZ>::MINB)
 k_fcol(float2* data, long long fstride, const float2* __restrict__ twg, long long s2_nl, int zero_k0,
        int band) {
-    pdl_enter();
+    pdl_wait();
     extern __shared__ __align__(16) float2 sm[];
     col2_pass_body<N, TZ, AXIS, FIN>(data, fstride, twg, s2_nl, zero_k0, band, blockIdx.x, blockIdx.y, blockIdx.z, sm);
 }
 template <int N, int TZ, int MODE>
 __global__ void __launch_bounds__(Col2Cfg<N, TZ>::THREADS, Col2Cfg<N, TZ>::MINB)
 k_xcol(const __grid_constant__ XExpArgs args, const float2* __restrict__ twg, float kF) {
-    pdl_enter();
+    pdl_wait();
     extern __shared__ __align__(16) float2 sm[];
     col2_xexp_body<N, TZ, MODE>(args, twg, kF, blockIdx.x, blockIdx.y, sm);
 }
 template <int N, int TZ>
 __global__ void __launch_bounds__(Col2Cfg<N, TZ>::THREADS, Col2Cfg<N, TZ>::MINB)
 k_ycol(const __grid_constant__ YZExpArgs args, const float2* __restrict__ twg, float kF) {
-    pdl_enter();
+    pdl_wait();
     extern __shared__ __align__(16) float2 sm[];
     col2_yexp_body<N, TZ>(args, twg, kF, blockIdx.x, blockIdx.y, sm);
 }
@@ -765,7 +765,7 @@ k_ycol(const __grid_constant__ YZExpArgs args, const float2* __restrict__ twg, f
 template <int N, int TZ, bool PREFETCH>
 __global__ void __launch_bounds__(TZ * Cfg<N>::PZ, (TZ * Cfg<N>::PZ <= 512) ? 2 : 1)
 k_zexp(YZExpArgs args, const float2* __restrict__ twg, float kF) {
-    pdl_enter();
+    pdl_wait();
     const int B = args.band;                     // > 0: inputs nonzero only at kz < B
     constexpr int M = N / 2, E = fft_elems(M), P = M / E, PITCH = Cfg<N>::PITCH, NT = TZ * P;
     extern __shared__ float2 sm[];
@@ -850,7 +850,7 @@ k_zexp(YZExpArgs args, const float2* __restrict__ twg, float kF) {
 template <int N, int TZ, int NT>
 __global__ void __launch_bounds__(TZ * Cfg<N>::PZ, 1)
 k_zexp_pairs(ZPairArgs args, const float2* __restrict__ twg, float kF) {
-    pdl_enter();
+    pdl_wait();
     constexpr int M = N / 2, E = fft_elems(M), P = M / E, PITCH = Cfg<N>::PITCH, NTH = TZ * P;
     constexpr int MAXP = kMaxPartners;         // partner fields of one output over all targets
     extern __shared__ float2 sm[];
@@ -1361,7 +1361,7 @@ __device__ __forceinline__ void shell_pass(const ShellArgs& args, const float2* 
 template <int N, int TZ, bool Y>
 __global__ void __launch_bounds__(TZ * (Col2<N>::ok ? Col2<N>::P : Cfg<N>::PC))
 k_shell(const __grid_constant__ ShellArgs args, const float2* __restrict__ twg) {
-    pdl_enter();
+    pdl_wait();
     extern __shared__ __align__(16) float2 sm[];
     shell_pass<N, TZ, Y>(args, twg, sm);
 }
@@ -1394,7 +1394,7 @@ template <int N, int TZ, int NF, bool TRI>
 __global__ void __launch_bounds__(TZ * Cfg<N>::PZ, (TZ * Cfg<N>::PZ <= 512) ? 2 : 1)
 k_zshell(const __grid_constant__ ShellArgs args, const float2* __restrict__ twg, double* __restrict__ partial,
          int f64) {
-    pdl_enter();
+    pdl_wait();
     constexpr int M = N / 2, E = fft_elems(M), P = M / E, PITCH = Cfg<N>::PITCH, NT = TZ * P;
     extern __shared__ float2 sm[];
     float2* tw = sm;

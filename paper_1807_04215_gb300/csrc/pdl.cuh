@@ -5,16 +5,18 @@ namespace gridspt {
 
 // Programmatic dependent launch. Every block of these kernels first waits for the
 // whole previous kernel of the stream (its writes are then visible), so results and
-// order are as without it; only the launch itself and the block start overlap
-// the previous kernel's end. The next kernel is let in when all blocks have started (no
-// block of this one then waits for an SM that the next one holds); the persistent z
-// passes let it in only when they end, except where each team has one row group:
-// blocks that only wait would keep SMs from the kernels of other streams.
+// order are as without it; only the launch itself overlaps the previous kernel's end.
+// The transform and shell passes (pdl_wait) let the next kernel in when their last block ends.
+// Letting it in as soon as all blocks have started places the next kernel's blocks
+// wherever there is room while this one runs: several on one SM, none on others, and
+// they stay there. Fifth order, early / at the end / no programmatic launch, replayed
+// from a graph and launched on a stream: 96^3 481 / 365 / 360 and 491 / 374 / 406 us,
+// 64^3 201 / 147 / 150 and 212 / 156 / 197, 128^3 533 / 492 / 492; r2c at 96^3 18.4 /
+// 14.6 / 15.6. The power, shell-sum and emulator kernels let it in early (pdl_enter): their
+// successors are small (the final sums of a power call: 0.6 us of 7 later otherwise),
+// and so do z passes whose teams have one row group each (c2r at 48^3: 0.5 of 13 us).
 // A pointer that an earlier kernel writes through is not __restrict__ here, or passes
 // pdl_fresh(): the compiler may move loads through a restrict parameter over the wait.
-// Recursion 64^3 85.5 -> 77.1 us, 16 bispectrum shells of 256^3 274 -> 225 us, 192^3
-// 2.29 -> 2.25 ms, from 256^3 on no difference; six 512^3 spectra 230 -> 207 us,
-// emulator: 4096 rows predicted 20.5 -> 18.6 us, training step 41 -> 39.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter() {
