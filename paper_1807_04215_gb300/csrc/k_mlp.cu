@@ -17,7 +17,7 @@
 // Measured (kernel times, bf16, 3 -> 128 -> 128 -> 160, against 8/16-block
 // kernels that read the weights from global memory in the chains):
 //   forward 256 rows 61 -> 9.5 us, 4096 rows 57 -> 21; backward 256 rows
-//   267 -> 19; mse 41 k elements 26 -> 7; Adam 6.5 (two launches) -> 7.5.
+//   267 -> 19; mse 41 k elements 26 -> 7. Loss and Adam: beside their kernels.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
@@ -483,20 +483,24 @@ k_mlp_mse(const float* __restrict__ y, const float* __restrict__ t, const float*
 }
 
 // Adam (Kingma & Ba 2015) on the FP32 master parameters; the step count lives
-// in device memory so that a captured training step can be replayed. One
-// cluster: every block reads the count, and after the cluster barrier one
-// thread increments it (no second launch).
+// in device memory (incremented by a launch before) so that a captured training
+// step can be replayed. Blocks over the whole GPU: one cluster of 16 blocks that
+// increments the count itself, without the first launch, took 5.7 us at 38 k
+// parameters, 11.8 at 133 k and 66 at 1 M in a graph against 3.2, 4.4 and 15, and a
+// whole step of 256 rows (38 k) takes 36 us either way.
+__global__ void k_step_inc(int* step) {
+    pdl_enter();
+    pdl_fresh(step);
+    *step += 1;
+}
 template <typename T>
-__global__ void __launch_bounds__(1024)
-k_mlp_adam(float* __restrict__ master, T* __restrict__ lowp, const float* __restrict__ grad, float* __restrict__ m,
-           float* __restrict__ v, int* __restrict__ step, long long n, float lr, float b1, float b2, float eps) {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cl = cg::this_cluster();
-    const int t = *reinterpret_cast<volatile int*>(step) + 1;
-    cl.barrier_arrive();                                          // this thread has read the old count
+__global__ void __launch_bounds__(256)
+k_mlp_adam(float* master, T* __restrict__ lowp, const float* grad, float* m, float* v, const int* step, long long n,
+           float lr, float b1, float b2, float eps) {
+    pdl_wait();
+    const int t = *step;
     const float c1 = 1.f - powf(b1, (float)t), c2 = 1.f - powf(b2, (float)t);
-#pragma unroll 2
-    for (long long i = (long long)blockIdx.x * 1024 + threadIdx.x; i < n; i += 1024LL * kOptCluster) {
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const float g = grad[i];
         const float mi = b1 * m[i] + (1.f - b1) * g;
         const float vi = b2 * v[i] + (1.f - b2) * g * g;
@@ -506,8 +510,6 @@ k_mlp_adam(float* __restrict__ master, T* __restrict__ lowp, const float* __rest
         master[i] = p;
         if (lowp) lowp[i] = from_f<T>(p);
     }
-    cl.barrier_wait();                                            // every thread has
-    if (blockIdx.x == 0 && threadIdx.x == 0) *step = t;
 }
 
 template <typename T>
@@ -621,11 +623,21 @@ cudaError_t launch_mlp_mse(const float* y, const float* t, const float* mask, lo
     return launch_cluster(k_mlp_mse, s, y, t, mask, n, dy, loss);
 }
 
+template <typename T>
+static cudaError_t mlp_adam(float* master, void* lowp, const float* grad, float* m, float* v, int* step, long long n,
+                            float lr, float b1, float b2, float eps, cudaStream_t s) {
+    pdl(k_step_inc, 1, 1, 0, s)(step);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const long long g = (n + 255) / 256;
+    pdl(k_mlp_adam<T>, (unsigned)(g < (1 << 30) ? g : 1 << 30), 256, 0, s)(master, static_cast<T*>(lowp), grad, m, v,
+                                                                          step, n, lr, b1, b2, eps);
+    return cudaGetLastError();
+}
 cudaError_t launch_mlp_adam(float* master, void* lowp, int bf16, const float* grad, float* m, float* v, int* step,
                             long long n, float lr, float b1, float b2, float eps, cudaStream_t s) {
-    return bf16 ? launch_cluster(k_mlp_adam<__nv_bfloat16>, s, master, (__nv_bfloat16*)lowp, grad, m, v, step, n, lr,
-                                 b1, b2, eps)
-                : launch_cluster(k_mlp_adam<float>, s, master, (float*)lowp, grad, m, v, step, n, lr, b1, b2, eps);
+    return bf16 ? mlp_adam<__nv_bfloat16>(master, lowp, grad, m, v, step, n, lr, b1, b2, eps, s)
+                : mlp_adam<float>(master, lowp, grad, m, v, step, n, lr, b1, b2, eps, s);
 }
 
 cudaError_t launch_mlp_convert(const float* src, void* dst, int bf16, long long n, cudaStream_t s) {
