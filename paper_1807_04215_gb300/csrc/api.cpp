@@ -67,11 +67,14 @@ gridspt_status cuda_fail(cudaError_t e, const char* where) {
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+}  // namespace
+
 // Host-side fault injection for tests (no GPU fault is ever caused): the
 // environment variable GRIDSPT_FAULT_INJECT holds a comma-separated list of
 //   plan_alloc  - the plan's second device allocation reports out-of-memory
 //   launch      - every kernel launch reports a launch failure without launching
-bool fault_inject(const char* what) {
+//   cluster     - the device holds no cluster of more than one block
+bool gridspt::fault_inject(const char* what) {
     const char* v = std::getenv("GRIDSPT_FAULT_INJECT");
     if (!v || !*v) return false;
     const size_t n = std::strlen(what);
@@ -82,6 +85,8 @@ bool fault_inject(const char* what) {
     }
     return false;
 }
+
+namespace {
 
 // ------------------------------------------------------------- profiling
 enum ProfKind {

@@ -12,6 +12,9 @@ constexpr int kMaxOrder = 8;
 // exceeds this, and the allocation-free entry point's static scratch is sized by it.
 constexpr int kPowerMaxBlocks = 1216;
 
+// Whether the environment asks for a host-side failure (api.cpp).
+bool fault_inject(const char* what);
+
 // Bits of the plan's device status word (read and cleared by gridspt_check).
 constexpr int kStatusWaitSelftest = 2;  // the bounded-wait self-test's wait gave up
 constexpr int kStatusNonFinite = 4;     // an estimator produced a NaN or infinite result

@@ -21,6 +21,8 @@
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
+#include <atomic>
+
 #include "fft_core.cuh"
 #include "gridspt_internal.h"
 #include "pdl.cuh"
@@ -426,60 +428,86 @@ k_mlp_grad(const float* __restrict__ x, int row0, int row1, int I, int H, int O,
 }
 
 // Masked mean-squared error: dy = 2 mask (y - t) / sum(mask); loss = sum(mask (y - t)^2) / sum(mask).
-// One cluster of 16 blocks (the sums are needed by every element of dy, and one
-// block alone is bound by its own load latency): block sums by a fixed tree,
-// exchanged through distributed shared memory, added in block order.
-constexpr int kOptCluster = 16;
+__device__ __forceinline__ void mse_term(float y, float t, float mask, float& s, float& c) {
+    const float d = (y - t) * mask;
+    s = fmaf(d, d, s);
+    c += mask;
+}
+__device__ __forceinline__ float2 warp_sum2(float s, float c) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        s += __shfl_down_sync(0xffffffffu, s, off);
+        c += __shfl_down_sync(0xffffffffu, c, off);
+    }
+    return make_float2(s, c);
+}
+// Sum over 1024 threads by a fixed tree, in thread 0 (rs: 32 entries).
+__device__ __forceinline__ float2 block_sum2(float s, float c, float2* rs) {
+    float2 v = warp_sum2(s, c);
+    if ((threadIdx.x & 31) == 0) rs[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x < 32) v = warp_sum2(rs[threadIdx.x].x, rs[threadIdx.x].y);
+    return v;
+}
+// The sums are needed by every element of dy, and one block alone is bound by its own
+// load latency, so the blocks are one cluster: the elements form kOptParts parts
+// (1024 consecutive ones in turn), whose sums are exchanged through distributed
+// shared memory and added in order. A cluster of fewer blocks (most_cluster) takes
+// several parts a block; the sums are the same bits.
+constexpr int kOptParts = 16;
 __global__ void __launch_bounds__(1024)
 k_mlp_mse(const float* __restrict__ y, const float* __restrict__ t, const float* __restrict__ mask, long long n,
           float* __restrict__ dy, float* __restrict__ loss) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     __shared__ float2 rs[32];
-    __shared__ float2 tot;
-    const long long i0 = (long long)blockIdx.x * 1024 + threadIdx.x, step = 1024LL * kOptCluster;
-    float s = 0.f, c = 0.f;
+    __shared__ float2 tot[kOptParts];
+    const int blocks = gridDim.x;                                 // one cluster: 16, 8 or 1
+    const long long step = 1024LL * kOptParts;
+    for (int part = blockIdx.x; part < kOptParts; part += blocks) {
+        float s = 0.f, c = 0.f;
 #pragma unroll 4
-    for (long long i = i0; i < n; i += step) {
-        const float d = (y[i] - t[i]) * mask[i];
-        s = fmaf(d, d, s);
-        c += mask[i];
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        s += __shfl_down_sync(0xffffffffu, s, off);
-        c += __shfl_down_sync(0xffffffffu, c, off);
-    }
-    if ((threadIdx.x & 31) == 0) rs[threadIdx.x >> 5] = make_float2(s, c);
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        s = rs[threadIdx.x].x;
-        c = rs[threadIdx.x].y;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            s += __shfl_down_sync(0xffffffffu, s, off);
-            c += __shfl_down_sync(0xffffffffu, c, off);
-        }
-        if (threadIdx.x == 0) tot = make_float2(s, c);
+        for (long long i = part * 1024LL + threadIdx.x; i < n; i += step) mse_term(y[i], t[i], mask[i], s, c);
+        const float2 v = block_sum2(s, c, rs);
+        if (threadIdx.x == 0) tot[part] = v;
+        if (part + blocks < kOptParts) __syncthreads();           // rs is free for the next part
     }
     cl.sync();
-    if (threadIdx.x < 32) {                                       // block sums, added in block order
-        const float2 v = threadIdx.x < kOptCluster ? *cl.map_shared_rank(&tot, threadIdx.x) : make_float2(0.f, 0.f);
-        s = c = 0.f;
+    if (threadIdx.x < 32) {                                       // the parts, added in order
+        const float2 v = threadIdx.x < kOptParts ? *cl.map_shared_rank(&tot[threadIdx.x], threadIdx.x % blocks)
+                                                 : make_float2(0.f, 0.f);
+        float s = 0.f, c = 0.f;
 #pragma unroll
-        for (int b = 0; b < kOptCluster; ++b) {
-            s += __shfl_sync(0xffffffffu, v.x, b);
-            c += __shfl_sync(0xffffffffu, v.y, b);
+        for (int q = 0; q < kOptParts; ++q) {
+            s += __shfl_sync(0xffffffffu, v.x, q);
+            c += __shfl_sync(0xffffffffu, v.y, q);
         }
         if (threadIdx.x == 0) rs[0] = make_float2(s, c);
     }
     cl.sync();                                                    // rs[0] in place; no block leaves while its sums are read
-    s = rs[0].x;
-    c = rs[0].y;
-    const float cnt = c > 0.f ? c : 1.f;
+    const float s = rs[0].x, c = rs[0].y, cnt = c > 0.f ? c : 1.f;
+    for (int part = blockIdx.x; part < kOptParts; part += blocks)
 #pragma unroll 4
-    for (long long i = i0; i < n; i += step) dy[i] = 2.f * (y[i] - t[i]) * mask[i] / cnt;
-    if (i0 == 0 && loss) *loss = s / cnt;
+        for (long long i = part * 1024LL + threadIdx.x; i < n; i += step) dy[i] = 2.f * (y[i] - t[i]) * mask[i] / cnt;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && loss) *loss = s / cnt;
+}
+// n <= 1024: the one part that has elements, in one block without the cluster's barriers; same bits
+// (in a graph 1.9 .. 2.3 us, a cluster 3.3 .. 3.8).
+__global__ void __launch_bounds__(1024)
+k_mlp_mse_one(const float* __restrict__ y, const float* __restrict__ t, const float* __restrict__ mask, int n,
+              float* __restrict__ dy, float* __restrict__ loss) {
+    __shared__ float2 rs[32], tot;
+    const int i = threadIdx.x;
+    const bool on = i < n;
+    const float yi = on ? y[i] : 0.f, ti = on ? t[i] : 0.f, mi = on ? mask[i] : 0.f;
+    float s = 0.f, c = 0.f;
+    if (on) mse_term(yi, ti, mi, s, c);
+    const float2 v = block_sum2(s, c, rs);
+    if (i == 0) tot = v;
+    __syncthreads();
+    const float cnt = tot.y > 0.f ? tot.y : 1.f;
+    if (on) dy[i] = 2.f * (yi - ti) * mi / cnt;
+    if (i == 0 && loss) *loss = tot.x / cnt;
 }
 
 // Adam (Kingma & Ba 2015) on the FP32 master parameters; the step count lives
@@ -600,27 +628,65 @@ cudaError_t launch_mlp_backward(const float* x, int B, int I, int H, int O, cons
     return cudaSuccess;
 }
 
-// One launch of a single cluster of kOptCluster blocks of 1024 threads.
-template <typename... P, typename... A>
-static cudaError_t launch_cluster(void (*k)(P...), cudaStream_t s, A... a) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t c{};
-    c.gridDim = dim3(kOptCluster);
+// One cluster of `blocks` blocks of 1024 threads (one block: an ordinary launch).
+static void cluster_config(cudaLaunchConfig_t& c, cudaLaunchAttribute& at, int blocks, cudaStream_t s) {
+    c.gridDim = dim3(blocks);
     c.blockDim = dim3(1024);
     c.stream = s;
-    cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = kOptCluster;
+    at.val.clusterDim.x = blocks;
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     c.attrs = &at;
-    c.numAttrs = 1;
+    c.numAttrs = blocks > 1 ? 1 : 0;
+}
+template <typename... P, typename... A>
+static cudaError_t launch_cluster(void (*k)(P...), int blocks, cudaStream_t s, A... a) {
+    if (blocks > 1 && fault_inject("cluster")) return cudaErrorInvalidClusterSize;
+    cudaLaunchConfig_t c{};
+    cudaLaunchAttribute at{};
+    cluster_config(c, at, blocks, s);
     return cudaLaunchKernelEx(&c, k, static_cast<P>(a)...);
+}
+
+// Largest cluster of 1024-thread blocks, of 16 (beyond the portable 8), 8 and 1, that
+// the device can hold (an SM limit or a partition may leave less room): asked once per
+// device.
+template <typename... P>
+static cudaError_t most_cluster(void (*k)(P...), int* blocks) {
+    static std::atomic<int> known[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::atomic<int>& most = known[dev & 63];
+    *blocks = 1;
+    if (fault_inject("cluster")) return cudaSuccess;
+    if (!most.load()) {
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+        int got = 1;
+        for (int want : {8, 16}) {
+            cudaLaunchConfig_t c{};
+            cudaLaunchAttribute at{};
+            cluster_config(c, at, want, nullptr);
+            int fit = 0;
+            if (cudaOccupancyMaxActiveClusters(&fit, k, &c) == cudaSuccess && fit > 0) got = want;
+            else cudaGetLastError();                              // (a size the device refuses)
+        }
+        most.store(got);
+    }
+    *blocks = most.load();
+    return cudaSuccess;
 }
 
 cudaError_t launch_mlp_mse(const float* y, const float* t, const float* mask, long long n, float* dy, float* loss,
                            cudaStream_t s) {
-    return launch_cluster(k_mlp_mse, s, y, t, mask, n, dy, loss);
+    if (n <= 1024) {
+        k_mlp_mse_one<<<1, 1024, 0, s>>>(y, t, mask, (int)n, dy, loss);
+        return cudaGetLastError();
+    }
+    int blocks = 1;
+    const cudaError_t e = most_cluster(k_mlp_mse, &blocks);
+    return e != cudaSuccess ? e : launch_cluster(k_mlp_mse, blocks, s, y, t, mask, n, dy, loss);
 }
 
 template <typename T>

@@ -1,4 +1,5 @@
-"""Emulator kernels away from the usual training step: many parameters.
+"""Emulator kernels away from the usual training step: devices without room for a
+large cluster, many parameters.
 
 Cost is compared within one tree: Adam moves 26 bytes a parameter where the
 conversion moves 6, so 4.3 times its time; twice that is the bound (one cluster
@@ -36,6 +37,31 @@ def graph_time(f, calls=20, rounds=7):
         torch.cuda.synchronize()
         best = min(best, a.elapsed_time(b) / calls)
     return best
+
+
+@pytest.mark.parametrize("n", [1, 1000, 1024, 1025, 20000, 50001])
+def test_loss_and_update_without_room_for_a_cluster(n, monkeypatch):
+    """The injected device refuses every cluster of more than one block: the
+    loss, its gradient and the update are those of the device that has room."""
+    net = g.MLP(3, 128, 160, bf16=True, seed=1)
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    y, t = (torch.randn(n, generator=gen, device="cuda") for _ in range(2))
+    mask = (torch.rand(n, generator=gen, device="cuda") < 0.8).float()
+    net.grad.copy_(torch.randn(net.n, generator=gen, device="cuda"))
+    start = [b.clone() for b in (net.master, net.lowp, net.m, net.v, net.step)]
+
+    def run():
+        for b, s in zip((net.master, net.lowp, net.m, net.v, net.step), start):
+            b.copy_(s)
+        dy, loss = torch.empty_like(y), torch.zeros(1, device="cuda")
+        net.mse(y, t, mask, dy, loss)
+        net.adam(1e-3)
+        return [b.clone() for b in (dy, loss, net.master, net.lowp, net.m, net.v, net.step)]
+
+    ref = run()
+    monkeypatch.setenv("GRIDSPT_FAULT_INJECT", "cluster")
+    for a, b in zip(run(), ref, strict=True):
+        assert torch.equal(a, b)
 
 
 def test_update_of_many_parameters_takes_the_whole_gpu():
