@@ -21,6 +21,7 @@
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <atomic>
 
 #include "fft_core.cuh"
@@ -46,7 +47,7 @@ __device__ __forceinline__ float silu_grad(float z) {
 }
 
 constexpr int kGradRows = 16;          // rows of one FMA chain of the parameter gradients
-constexpr int kWBytes = 49152;         // one of the two weight buffers (32-bit 128 x 128 takes two chunks)
+constexpr int kWBytes = 49152;         // one of the two weight buffers at most (32-bit 128 x 128 takes two chunks)
 
 __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
@@ -65,20 +66,48 @@ __device__ __forceinline__ bool aligned_to(const void* p, int bytes) {
 
 // Copy rows x C elements (contiguous in global memory) to shared rows of `pitch`
 // elements: 16-byte or 4-byte asynchronous copies where addresses and lengths
-// allow, plain loads otherwise (an odd C of bfloat16).
+// allow, plain loads otherwise (an odd C of bfloat16), eight in flight a thread
+// (one at a time: 97 columns to 161, 25 of the 31 us of any batch up to 4096 rows).
+template <typename T>
+__device__ __noinline__ void stage_plain(T* dst, int pitch, const T* src, int rows, int C, long long src_pitch) {
+    const int nt = blockDim.x, dr = nt / C, dj = nt - dr * C;
+    int r = threadIdx.x / C, j = threadIdx.x - r * C;
+    while (r < rows) {
+        T v[8];
+        int to[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            to[u] = r < rows ? r * pitch + j : -1;
+            if (to[u] >= 0) v[u] = src[r * src_pitch + j];
+            r += dr;
+            j += dj;
+            if (j >= C) {
+                j -= C;
+                ++r;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (to[u] >= 0) dst[to[u]] = v[u];
+    }
+}
 template <typename T>
 __device__ void stage_rows(T* dst, int pitch, const T* src, int rows, int C, long long src_pitch) {
     constexpr int S = sizeof(T), V = 16 / S, W = 4 / S;
-    const int e = C % V == 0 && pitch % V == 0 && src_pitch % V == 0 && aligned_to(src, 16)   ? V
-                  : C % W == 0 && pitch % W == 0 && src_pitch % W == 0 && aligned_to(src, 4) ? W : 1;
-    const int nt = blockDim.x, q = C / e, dr = nt / q, dj = nt - dr * q;   // stepping (r, j): no division per copy
+    const bool vec = C % V == 0 && pitch % V == 0 && src_pitch % V == 0 && aligned_to(src, 16);
+    if constexpr (W > 1) {
+        if (!vec && !(C % W == 0 && pitch % W == 0 && src_pitch % W == 0 && aligned_to(src, 4))) {
+            stage_plain(dst, pitch, src, rows, C, src_pitch);
+            return;
+        }
+    }
+    const int e = vec ? V : W, nt = blockDim.x, q = C / e, dr = nt / q, dj = nt - dr * q;   // stepping (r, j): no division per copy
     int r = threadIdx.x / q, j = threadIdx.x - r * q;
     while (r < rows) {
         T* d = dst + r * pitch + j * e;
         const T* g = src + r * src_pitch + j * e;
-        if (e == V) cp_async16b(d, g);
-        else if (e == W && S * W == 4) cp_async4(d, g);
-        else *d = *g;
+        if (vec) cp_async16b(d, g);
+        else cp_async4(d, g);
         r += dr;
         j += dj;
         if (j >= q) {
@@ -113,6 +142,14 @@ template <> struct FwdTile<32> { static constexpr int RT = 4, CT = 2; };
 // neighbouring columns spread over the banks
 template <int R> __host__ __device__ constexpr int row_pitch() { return R == 2 ? 2 : R + 4; }
 __host__ __device__ constexpr int even(int n) { return (n + 1) & ~1; }
+// Weight chunks of the forward pass: k rows of K at once, elements of a row in shared memory.
+template <typename T>
+__host__ __device__ constexpr int fwd_chunk(int K, int C) {
+    const int fit = kWBytes / (even(C) * (int)sizeof(T));
+    return K < fit ? K : fit;
+}
+template <typename T>
+__host__ __device__ constexpr int fwd_pitch(int C) { return C % (16 / (int)sizeof(T)) == 0 ? C : even(C); }
 
 }  // namespace
 
@@ -123,14 +160,14 @@ __host__ __device__ constexpr int even(int n) { return (n + 1) & ~1; }
 template <typename T, int R>
 __global__ void __launch_bounds__(256 / FwdTile<R>::CT * (R / FwdTile<R>::RT))
 k_mlp_forward(const float* __restrict__ x, int B, int I, int H, int O, const T* __restrict__ theta,
-              float* __restrict__ y, float* __restrict__ act) {
-    pdl_enter();
+              float* __restrict__ y, float* __restrict__ act, int wbytes) {
+    pdl_wait();
     pdl_fresh(x);
     pdl_fresh(theta);
     constexpr int RT = FwdTile<R>::RT, CT = FwdTile<R>::CT, RP = row_pitch<R>(), G = R / RT;
     extern __shared__ __align__(16) char smraw[];
-    T* wb[2] = {reinterpret_cast<T*>(smraw), reinterpret_cast<T*>(smraw + kWBytes)};
-    float* hin = reinterpret_cast<float*>(smraw + 2 * kWBytes);    // [max(I, H)][RP], input of the layer
+    T* wb[2] = {reinterpret_cast<T*>(smraw), reinterpret_cast<T*>(smraw + wbytes)};
+    float* hin = reinterpret_cast<float*>(smraw + 2 * wbytes);     // [max(I, H)][RP], input of the layer
     float* hout = hin + (H > I ? H : I) * RP;                      // [H][RP]
     float* bs = hout + H * RP;                                     // b1[H], b2[H], b3[O]
     const T* W1 = theta;
@@ -141,16 +178,13 @@ k_mlp_forward(const float* __restrict__ x, int B, int I, int H, int O, const T* 
     auto layer_w = [&](int l) { return l == 0 ? W1 : l == 1 ? W2 : W3; };
     auto layer_c = [&](int l) { return l == 2 ? O : H; };
     auto layer_k = [&](int l) { return l == 0 ? I : H; };
-    auto chunk_k = [&](int l) {
-        const int fit = kWBytes / (even(layer_c(l)) * (int)sizeof(T));
-        return layer_k(l) < fit ? layer_k(l) : fit;
-    };
+    auto chunk_k = [&](int l) { return fwd_chunk<T>(layer_k(l), layer_c(l)); };
     const bool pairs = O % 2 == 0 && aligned_to(y, 8);
     int nl = 0, nk = 0, nbuf = 0;                                  // next chunk to issue
     auto issue = [&]() {
         if (nl < 3) {
             const int C = layer_c(nl), kc = chunk_k(nl), left = layer_k(nl) - nk, n = left < kc ? left : kc;
-            stage_rows(wb[nbuf], C % (16 / (int)sizeof(T)) == 0 ? C : even(C), layer_w(nl) + (long long)nk * C, n, C, C);
+            stage_rows(wb[nbuf], fwd_pitch<T>(C), layer_w(nl) + (long long)nk * C, n, C, C);
             nk += n;
             if (nk == layer_k(nl)) { nk = 0; ++nl; }
             nbuf ^= 1;
@@ -161,7 +195,7 @@ k_mlp_forward(const float* __restrict__ x, int B, int I, int H, int O, const T* 
     issue();
     for (int i = threadIdx.x; i < R * I; i += blockDim.x) {
         const int r = i / I, k = i - r * I;
-        hin[k * RP + r] = r0 + r < B ? x[(long long)(r0 + r) * I + k] : 0.f;
+        hin[k * RP + r] = r0 + r < B ? x[(long long)(r0 + r) * I + k] : 1.f;   // (0 / n: the division's slow path)
     }
     for (int i = threadIdx.x; i < 2 * H + O; i += blockDim.x)
         bs[i] = to_f<T>(i < H ? W1[(long long)I * H + i] : i < 2 * H ? W2[(long long)H * H + i - H]
@@ -170,7 +204,7 @@ k_mlp_forward(const float* __restrict__ x, int B, int I, int H, int O, const T* 
     int buf = 0;
     for (int l = 0; l < 3; ++l) {
         const int K = layer_k(l), C = layer_c(l), kc = chunk_k(l);
-        const int CP = C % (16 / (int)sizeof(T)) == 0 ? C : even(C);
+        const int CP = fwd_pitch<T>(C);
         const int nc = (C + CT - 1) / CT, ntask = nc * G;         // a warp's tasks: neighbouring columns, one row group
         const float* bias = bs + l * H;
         float2 acc[CT][RT / 2];
@@ -251,6 +285,64 @@ k_mlp_forward(const float* __restrict__ x, int B, int I, int H, int O, const T* 
     }
 }
 
+// The network for 32 rows per block, the weights read from global memory in the
+// chains (same chains): a block of 256 threads and a few kilobytes, so many share an SM.
+constexpr int kDenseRows = 32;
+template <typename T>
+__device__ void dense(const float* __restrict__ in, int K, const T* __restrict__ W, const T* __restrict__ b, int C,
+                      float* __restrict__ out) {
+    constexpr int RG = kDenseRows / 16;
+    for (int w = threadIdx.x; w < C * RG; w += blockDim.x) {       // one column of 16 rows
+        const int c = w % C, g = w / C;
+        float acc[16];
+        const float bc = to_f<T>(b[c]);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) acc[j] = bc;
+        for (int k = 0; k < K; ++k) {
+            const float wk = to_f<T>(W[(long long)k * C + c]);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) acc[j] = fmaf(in[(g * 16 + j) * K + k], wk, acc[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < 16; ++j) out[(g * 16 + j) * C + c] = acc[j];
+    }
+}
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_mlp_forward_rows(const float* __restrict__ x, int B, int I, int H, int O, const T* __restrict__ theta,
+                   float* __restrict__ y, float* __restrict__ act) {
+    constexpr int R = kDenseRows;
+    extern __shared__ float smf[];
+    float* in = smf;                                               // R x max(I, H)
+    float* out = in + R * (I > H ? I : H);                         // R x max(H, O)
+    const int r0 = blockIdx.x * R;
+    for (int i = threadIdx.x; i < R * I; i += blockDim.x)
+        in[i] = r0 + i / I < B ? x[(long long)r0 * I + i] : 0.f;
+    __syncthreads();
+    const T* W = theta;
+    for (int l = 0; l < 3; ++l) {
+        const int K = l ? H : I, C = l == 2 ? O : H;
+        dense<T>(in, K, W, W + (long long)K * C, C, out);
+        W += (long long)K * C + C;
+        __syncthreads();
+        for (int i = threadIdx.x; i < R * C; i += blockDim.x) {
+            const int r = i / C, c = i - r * C;
+            const bool on = r0 + r < B;
+            if (l == 2) {
+                if (on) y[(long long)r0 * O + i] = out[i];
+            } else {
+                const float z = out[i], a = round_t<T>(silu(z));
+                if (act && on) {
+                    act[(long long)(r0 + r) * 4 * H + 2 * l * H + c] = z;
+                    act[(long long)(r0 + r) * 4 * H + (2 * l + 1) * H + c] = a;
+                }
+                in[i] = a;
+            }
+        }
+        __syncthreads();
+    }
+}
+
 // Deltas of the hidden layers for R rows per block, d2 = (dy W3^T) silu'(z2) and
 // d1 = (d2 W2^T) silu'(z1), to [row][H] scratch. The weights' rows are staged
 // with an odd pitch in 4-byte words, so the threads of a warp (one hidden unit
@@ -260,7 +352,7 @@ template <typename T, int R>
 __global__ void __launch_bounds__(R == 2 ? 256 : 512)
 k_mlp_delta(int row0, int row1, int I, int H, int O, const T* __restrict__ theta, const float* __restrict__ act,
             const float* __restrict__ dy, float* __restrict__ d2, float* __restrict__ d1) {
-    pdl_enter();
+    pdl_wait();
     pdl_fresh(theta);
     pdl_fresh(act);
     pdl_fresh(dy);
@@ -363,7 +455,7 @@ __global__ void __launch_bounds__(kGT * kGT)
 k_mlp_grad(const float* __restrict__ x, int row0, int row1, int I, int H, int O, const float* __restrict__ act,
            const float* __restrict__ dy, const float* __restrict__ d2, const float* __restrict__ d1, int first,
            float* __restrict__ grad) {
-    pdl_enter();
+    pdl_wait();
     pdl_fresh(x);
     pdl_fresh(act);
     pdl_fresh(dy);
@@ -550,51 +642,83 @@ __global__ void k_convert(const float* __restrict__ src, T* __restrict__ dst, lo
 long long mlp_params(int I, int H, int O) { return (long long)I * H + H + (long long)H * H + H + (long long)H * O + O; }
 int mlp_bwd_blocks(int B) { return (B + kGradRows - 1) / kGradRows; }
 
-// The limit of the widest network (256) for every call: two threads with networks
+// All of a block's shared memory as the limit for every call: two threads with networks
 // of different widths must not lower it under one another's launch.
-template <int R, typename K>
+template <typename K>
 static cudaError_t smem_attr(K k) {
-    constexpr size_t most = 2 * (size_t)kWBytes + sizeof(float) * (size_t)(row_pitch<R>() * 2 * 256 + 3 * 256);
-    static_assert(most <= 232448, "rows of the widest network exceed shared memory");
-    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
 }
 
 // Rows per block: two while that gives at most two blocks per SM (304), eight
 // up to eight rows an SM block pair, then 32 (the weights are read once per block).
-static int fwd_rows(int B) { return B <= 608 ? 2 : B <= 2432 ? 8 : 32; }
+// 0: k_mlp_forward_rows, where a block's fixed cost counts for more than its loads do:
+// a few hidden units (3 -> 1 -> 1 -> 1, 4096 rows: 3.4 us against 4.8), and large batches
+// with a layer that is wide against the hidden ones (block of 640 threads for little work; 3 -> 16 ->
+// 16 -> 160, 65536 rows: 44 against 92; 64 hidden units: 136 / 144) or with odd rows,
+// which are copied by single elements (97 -> 161, 65536 rows: bf16 241 / 275, FP32 244 / 265).
+static int fwd_rows(int B, int H, int O, bool bf16) {
+    if (H <= 2 || (H <= 4 && B > 608) || (B >= 8192 && O >= 5 * H) ||
+        (B >= (bf16 ? 16384 : 32768) && H < 128 && (O & 1)))
+        return 0;
+    return B <= 608 ? 2 : B <= 2432 ? 8 : 32;
+}
 
+// The weight buffers hold the largest chunk, no more: blocks of a narrow network are
+// short chains, and several of them have to share an SM (3 -> 64 -> 64 -> 64, 65536 rows:
+// 102 us with two 48 KB buffers, 63 now; 3 -> 16 -> 16 -> 16 38 and 16).
 template <typename T, int R>
 static cudaError_t mlp_forward_r(const float* x, int B, int I, int H, int O, const void* theta, float* y, float* act,
                                  cudaStream_t s) {
-    const size_t sm = 2 * (size_t)kWBytes +
+    const int K[3] = {I, H, H}, C[3] = {H, H, O};
+    int wbytes = 0;
+    for (int l = 0; l < 3; ++l)
+        wbytes = std::max(wbytes, fwd_chunk<T>(K[l], C[l]) * fwd_pitch<T>(C[l]) * (int)sizeof(T));
+    wbytes = (wbytes + 15) & ~15;
+    const size_t sm = 2 * (size_t)wbytes +
                       sizeof(float) * ((size_t)row_pitch<R>() * ((H > I ? H : I) + H) + 2 * H + O);
-    cudaError_t e = smem_attr<R>(k_mlp_forward<T, R>);
+    cudaError_t e = smem_attr(k_mlp_forward<T, R>);
     if (e != cudaSuccess) return e;
     const int wide = H > O ? H : O, ct = FwdTile<R>::CT;
     int nt = (((wide + ct - 1) / ct) * (R / FwdTile<R>::RT) + 31) / 32 * 32;
-    if (nt < 256) nt = 256;                                        // the copies want threads too
+    const int copies = std::min(256, std::max(128, (wbytes / 16 + 31) / 32 * 32));   // the copies want threads too
+    if (nt < copies) nt = copies;
     pdl(k_mlp_forward<T, R>, (unsigned)((B + R - 1) / R), nt, sm, s)(x, B, I, H, O, static_cast<const T*>(theta),
-                                                                         y, act);
+                                                                         y, act, wbytes);
     return cudaGetLastError();
 }
 
+template <typename T>
+static cudaError_t mlp_forward_rows(const float* x, int B, int I, int H, int O, const void* theta, float* y, float* act,
+                                    cudaStream_t s) {
+    const size_t sm = sizeof(float) * kDenseRows * (size_t)((I > H ? I : H) + (H > O ? H : O));
+    cudaError_t e = smem_attr(k_mlp_forward_rows<T>);
+    if (e != cudaSuccess) return e;
+    k_mlp_forward_rows<T><<<(unsigned)((B + kDenseRows - 1) / kDenseRows), 256, sm, s>>>(
+        x, B, I, H, O, static_cast<const T*>(theta), y, act);
+    return cudaGetLastError();
+}
+
+template <typename T>
+static cudaError_t mlp_forward(const float* x, int B, int I, int H, int O, const void* theta, float* y, float* act,
+                               cudaStream_t s) {
+    switch (fwd_rows(B, H, O, sizeof(T) == 2)) {
+        case 2: return mlp_forward_r<T, 2>(x, B, I, H, O, theta, y, act, s);
+        case 8: return mlp_forward_r<T, 8>(x, B, I, H, O, theta, y, act, s);
+        case 32: return mlp_forward_r<T, 32>(x, B, I, H, O, theta, y, act, s);
+        default: return mlp_forward_rows<T>(x, B, I, H, O, theta, y, act, s);
+    }
+}
 cudaError_t launch_mlp_forward(const float* x, int B, int I, int H, int O, const void* theta, int bf16, float* y,
                                float* act, cudaStream_t s) {
-    const int r = fwd_rows(B);
-    if (bf16)
-        return r == 2   ? mlp_forward_r<__nv_bfloat16, 2>(x, B, I, H, O, theta, y, act, s)
-               : r == 8 ? mlp_forward_r<__nv_bfloat16, 8>(x, B, I, H, O, theta, y, act, s)
-                        : mlp_forward_r<__nv_bfloat16, 32>(x, B, I, H, O, theta, y, act, s);
-    return r == 2   ? mlp_forward_r<float, 2>(x, B, I, H, O, theta, y, act, s)
-           : r == 8 ? mlp_forward_r<float, 8>(x, B, I, H, O, theta, y, act, s)
-                    : mlp_forward_r<float, 32>(x, B, I, H, O, theta, y, act, s);
+    return bf16 ? mlp_forward<__nv_bfloat16>(x, B, I, H, O, theta, y, act, s)
+                : mlp_forward<float>(x, B, I, H, O, theta, y, act, s);
 }
 
 template <typename T, int R>
 static cudaError_t mlp_delta_r(int row0, int row1, int I, int H, int O, const void* theta, const float* act,
                                const float* dy, float* d2, float* d1, cudaStream_t s) {
     const size_t sm = 2 * (size_t)kWBytes + sizeof(float) * (size_t)row_pitch<R>() * ((O > H ? O : H) + H);
-    cudaError_t e = smem_attr<R>(k_mlp_delta<T, R>);
+    cudaError_t e = smem_attr(k_mlp_delta<T, R>);
     if (e != cudaSuccess) return e;
     const int need = (H * (R == 2 ? 1 : 2) + 31) / 32 * 32, nt = need < 256 ? 256 : need;
     pdl(k_mlp_delta<T, R>, (unsigned)((row1 - row0 + R - 1) / R), nt, sm, s)(

@@ -12,7 +12,8 @@ namespace gridspt {
 // they stay there. Fifth order, early / at the end / no programmatic launch, replayed
 // from a graph and launched on a stream: 96^3 481 / 365 / 360 and 491 / 374 / 406 us,
 // 64^3 201 / 147 / 150 and 212 / 156 / 197, 128^3 533 / 492 / 492; r2c at 96^3 18.4 /
-// 14.6 / 15.6. The power, shell-sum and emulator kernels let it in early (pdl_enter): their
+// 14.6 / 15.6. So do the emulator's layers (2400 rows of 3 -> 64 -> 64 -> 160, one call
+// after the other: 11.9 / 9.0 us). The power and shell-sum kernels let it in early (pdl_enter): their
 // successors are small (the final sums of a power call: 0.6 us of 7 later otherwise),
 // and so do z passes whose teams have one row group each (c2r at 48^3: 0.5 of 13 us).
 // A pointer that an earlier kernel writes through is not __restrict__ here, or passes

@@ -1,19 +1,23 @@
 """Emulator kernels away from the usual training step: devices without room for a
-large cluster, many parameters.
+large cluster, many parameters, narrow networks and odd rows in large batches.
 
-Cost is compared within one tree: Adam moves 26 bytes a parameter where the
-conversion moves 6, so 4.3 times its time; twice that is the bound (one cluster
-for every size took 20 times)."""
+Values: as in test_gpu_mlp_tiles. Cost is compared within one tree. Adam moves 26
+bytes a parameter where the conversion moves 6, so 4.3 times its time; twice that is
+the bound (one cluster for every size took 16 times). A narrow network's pass reads
+and writes little more than its output: bounds in copies of it (they took 20, 19 and 11, and 6, 8 and 5 now)."""
 import math
 
+import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():  # pragma: no cover
     pytest.skip("needs a CUDA GPU", allow_module_level=True)
 
+from oracle import mlp as om  # noqa: E402
 from paper_1807_04215_gb300 import _lib  # noqa: E402
 from paper_1807_04215_gb300 import gridspt as g  # noqa: E402
+from tests import inputs  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -82,3 +86,29 @@ def test_update_of_many_parameters_takes_the_whole_gpu():
 
     times = graph_time(adam), graph_time(convert)
     assert times[0] <= 9 * times[1], times
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("B,I,H,O", [(1, 3, 2, 1), (33, 1, 1, 256), (700, 3, 4, 4), (8200, 3, 16, 160), (8192, 8, 7, 35),
+                                     (16385, 2, 33, 33), (32769, 3, 97, 21)])
+def test_forward_of_narrow_and_odd_networks(bf16, B, I, H, O):
+    net = g.MLP(I, H, O, bf16=bf16, seed=B)
+    x = inputs.rng(B + H).standard_normal((B, I)).astype(np.float32)
+    y_ref, _ = om.forward(x.astype(np.float64), net.master.double().cpu().numpy(), H, O,
+                          om.bf16_round if bf16 else om.ident)
+    act = torch.full((B, 4 * H), float("nan"), device="cuda")
+    y = net.forward(torch.from_numpy(x).cuda(), act=act)
+    assert torch.equal(y, net.forward(torch.from_numpy(x).cuda()))
+    assert np.abs(y.double().cpu().numpy() - y_ref).max() <= (1e-2 if bf16 else 1e-5) * np.abs(y_ref).max()
+    z, a = act.view(B, 2, 2, H).unbind(2)
+    s = torch.nn.functional.silu(z)
+    assert torch.allclose(a, s.bfloat16().float() if bf16 else s, rtol=2.0 ** -7 if bf16 else 1e-6, atol=1e-30)
+
+
+@pytest.mark.parametrize("H,O,copies", [(1, 1, 12), (16, 16, 12), (16, 160, 8)])
+def test_narrow_forward_in_copies_of_its_output(H, O, copies):
+    B = 65536
+    net = g.MLP(3, H, O, bf16=True, seed=1)
+    x, y, z = torch.rand(B, 3, device="cuda"), torch.empty(B, O, device="cuda"), torch.empty(B, O, device="cuda")
+    times = graph_time(lambda: net.forward(x, y=y)), graph_time(lambda: z.copy_(y))
+    assert times[0] <= copies * times[1], times
