@@ -17,7 +17,9 @@
 // Measured (kernel times, bf16, 3 -> 128 -> 128 -> 160, against 8/16-block
 // kernels that read the weights from global memory in the chains):
 //   forward 256 rows 61 -> 9.5 us, 4096 rows 57 -> 21; backward 256 rows
-//   267 -> 19; mse 41 k elements 26 -> 7. Loss and Adam: beside their kernels.
+//   267 -> 19; mse 41 k elements 26 -> 7. One after the other in a graph: forward of 256
+//   rows 42.6 -> 7.6 us, 4096 rows 43 -> 18.2, backward 257 -> 12.6 and 501 -> 80. Where
+//   the row kernels of before are the faster ones (narrow networks): fwd_rows, mlp_backward.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
@@ -348,39 +350,41 @@ k_mlp_forward_rows(const float* __restrict__ x, int B, int I, int H, int O, cons
 // with an odd pitch in 4-byte words, so the threads of a warp (one hidden unit
 // each) read distinct banks; the chain of an output runs over the columns in
 // order, in chunks where a row block does not fit a buffer.
+// Columns per chunk: an even number, pitch = columns + one or two words (odd in words).
+template <typename T>
+__host__ __device__ constexpr int delta_cols(int all, int H) {
+    constexpr int W = 4 / (int)sizeof(T);
+    const int n = (kWBytes / (H * (int)sizeof(T)) - 2 * W - 2) & ~(2 * W - 1);
+    return all < n ? all : n;
+}
+template <typename T>
+__host__ __device__ constexpr int delta_pitch(int n) {             // elements; odd in 4-byte words
+    constexpr int W = 4 / (int)sizeof(T);
+    return (((n + W - 1) / W) | 1) * W;
+}
 template <typename T, int R>
 __global__ void __launch_bounds__(R == 2 ? 256 : 512)
-k_mlp_delta(int row0, int row1, int I, int H, int O, const T* __restrict__ theta, const float* __restrict__ act,
-            const float* __restrict__ dy, float* __restrict__ d2, float* __restrict__ d1) {
+k_mlp_delta(int B, int I, int H, int O, const T* __restrict__ theta, const float* __restrict__ act,
+            const float* __restrict__ dy, float* __restrict__ d2, float* __restrict__ d1, int wbytes, int early) {
     pdl_wait();
+    if (early) pdl_release();
     pdl_fresh(theta);
     pdl_fresh(act);
     pdl_fresh(dy);
     constexpr int RT = R == 2 ? 2 : 4, G = R / RT, RP = row_pitch<R>();
-    constexpr int W = 4 / (int)sizeof(T);
     extern __shared__ __align__(16) char smraw[];
-    T* wb[2] = {reinterpret_cast<T*>(smraw), reinterpret_cast<T*>(smraw + kWBytes)};
-    float* din = reinterpret_cast<float*>(smraw + 2 * kWBytes);    // [max(O, H)][RP]
+    T* wb[2] = {reinterpret_cast<T*>(smraw), reinterpret_cast<T*>(smraw + wbytes)};
+    float* din = reinterpret_cast<float*>(smraw + 2 * wbytes);     // [max(O, H)][RP]
     float* dmid = din + (O > H ? O : H) * RP;                      // [H][RP]
     const T* W2 = theta + (long long)I * H + H;
     const T* W3 = W2 + (long long)H * H + H;
-    const int r0 = row0 + blockIdx.x * R;
-    // columns per chunk: an even number, pitch = columns + one or two words (odd in words)
-    auto cols = [&](int l) {
-        int n = kWBytes / (H * (int)sizeof(T)) - 2 * W - 2;
-        n &= ~(2 * W - 1);
-        const int all = l ? H : O;
-        return all < n ? all : n;
-    };
-    auto pitch = [&](int n) {                                      // elements; odd in 4-byte words
-        const int words = (n + W - 1) / W;
-        return (words | 1) * W;
-    };
+    const int r0 = blockIdx.x * R;
+    auto cols = [&](int l) { return delta_cols<T>(l ? H : O, H); };
     int nl = 0, nk = 0, nbuf = 0;
     auto issue = [&]() {
         if (nl < 2) {
             const int all = nl ? H : O, kc = cols(nl), n = all - nk < kc ? all - nk : kc;
-            stage_rows(wb[nbuf], pitch(kc), (nl ? W2 : W3) + nk, H, n, (long long)all);
+            stage_rows(wb[nbuf], delta_pitch<T>(kc), (nl ? W2 : W3) + nk, H, n, (long long)all);
             nk += n;
             if (nk == all) { nk = 0; ++nl; }
             nbuf ^= 1;
@@ -391,11 +395,11 @@ k_mlp_delta(int row0, int row1, int I, int H, int O, const T* __restrict__ theta
     issue();
     for (int i = threadIdx.x; i < R * O; i += blockDim.x) {
         const int r = i / O, o = i - r * O;
-        din[o * RP + r] = r0 + r < row1 ? dy[(long long)(r0 + r) * O + o] : 0.f;
+        din[o * RP + r] = r0 + r < B ? dy[(long long)(r0 + r) * O + o] : 0.f;
     }
     int buf = 0;
     for (int l = 0; l < 2; ++l) {
-        const int K = l ? H : O, kc = cols(l), WP = pitch(kc);
+        const int K = l ? H : O, kc = cols(l), WP = delta_pitch<T>(kc);
         const int h = threadIdx.x % H, rt = (threadIdx.x / H) * RT;
         const bool on = threadIdx.x < H * G;
         float2 acc[RT / 2];
@@ -403,7 +407,7 @@ k_mlp_delta(int row0, int row1, int I, int H, int O, const T* __restrict__ theta
 #pragma unroll
         for (int j = 0; j < RT; ++j) {
             const int row = r0 + rt + j;
-            z[j] = on && row < row1 ? act[(long long)row * 4 * H + (l ? 0 : 2) * H + h] : 0.f;
+            z[j] = on && row < B ? act[(long long)row * 4 * H + (l ? 0 : 2) * H + h] : 0.f;
             if (j % 2 == 0) acc[j / 2] = make_float2(0.f, 0.f);
         }
         for (int k0 = 0; k0 < K; k0 += kc) {
@@ -435,9 +439,9 @@ k_mlp_delta(int row0, int row1, int I, int H, int O, const T* __restrict__ theta
                 const int row = r0 + rt + j;
                 const float s = (j & 1) ? acc[j / 2].y : acc[j / 2].x;
                 float d = 0.f;
-                if (row < row1) {
+                if (row < B) {
                     d = s * silu_grad(z[j]);
-                    (l ? d1 : d2)[(long long)(row - row0) * H + h] = d;
+                    (l ? d1 : d2)[(long long)row * H + h] = d;
                 }
                 if (l == 0) dmid[h * RP + rt + j] = d;
             }
@@ -448,20 +452,21 @@ k_mlp_delta(int row0, int row1, int I, int H, int O, const T* __restrict__ theta
 // Parameter gradients as 16 x 16 tiles of the three products (rows contracted):
 // W3: a2^T dy, W2: a1^T d2, W1: x^T d1; one element a thread, the next 64 rows
 // loaded into registers while the current ones are summed. Rows are summed in
-// chains of 16, the chains added in row order (on top of the values already in
-// grad unless `first`); tiles of the first k rows add the bias sums.
+// chains of 16, the chains added in row order; tiles of the first k rows add the bias
+// sums. blockIdx.y: a part of `per` rows, to grad + blockIdx.y * np.
 constexpr int kGT = 16, kGChunk = 64;
 __global__ void __launch_bounds__(kGT * kGT)
-k_mlp_grad(const float* __restrict__ x, int row0, int row1, int I, int H, int O, const float* __restrict__ act,
-           const float* __restrict__ dy, const float* __restrict__ d2, const float* __restrict__ d1, int first,
-           float* __restrict__ grad) {
+k_mlp_grad(const float* __restrict__ x, int B, int per, int I, int H, int O, const float* __restrict__ act,
+           const float* __restrict__ dy, const float* __restrict__ d2, const float* __restrict__ d1,
+           float* __restrict__ grad, long long np) {
     pdl_wait();
     pdl_fresh(x);
     pdl_fresh(act);
     pdl_fresh(dy);
     pdl_fresh(d2);
     pdl_fresh(d1);
-    pdl_fresh(grad);
+    const int row0 = blockIdx.y * per, rows = B - row0 < per ? B - row0 : per;
+    grad += blockIdx.y * np;
     constexpr int PER = kGChunk / kGT;
     __shared__ float ls[2][kGChunk][kGT], rs[2][kGChunk][kGT];
     const int th = (H + kGT - 1) / kGT, to = (O + kGT - 1) / kGT;
@@ -478,8 +483,7 @@ k_mlp_grad(const float* __restrict__ x, int row0, int row1, int I, int H, int O,
     const bool lok = lk < K, rok = n < C, live = k < K && rok, bias = kt == 0 && tk == 0 && rok;
     const int lp = layer == 0 ? I : 4 * H, rp = C;
     const float* left = (layer == 0 ? x : act + (layer == 1 ? H : 3 * H)) + (long long)(row0 + tk) * lp + lk;
-    const float* right = (layer == 2 ? dy + (long long)row0 * rp : layer == 1 ? d2 : d1) + (long long)tk * rp + n;
-    const int rows = row1 - row0;
+    const float* right = (layer == 2 ? dy : layer == 1 ? d2 : d1) + (long long)(row0 + tk) * rp + n;
     float lv[PER], rv[PER];
     auto load = [&](int c0) {
 #pragma unroll
@@ -489,7 +493,7 @@ k_mlp_grad(const float* __restrict__ x, int row0, int row1, int I, int H, int O,
             rv[q] = rok && r + tk < rows ? right[(long long)r * rp] : 0.f;
         }
     };
-    float tot = first || !live ? 0.f : gw[(long long)k * C + n], tb = first || !bias ? 0.f : gb[n];
+    float tot = 0.f, tb = 0.f;
     load(0);
     int buf = 0;
     for (int c0 = 0; c0 < rows; c0 += kGChunk) {
@@ -500,9 +504,7 @@ k_mlp_grad(const float* __restrict__ x, int row0, int row1, int I, int H, int O,
         }
         __syncthreads();                       // (the other buffer's readers passed the previous barrier's chunk)
         if (c0 + kGChunk < rows) load(c0 + kGChunk);
-#pragma unroll
-        for (int g = 0; g < kGChunk; g += kGradRows) {
-            if (c0 + g >= rows) break;
+        auto chain = [&](int g) {
             float s = 0.f, sb = 0.f;
 #pragma unroll
             for (int r = 0; r < kGradRows; ++r) {
@@ -512,11 +514,128 @@ k_mlp_grad(const float* __restrict__ x, int row0, int row1, int I, int H, int O,
             }
             tot += s;
             tb += sb;
+        };
+        if (c0 + kGChunk <= rows) {            // four chains side by side
+#pragma unroll
+            for (int g = 0; g < kGChunk; g += kGradRows) chain(g);
+        } else {
+#pragma unroll 1
+            for (int g = 0; c0 + g < rows; g += kGradRows) chain(g);
         }
         buf ^= 1;
     }
     if (live) gw[(long long)k * C + n] = tot;
     if (bias) gb[n] = tb;
+}
+
+// Backward of sum(dy * y) for kGradRows rows in one block, the deltas in shared memory:
+// the block's gradient (one chain, parameter layout) to part + blockIdx.x * np. For
+// networks whose workspace does not hold the deltas of the batch (I + H + O below about 30),
+// and for H, O <= 16 between 64 and 1024 rows (3 -> 16 -> 16 -> 16, 256 rows: 6.2 against 7.4 us).
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_mlp_backward_rows(const float* __restrict__ x, int B, int I, int H, int O, const T* __restrict__ theta,
+               const float* __restrict__ act, const float* __restrict__ dy, float* __restrict__ part) {
+    constexpr int R = kGradRows;
+    extern __shared__ float sm[];
+    float* xs = sm;              // R x I
+    float* z1 = xs + R * I;      // R x H
+    float* a1 = z1 + R * H;
+    float* z2 = a1 + R * H;
+    float* a2 = z2 + R * H;
+    float* d3 = a2 + R * H;      // R x O
+    float* d2 = d3 + R * O;      // R x H
+    float* d1 = d2 + R * H;      // R x H
+    const T* W2 = theta + I * H + H;
+    const T* W3 = W2 + H * H + H;
+    const long long np = (long long)I * H + H + (long long)H * H + H + (long long)H * O + O;
+    float* g = part + blockIdx.x * np;
+    float* gW1 = g;
+    float* gb1 = gW1 + I * H;
+    float* gW2 = gb1 + H;
+    float* gb2 = gW2 + H * H;
+    float* gW3 = gb2 + H;
+    float* gb3 = gW3 + H * O;
+    const int r0 = blockIdx.x * R;
+    for (int i = threadIdx.x; i < R * I; i += blockDim.x) {
+        const int r = i / I;
+        xs[i] = r0 + r < B ? x[(long long)(r0 + r) * I + (i % I)] : 0.f;
+    }
+    for (int i = threadIdx.x; i < R * H; i += blockDim.x) {
+        const int r = i / H, c = i % H;
+        const bool ok = r0 + r < B;
+        const float* ar = act + (long long)(r0 + r) * 4 * H;
+        z1[i] = ok ? ar[c] : 0.f;
+        a1[i] = ok ? ar[H + c] : 0.f;
+        z2[i] = ok ? ar[2 * H + c] : 0.f;
+        a2[i] = ok ? ar[3 * H + c] : 0.f;
+    }
+    for (int i = threadIdx.x; i < R * O; i += blockDim.x) {
+        const int r = i / O;
+        d3[i] = r0 + r < B ? dy[(long long)(r0 + r) * O + (i % O)] : 0.f;
+    }
+    __syncthreads();
+    // output layer
+    for (int w = threadIdx.x; w < H * O; w += blockDim.x) {
+        const int h = w / O, o = w % O;
+        float s = 0.f;
+        for (int r = 0; r < R; ++r) s = fmaf(a2[r * H + h], d3[r * O + o], s);
+        gW3[w] = s;
+    }
+    for (int o = threadIdx.x; o < O; o += blockDim.x) {
+        float s = 0.f;
+        for (int r = 0; r < R; ++r) s += d3[r * O + o];
+        gb3[o] = s;
+    }
+    for (int w = threadIdx.x; w < R * H; w += blockDim.x) {
+        const int r = w / H, h = w % H;
+        float s = 0.f;
+        for (int o = 0; o < O; ++o) s = fmaf(d3[r * O + o], to_f<T>(W3[(long long)h * O + o]), s);
+        d2[w] = s * silu_grad(z2[w]);
+    }
+    __syncthreads();
+    // second hidden layer
+    for (int w = threadIdx.x; w < H * H; w += blockDim.x) {
+        const int k = w / H, h = w % H;
+        float s = 0.f;
+        for (int r = 0; r < R; ++r) s = fmaf(a1[r * H + k], d2[r * H + h], s);
+        gW2[w] = s;
+    }
+    for (int h = threadIdx.x; h < H; h += blockDim.x) {
+        float s = 0.f;
+        for (int r = 0; r < R; ++r) s += d2[r * H + h];
+        gb2[h] = s;
+    }
+    for (int w = threadIdx.x; w < R * H; w += blockDim.x) {
+        const int r = w / H, k = w % H;
+        float s = 0.f;
+        for (int h = 0; h < H; ++h) s = fmaf(d2[r * H + h], to_f<T>(W2[(long long)k * H + h]), s);
+        d1[w] = s * silu_grad(z1[w]);
+    }
+    __syncthreads();
+    // first layer
+    for (int w = threadIdx.x; w < I * H; w += blockDim.x) {
+        const int i = w / H, h = w % H;
+        float s = 0.f;
+        for (int r = 0; r < R; ++r) s = fmaf(xs[r * I + i], d1[r * H + h], s);
+        gW1[w] = s;
+    }
+    for (int h = threadIdx.x; h < H; h += blockDim.x) {
+        float s = 0.f;
+        for (int r = 0; r < R; ++r) s += d1[r * H + h];
+        gb1[h] = s;
+    }
+}
+
+// grad[i] = sum (in order) of part[b][i]
+__global__ void k_mlp_reduce(const float* __restrict__ part, int nblocks, long long np, float* __restrict__ grad) {
+    pdl_wait();
+    pdl_fresh(part);
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < np; i += (long long)gridDim.x * blockDim.x) {
+        float s = 0.f;
+        for (int b = 0; b < nblocks; ++b) s += part[b * np + i];
+        grad[i] = s;
+    }
 }
 
 // Masked mean-squared error: dy = 2 mask (y - t) / sum(mask); loss = sum(mask (y - t)^2) / sum(mask).
@@ -715,41 +834,60 @@ cudaError_t launch_mlp_forward(const float* x, int B, int I, int H, int O, const
 }
 
 template <typename T, int R>
-static cudaError_t mlp_delta_r(int row0, int row1, int I, int H, int O, const void* theta, const float* act,
-                               const float* dy, float* d2, float* d1, cudaStream_t s) {
-    const size_t sm = 2 * (size_t)kWBytes + sizeof(float) * (size_t)row_pitch<R>() * ((O > H ? O : H) + H);
+static cudaError_t mlp_delta_r(int B, int I, int H, int O, const void* theta, const float* act, const float* dy,
+                               float* d2, float* d1, int next, cudaStream_t s) {
+    int wbytes = 0;
+    for (int all : {O, H})
+        wbytes = std::max(wbytes, H * delta_pitch<T>(delta_cols<T>(all, H)) * (int)sizeof(T));
+    wbytes = (wbytes + 15) & ~15;
+    const size_t sm = 2 * (size_t)wbytes + sizeof(float) * (size_t)row_pitch<R>() * ((O > H ? O : H) + H);
     cudaError_t e = smem_attr(k_mlp_delta<T, R>);
     if (e != cudaSuccess) return e;
-    const int need = (H * (R == 2 ? 1 : 2) + 31) / 32 * 32, nt = need < 256 ? 256 : need;
-    pdl(k_mlp_delta<T, R>, (unsigned)((row1 - row0 + R - 1) / R), nt, sm, s)(
-        row0, row1, I, H, O, static_cast<const T*>(theta), act, dy, d2, d1);
+    const int need = (H * (R == 2 ? 1 : 2) + 31) / 32 * 32, nt = need < 256 ? 256 : need, blocks = (B + R - 1) / R;
+    pdl(k_mlp_delta<T, R>, (unsigned)blocks, nt, sm, s)(B, I, H, O, static_cast<const T*>(theta), act, dy, d2, d1, wbytes,
+                                                        blocks + next <= 152);
     return cudaGetLastError();
 }
+// Parts of the rows that the gradient tiles are split into: one tile an SM, 128 rows a
+// part at least. Backward of 16384 rows (bf16), unsplit / split: 3 -> 16 -> 16 -> 16
+// (3 tiles) 223 / 31 us, 3 -> 16 -> 16 -> 160 (12) 244 / 59, 3 -> 64 -> 64 -> 160 (60) 261 / 160.
+static int grad_parts(int B, int tiles) { return std::max(1, std::min(152 / tiles, B / 128)); }
 
-// The deltas of as many rows as the workspace holds (all of them unless H + O
-// is below about 30), then the gradient tiles over those rows.
+// The deltas of all rows, then the gradient tiles over the rows: in parts of rows
+// where the tiles are fewer than the SMs, added in order.
+template <typename T>
+static cudaError_t mlp_backward(const float* x, int B, int I, int H, int O, const void* theta, const float* act,
+                                const float* dy, float* ws, float* grad, cudaStream_t s) {
+    const long long np = mlp_params(I, H, O), room = (long long)mlp_bwd_blocks(B) * np;
+    const int th = (H + kGT - 1) / kGT, to = (O + kGT - 1) / kGT, tiles = th * (to + th + 1);
+    int parts = grad_parts(B, tiles);
+    const int per = ((B + parts - 1) / parts + kGChunk - 1) / kGChunk * kGChunk;
+    parts = (B + per - 1) / per;
+    cudaError_t e;
+    if (2LL * H * B + (parts > 1 ? parts * np : 0) > room || (tiles <= 3 && B > 64 && B < 1024)) {
+        e = smem_attr(k_mlp_backward_rows<T>);
+        if (e != cudaSuccess) return e;
+        k_mlp_backward_rows<T><<<mlp_bwd_blocks(B), 256, sizeof(float) * (size_t)kGradRows * (I + 6 * H + O), s>>>(
+            x, B, I, H, O, static_cast<const T*>(theta), act, dy, ws);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        pdl(k_mlp_reduce, (unsigned)((np + 255) / 256), 256, 0, s)(ws, mlp_bwd_blocks(B), np, grad);
+        return cudaGetLastError();
+    }
+    float* d2 = ws;
+    float* d1 = d2 + (long long)B * H;
+    float* part = d1 + (long long)B * H;
+    e = B <= 608 ? mlp_delta_r<T, 2>(B, I, H, O, theta, act, dy, d2, d1, tiles * parts, s)
+                 : mlp_delta_r<T, 8>(B, I, H, O, theta, act, dy, d2, d1, tiles * parts, s);
+    if (e != cudaSuccess) return e;
+    pdl(k_mlp_grad, dim3(tiles, parts), kGT * kGT, 0, s)(x, B, per, I, H, O, act, dy, d2, d1, parts > 1 ? part : grad, np);
+    if ((e = cudaGetLastError()) != cudaSuccess || parts == 1) return e;
+    pdl(k_mlp_reduce, (unsigned)((np + 255) / 256), 256, 0, s)(part, parts, np, grad);
+    return cudaGetLastError();
+}
 cudaError_t launch_mlp_backward(const float* x, int B, int I, int H, int O, const void* theta, int bf16,
                                 const float* act, const float* dy, float* part, float* grad, cudaStream_t s) {
-    const long long np = mlp_params(I, H, O), cap = (long long)mlp_bwd_blocks(B) * np / (2 * H);   // rows; np >= 5 H
-    long long rows = cap < B ? cap : B;
-    if (rows < B && rows >= kGradRows) rows -= rows % kGradRows;
-    float* d2 = part;
-    float* d1 = part + rows * H;
-    const int th = (H + kGT - 1) / kGT, to = (O + kGT - 1) / kGT;
-    cudaError_t e;
-    for (long long r0 = 0; r0 < B; r0 += rows) {
-        const int a = (int)r0, b = (int)(r0 + rows < B ? r0 + rows : B);
-        if (b - a <= 608)
-            e = bf16 ? mlp_delta_r<__nv_bfloat16, 2>(a, b, I, H, O, theta, act, dy, d2, d1, s)
-                     : mlp_delta_r<float, 2>(a, b, I, H, O, theta, act, dy, d2, d1, s);
-        else
-            e = bf16 ? mlp_delta_r<__nv_bfloat16, 8>(a, b, I, H, O, theta, act, dy, d2, d1, s)
-                     : mlp_delta_r<float, 8>(a, b, I, H, O, theta, act, dy, d2, d1, s);
-        if (e != cudaSuccess) return e;
-        pdl(k_mlp_grad, (unsigned)(th * (to + th + 1)), kGT * kGT, 0, s)(x, a, b, I, H, O, act, dy, d2, d1, r0 == 0, grad);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    return bf16 ? mlp_backward<__nv_bfloat16>(x, B, I, H, O, theta, act, dy, part, grad, s)
+                : mlp_backward<float>(x, B, I, H, O, theta, act, dy, part, grad, s);
 }
 
 // One cluster of `blocks` blocks of 1024 threads (one block: an ordinary launch).

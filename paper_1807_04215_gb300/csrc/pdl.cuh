@@ -12,10 +12,12 @@ namespace gridspt {
 // they stay there. Fifth order, early / at the end / no programmatic launch, replayed
 // from a graph and launched on a stream: 96^3 481 / 365 / 360 and 491 / 374 / 406 us,
 // 64^3 201 / 147 / 150 and 212 / 156 / 197, 128^3 533 / 492 / 492; r2c at 96^3 18.4 /
-// 14.6 / 15.6. So do the emulator's layers (2400 rows of 3 -> 64 -> 64 -> 160, one call
-// after the other: 11.9 / 9.0 us). The power and shell-sum kernels let it in early (pdl_enter): their
-// successors are small (the final sums of a power call: 0.6 us of 7 later otherwise),
-// and so do z passes whose teams have one row group each (c2r at 48^3: 0.5 of 13 us).
+// 14.6 / 15.6. So do the emulator's layers (2400 rows of 3 -> 64 -> 64 -> 160, one call after the
+// other: 11.9 / 9.0 us; backward of 1024 rows of 3 -> 128 -> 128 -> 160: 44 / 25), except a delta
+// kernel that leaves an SM to each block of its successor. The power and shell-sum kernels
+// let it in early (pdl_enter): their successors are small (the final sums of a power call:
+// 0.6 us of 7 later otherwise), and so do z passes whose teams have one row group each
+// (c2r at 48^3: 0.5 of 13 us).
 // A pointer that an earlier kernel writes through is not __restrict__ here, or passes
 // pdl_fresh(): the compiler may move loads through a restrict parameter over the wait.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -112,3 +112,43 @@ def test_narrow_forward_in_copies_of_its_output(H, O, copies):
     x, y, z = torch.rand(B, 3, device="cuda"), torch.empty(B, O, device="cuda"), torch.empty(B, O, device="cuda")
     times = graph_time(lambda: net.forward(x, y=y)), graph_time(lambda: z.copy_(y))
     assert times[0] <= copies * times[1], times
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("B,I,H,O", [(16, 3, 1, 1), (65, 3, 16, 16), (64, 3, 16, 16), (1023, 2, 16, 9), (1024, 3, 16, 16),
+                                     (4099, 3, 8, 100), (129, 3, 17, 1), (9000, 8, 64, 33), (2049, 3, 4, 4)])
+def test_backward_in_row_parts_and_of_narrow_networks(bf16, B, I, H, O):
+    """Sums over B rows in parts: against FP64, (B / 16 + 16) 2^-24 of the sum of
+    magnitudes at worst, below 1e-5 of the largest gradient for these inputs with the
+    factor that random signs leave (sqrt)."""
+    net = g.MLP(I, H, O, bf16=bf16, seed=B)
+    r = inputs.rng(B + H)
+    x, dy = (r.standard_normal((B, k)).astype(np.float32) for k in (I, O))
+    rnd = om.bf16_round if bf16 else om.ident
+    theta = net.master.double().cpu().numpy()
+    _, acts = om.forward(x.astype(np.float64), theta, H, O, rnd)
+    act = torch.empty(B, 4 * H, device="cuda")
+    xd, dyd = torch.from_numpy(x).cuda(), torch.from_numpy(dy).cuda()
+    net.forward(xd, act=act)
+    ws = torch.full((net.ws_bytes(B) + 4096,), 255, dtype=torch.uint8, device="cuda")
+    net.grad.fill_(float("nan"))
+    grad = net.backward(xd, act, dyd, ws[:net.ws_bytes(B)]).clone()
+    assert bool((ws[net.ws_bytes(B):] == 255).all())
+    assert torch.equal(grad, net.backward(xd, act, dyd, ws[:net.ws_bytes(B)]))
+    ref = om.backward(x.astype(np.float64), theta, H, O, acts, dy.astype(np.float64), rnd)
+    assert np.abs(grad.double().cpu().numpy() - ref).max() <= (1e-2 if bf16 else 1e-5) * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("H,O", [(16, 16), (16, 160)])
+def test_narrow_backward_is_spread_over_the_rows(H, O):
+    """A batch four times the size of one that leaves most of the GPU idle takes less than
+    three times as long (one block a tile whatever the batch: 3.2 to 3.4)."""
+    times = []
+    for B in (1024, 4096):
+        net = g.MLP(3, H, O, bf16=True, seed=1)
+        x, dy = torch.rand(B, 3, device="cuda"), torch.randn(B, O, device="cuda")
+        act = torch.empty(B, 4 * H, device="cuda")
+        net.forward(x, act=act)
+        ws = torch.empty(net.ws_bytes(B), dtype=torch.uint8, device="cuda")
+        times.append(graph_time(lambda: net.backward(x, act, dy, ws)))
+    assert times[1] <= 3 * times[0], times
