@@ -217,7 +217,7 @@ template <int N, int TZ, int AXIS, bool FIN>
 __global__ void __launch_bounds__(TZ * Cfg<N>::PC)
 k_colpass(float2* data, long long fstride, const float2* __restrict__ twg,
           long long s2_nl, int zero_k0, int band) {
-    pdl_wait();
+    pdl_pass<N>();
     extern __shared__ float2 sm[];
     colpass_body<N, TZ, AXIS, FIN>(data, fstride, twg, s2_nl, zero_k0, band, blockIdx.x, blockIdx.y, blockIdx.z,
                                    sm);
@@ -227,7 +227,7 @@ k_colpass(float2* data, long long fstride, const float2* __restrict__ twg,
 template <int N, int TZ>
 __global__ void __launch_bounds__(TZ * Cfg<N>::PZ)
 k_zr2c(const float2* in, float2* out, long long fstride, const float2* __restrict__ twg, float scale, int band) {
-    pdl_wait();
+    pdl_pass<N>();
     constexpr int M = N / 2, E = fft_elems(M), P = M / E, PITCH = Cfg<N>::PITCH;
     extern __shared__ float2 sm[];
     float2* tw = sm;
@@ -451,7 +451,7 @@ __device__ __forceinline__ void xexp_body(const XExpArgs& args, const float2* __
 template <int N, int TZ, int MODE>
 __global__ void __launch_bounds__(TZ * Cfg<N>::PC, xexp_min_blocks<N, TZ, MODE>())
 k_xexp(const __grid_constant__ XExpArgs args, const float2* __restrict__ twg, float kF, float inv_kF2) {
-    pdl_wait();
+    pdl_pass<N>();
     extern __shared__ __align__(16) float2 sm[];
     xexp_body<N, TZ, MODE>(args, twg, kF, inv_kF2, blockIdx.x, blockIdx.y, sm);
 }
@@ -525,7 +525,7 @@ __device__ __forceinline__ void yexp_body(const YZExpArgs& args, const float2* _
 template <int N, int TZ>
 __global__ void __launch_bounds__(TZ * Cfg<N>::PC, col_min_blocks<N, TZ>())
 k_yexp(const __grid_constant__ YZExpArgs args, const float2* __restrict__ twg, float kF) {
-    pdl_wait();
+    pdl_pass<N>();
     extern __shared__ __align__(16) float2 sm[];
     yexp_body<N, TZ>(args, twg, kF, blockIdx.x, blockIdx.y, sm);
 }
@@ -765,7 +765,7 @@ k_ycol(const __grid_constant__ YZExpArgs args, const float2* __restrict__ twg, f
 template <int N, int TZ, bool PREFETCH>
 __global__ void __launch_bounds__(TZ * Cfg<N>::PZ, (TZ * Cfg<N>::PZ <= 512) ? 2 : 1)
 k_zexp(YZExpArgs args, const float2* __restrict__ twg, float kF) {
-    pdl_wait();
+    pdl_pass<N>();
     const int B = args.band;                     // > 0: inputs nonzero only at kz < B
     constexpr int M = N / 2, E = fft_elems(M), P = M / E, PITCH = Cfg<N>::PITCH, NT = TZ * P;
     extern __shared__ float2 sm[];
@@ -850,7 +850,7 @@ k_zexp(YZExpArgs args, const float2* __restrict__ twg, float kF) {
 template <int N, int TZ, int NT>
 __global__ void __launch_bounds__(TZ * Cfg<N>::PZ, 1)
 k_zexp_pairs(ZPairArgs args, const float2* __restrict__ twg, float kF) {
-    pdl_wait();
+    pdl_pass<N>();
     constexpr int M = N / 2, E = fft_elems(M), P = M / E, PITCH = Cfg<N>::PITCH, NTH = TZ * P;
     constexpr int MAXP = kMaxPartners;         // partner fields of one output over all targets
     extern __shared__ float2 sm[];
