@@ -1309,7 +1309,7 @@ k_zrow(const __grid_constant__ ZPairArgs args, const float2* __restrict__ twg, f
     pdl_wait();
     extern __shared__ __align__(16) float2 sm[];
     const int teams = blockDim.x / RowCfg<N>::TL;
-    if ((long long)gridDim.x * teams * RowCfg<N>::RW >= (long long)N * N) pdl_release();   // no second row group
+    if constexpr (N <= 48) pdl_release();
     zrow_body<N, NT, BAND>(args, twg, kF, (long long)blockIdx.x * teams, (long long)gridDim.x * teams, sm, false,
                            maxp);
 }

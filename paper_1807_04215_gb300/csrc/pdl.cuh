@@ -16,9 +16,9 @@ namespace gridspt {
 // other: 11.9 / 9.0 us; backward of 1024 rows of 3 -> 128 -> 128 -> 160: 44 / 25), except a delta
 // kernel that leaves an SM to each block of its successor. The power and shell-sum kernels
 // let it in early (pdl_enter): their successors are small (the final sums of a power call:
-// 0.6 us of 7 later otherwise), so do z passes whose teams have one row group each (c2r
-// at 48^3: 0.5 of 13 us) and the passes of grids up to 24^3, which leave most SMs empty
-// (divergence form, eighth order: 8^3 98 / 112 us, 24^3 223 / 235; at 48^3 272 / 250).
+// 0.6 us of 7 later otherwise), so do the passes of grids up to 24^3, which leave most SMs
+// empty (divergence form, eighth order: 8^3 98 / 112 us, 24^3 223 / 235; at 48^3 272 / 250),
+// and warp-row z passes up to 48^3 (c2r 12.4 / 12.9; fifth order at 96^3 375 / 369).
 // A pointer that an earlier kernel writes through is not __restrict__ here, or passes
 // pdl_fresh(): the compiler may move loads through a restrict parameter over the wait.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
