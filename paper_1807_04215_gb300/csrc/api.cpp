@@ -1365,8 +1365,10 @@ gridspt_status gridspt_autotune(gridspt_plan p, void* scratch, size_t scratch_by
     // per pass, on scratch fields: the x and y expansions of orders 1 .. n_max - 1
     // as a run from delta_1 launches them (order 1 and the band-limited orders
     // move only their band columns, so the timing weighs the variants as the
-    // run does); the z expansion of an order >= 2 (12 -> 17, store-only and
-    // fused with pair products); the forward passes of delta_n, theta_n
+    // run does); their z expansions fused with pair products and the finished rows'
+    // forward z pass (timed store-only and without that pass, 96^3 was tuned to tiles:
+    // fifth order 404 us against 365), or the divergence form's four fields; the
+    // forward passes of delta_n, theta_n
     auto run = [&](const Geo& g, int pass) -> cudaError_t {
         XExpArgs xa{};
         YZExpArgs ya{}, za{};
@@ -1409,25 +1411,48 @@ gridspt_status gridspt_autotune(gridspt_plan p, void* scratch, size_t scratch_by
                 za.in_stride = F;
                 za.out = f0 + 12 * F;
                 za.out_stride = F;
-                cudaError_t ez = launch_zexp(g, za, s);
-                if (ez != cudaSuccess) return ez;
-                // and the form fused with pair products: one target, order-1
-                // partners in fields 0..12, partial sums in from fields 13, 14,
-                // outputs to fields 15, 16 (nothing written is read in the launch)
-                ZPairArgs pa{};
-                pa.z = za;
-                pa.cells = field_floats(p);
-                pa.ntargets = 1;
-                PairTarget& T = pa.t[0];
-                T.partner = reinterpret_cast<const float*>(f0);
-                pair_table(1, T);
-                T.acc_in_a = reinterpret_cast<const float*>(f0 + 13 * F);
-                T.acc_in_b = reinterpret_cast<const float*>(f0 + 14 * F);
-                T.out_a = reinterpret_cast<float*>(f0 + 15 * F);
-                T.out_b = reinterpret_cast<float*>(f0 + 16 * F);
-                T.ca0 = T.cb1 = 1.f;
-                T.ca1 = T.cb0 = 0.f;
-                return launch_zexp_pairs(g, pa, s);
+                if (p->d.form == GRIDSPT_FORM_DIVERGENCE) {
+                    za.nout = 4;
+                    return launch_zexp(g, za, s);
+                }
+                // orders 1 .. n_max - 1 with their bands and targets (real fields are not
+                // stored): partners of orders 1 and 2 in fields 0..16, finished rows to
+                // fields 17, 18, partial sums from 21..24 to 19, 20 (nothing written is
+                // read in the launch); the finished rows forward along z, in the same
+                // launch or after it
+                for (int m = 1; m < std::max(2, p->d.n_max); ++m) {
+                    XExpArgs xm{};
+                    YZExpArgs ym{};
+                    ZPairArgs pa{};
+                    expansion_codes(m, xm, ym, pa.z);
+                    double fx = 1.0, fyi = 1.0, fyo = 1.0;
+                    if (m == 1) order1_band(p, xm, ym, pa.z, &fx, &fyi, &fyo);
+                    else if (const int band = order_band(p, m, 2)) set_band(p, band, xm, ym, pa.z, &fx, &fyi, &fyo);
+                    pa.z.in = f0;
+                    pa.z.in_stride = F;
+                    pa.cells = field_floats(p);
+                    pa.ntargets = m > 2 && m + 2 <= p->d.n_max ? 2 : 1;
+                    const int band = forward_band(p, m + 1, 2);
+                    for (int t = 0; t < pa.ntargets; ++t) {
+                        PairTarget& T = pa.t[t];
+                        T.partner = reinterpret_cast<const float*>(f0);
+                        pair_table(1 + t, T);
+                        if (m > 1) {
+                            T.acc_in_a = reinterpret_cast<const float*>(f0 + (21 + 2 * t) * F);
+                            T.acc_in_b = reinterpret_cast<const float*>(f0 + (22 + 2 * t) * F);
+                        }
+                        T.out_a = reinterpret_cast<float*>(f0 + (17 + 2 * t) * F);
+                        T.out_b = reinterpret_cast<float*>(f0 + (18 + 2 * t) * F);
+                        T.ca0 = T.cb1 = 1.f;
+                        T.r2c = t == 0 && zexp_pairs_r2c(g) ? 1 : 0;
+                        T.r2c_band = T.r2c ? band : 0;
+                    }
+                    cudaError_t ez = launch_zexp_pairs(g, pa, s);
+                    if (ez == cudaSuccess && !pa.t[0].r2c)
+                        ez = launch_zr2c(g, f0 + 17 * F, f0 + 17 * F, F, 2, 1.0f, band, s);
+                    if (ez != cudaSuccess) return ez;
+                }
+                return cudaSuccess;
             }
             default: return launch_zr2c(g, f0, f0, F, 2, 1.0f, 0, s);
         }
@@ -1436,13 +1461,14 @@ gridspt_status gridspt_autotune(gridspt_plan p, void* scratch, size_t scratch_by
     for (int pass = 0; pass < TV_COUNT && e == cudaSuccess; ++pass) {
         float tbest = 0.f;
         best[pass] = 0;
+        const int reps = pass == TV_ZEXP && p->geo.N >= 128 ? 1 : 3;   // (all orders: long enough)
         for (int v = 0; v < kTuneVariants[pass] && e == cudaSuccess; ++v) {
             if (tune_variant(p->geo.N, pass, v) != v) continue;   // runs as another one
             Geo g = p->geo;
             g.var[pass] = v;
             e = run(g, pass);   // warm-up
             if (e == cudaSuccess) e = cudaEventRecord(a, s);
-            for (int r = 0; r < 3 && e == cudaSuccess; ++r) e = run(g, pass);
+            for (int r = 0; r < reps && e == cudaSuccess; ++r) e = run(g, pass);
             if (e == cudaSuccess) e = cudaEventRecord(b, s);
             if (e == cudaSuccess) e = cudaEventSynchronize(b);
             float t = 0.f;
