@@ -139,8 +139,8 @@ gridspt_status gridspt_linear_amplitude(const gridspt_cosmo* cosmo, double* ampl
  * fields; u = (r + 1/2) 2^-32, g1 + i g2 = sqrt(-2 ln u1) e^{2 pi i u2},
  * delta(c) = sqrt(P(|k|) / L^3) (g1 + i g2) / sqrt(2), delta(-c) = conj.
  * Zero: k = 0, Nyquist modes and |s|^2 > (kcut_lin / k_F)^2. Formed in pairs of
- * FP32 numbers (relative error 2e-13; the amplitudes' table and sigma_8
- * in FP64, on the device), stored as FP32. */
+ * FP32 numbers (error below 1e-12 of the modulus; the amplitudes' table and sigma_8
+ * in FP64, on the device), stored as FP32; an amplitude beyond FP32 gives infinities. */
 gridspt_status gridspt_make_linear_field(gridspt_plan plan, const gridspt_cosmo* cosmo,
                                          const uint64_t* seeds, void* delta1_k,
                                          gridspt_stream stream);

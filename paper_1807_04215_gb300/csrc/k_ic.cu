@@ -25,9 +25,9 @@
 // by table and short polynomial (P. T. P. Tang's table-driven scheme, ACM TOMS 16,
 // 1990: ln u = k ln 2 - ln r + log1p(h r - 1), h r - 1 exact in integers; the
 // angle-addition theorem; one Newton step for the square root). Their relative
-// error is below 1e-12, the FP32 result's rounding 6e-8. Rows are visited plane
-// by plane in a scattered order of kx, so planes with modes inside the cut run
-// beside planes that are only written. 512^3: 345 us a realisation with FP64 log,
+// error is below 1e-12 of the modulus (4e-13: the tail of log1p in FP32), the FP32
+// result's rounding 6e-8. Rows are visited plane by plane in a scattered order of kx,
+// so planes with modes inside the cut run beside planes that are only written. 512^3: 345 us a realisation with FP64 log,
 // sincospi and a 64-bit division per element, 250 with FP64 tables, 93 now.
 // The amplitude A is the Simpson sum of gridspt_linear_amplitude, formed on the
 // device in FP64 (65537 integrands: 4.6 ms per call on the host, 32 us here).
@@ -81,6 +81,10 @@ __device__ __forceinline__ float2 renorm(float h, float l) {          // |l| sma
     const float s = __fadd_rn(h, l);
     return make_float2(s, __fsub_rn(l, __fsub_rn(s, h)));
 }
+
+// A pair rounded to FP32. An infinite value's error is infinite or not a number: it is
+// clamped (a finite one is below 2^-24 of FP32's largest number), so the value stays.
+__device__ __forceinline__ float pair_value(float2 p) { return __fadd_rn(p.x, fminf(fmaxf(p.y, -3e31f), 3e31f)); }
 
 // (g1, g2) = sqrt(-2 ln u1) (cos 2 pi u2, sin 2 pi u2), u = (r + 1/2) 2^-32, as pairs.
 // logt[i - 128] = -ln(r_i / 512) with r_i = 131072 / i rounded to an integer;
@@ -163,7 +167,8 @@ k_ic(IcArgs a, int N, int M, int step) {
                     float2 g1, g2;
                     box_muller(r.x, r.y, logt, cst, g1, g2);
                     const float2 sd = a.table[s2], re = pair_mul(sd, g1), im = pair_mul(sd, g2);
-                    v = make_float2(__fadd_rn(re.x, re.y), canon ? __fadd_rn(im.x, im.y) : -__fadd_rn(im.x, im.y));
+                    const float a1 = pair_value(re), a2 = pair_value(im);
+                    v = make_float2(a1, canon ? a2 : -a2);
                 }
                 out[kz] = v;
             }
