@@ -447,6 +447,19 @@ gridspt_status gridspt_check(gridspt_plan plan, gridspt_stream stream);
  * the next gridspt_check reports GRIDSPT_E_TIMEOUT. Nothing faults or hangs. */
 gridspt_status gridspt_selftest_bounded_wait(gridspt_plan plan, gridspt_stream stream);
 
+/* Kernel self-tests on device buffers (16-byte aligned).
+ * Columns: in, out float2[2][N][width], N the plan's grid (128, 256, 512, 1024),
+ *   width 16, or 32 up to N = 256: the length-N transforms of direction +1
+ *   (backward) or -1 (forward) along the second index, unnormalised, by the
+ *   one-exchange transform or the one with an exchange per stage. The results
+ *   are equal.
+ * Normals: words uint32[n][2], out double[n][2]: g1, g2 of gridspt_make_linear_field
+ *   for r = words[i], before the rounding to FP32. */
+gridspt_status gridspt_selftest_columns(gridspt_plan plan, int32_t width, int32_t direction, int32_t one_exchange,
+                                        const void* in, void* out, gridspt_stream stream);
+gridspt_status gridspt_selftest_normals(gridspt_plan plan, const void* words, int32_t n, double* out,
+                                        gridspt_stream stream);
+
 /* Message for the last non-OK status returned on this thread ("" if none). */
 const char* gridspt_last_error(void);
 

@@ -1513,6 +1513,32 @@ gridspt_status gridspt_selftest_bounded_wait(gridspt_plan p, gridspt_stream stre
     return GRIDSPT_OK;
 }
 
+gridspt_status gridspt_selftest_columns(gridspt_plan p, int32_t width, int32_t direction, int32_t one_exchange,
+                                        const void* in, void* out, gridspt_stream stream) {
+    g_err[0] = 0;
+    if (check_plan(p)) return GRIDSPT_E_INVALID;
+    const int N = p->geo.N;
+    if (!in || !out || !aligned16(in) || !aligned16(out)) return fail(GRIDSPT_E_INVALID, "columns NULL or not 16-byte aligned");
+    if ((direction != 1 && direction != -1) || N < 128 || (N & (N - 1)) != 0 || !(width == 16 || (width == 32 && N <= 256)))
+        return fail(GRIDSPT_E_INVALID, "no column self-test for N=%d, width=%d, direction=%d", N, width, direction);
+    if (gridspt_status st = set_device(p)) return st;
+    CK(launch_columns_selftest(N, width, direction, one_exchange != 0, static_cast<const float2*>(in),
+                               static_cast<float2*>(out), p->geo.tw, (cudaStream_t)stream), "column self-test");
+    return GRIDSPT_OK;
+}
+
+gridspt_status gridspt_selftest_normals(gridspt_plan p, const void* words, int32_t n, double* out,
+                                        gridspt_stream stream) {
+    g_err[0] = 0;
+    if (check_plan(p)) return GRIDSPT_E_INVALID;
+    if (!words || !out || !aligned16(words) || !aligned16(out) || n < 1)
+        return fail(GRIDSPT_E_INVALID, "words/out NULL or not 16-byte aligned, or n < 1");
+    if (gridspt_status st = set_device(p)) return st;
+    CK(launch_normals_selftest(static_cast<const uint2*>(words), n, reinterpret_cast<const float2*>(p->ic_angles + kIcAngles),
+                               p->ic_angles, reinterpret_cast<double2*>(out), (cudaStream_t)stream), "normals self-test");
+    return GRIDSPT_OK;
+}
+
 // ---------------------------------------------------------- emulator MLP
 }  // extern "C"
 namespace {

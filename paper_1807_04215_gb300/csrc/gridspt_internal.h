@@ -209,6 +209,10 @@ cudaError_t launch_ic_table(const IcArgs& a, cudaStream_t s);
 // One block waits on an mbarrier that nothing completes; the bounded wait gives
 // up and sets *status (exercises the timeout path without hanging the GPU).
 cudaError_t launch_wait_selftest(int* status, cudaStream_t s);
+cudaError_t launch_columns_selftest(int N, int width, int dir, int one, const float2* in, float2* out, const float2* tw,
+                                    cudaStream_t s);
+cudaError_t launch_normals_selftest(const uint2* words, int n, const float2* logs, const float4* angles, double2* out,
+                                    cudaStream_t s);
 cudaError_t launch_xexp(const Geo& g, const XExpArgs& a, cudaStream_t s);
 cudaError_t launch_yexp(const Geo& g, const YZExpArgs& a, cudaStream_t s);
 cudaError_t launch_zexp(const Geo& g, const YZExpArgs& a, cudaStream_t s);

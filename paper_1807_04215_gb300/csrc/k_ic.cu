@@ -249,4 +249,19 @@ cudaError_t launch_ic(const Geo& g, const IcArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// Self-test: the two deviates of given Philox words, value and error added in FP64.
+__global__ void k_normals_selftest(const uint2* __restrict__ words, int n, const float2* __restrict__ logs,
+                                   const float4* __restrict__ angles, double2* __restrict__ out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    float2 g1, g2;
+    box_muller(words[i].x, words[i].y, logs, angles, g1, g2);
+    out[i] = make_double2((double)g1.x + (double)g1.y, (double)g2.x + (double)g2.y);
+}
+cudaError_t launch_normals_selftest(const uint2* words, int n, const float2* logs, const float4* angles, double2* out,
+                                    cudaStream_t s) {
+    k_normals_selftest<<<(n + 255) / 256, 256, 0, s>>>(words, n, logs, angles, out);
+    return cudaGetLastError();
+}
+
 }  // namespace gridspt
