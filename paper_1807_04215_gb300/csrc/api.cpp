@@ -346,11 +346,13 @@ gridspt_status gridspt_plan_create(const gridspt_desc* d, gridspt_plan* out) {
     }
     // Pass variants of a plan that is not autotuned (all variants are bitwise
     // equal). Warp-row z passes from N = 64 on: run_orders (n_max = 5) with tiles
-    // / warp rows takes 0.217 / 0.273 ms at 32^3, 0.312 / 0.367 at 48^3, 0.253 /
-    // 0.236 at 64^3, 0.460 / 0.456 at 96^3, 0.92 / 0.59 at 128^3, 3.15 / 2.60 at
-    // 192^3, 6.38 / 3.90 at 256^3, 41.6 / 29.8 at 512^3. The z forward pass from
-    // N = 256 on: r2c 0.048 / 0.052 ms at 192^3, 0.089 / 0.085 at 256^3, 0.70 /
-    // 0.64 at 512^3.
+    // / warp rows, replayed from a graph, takes 0.200 / 0.147 ms at 64^3, 0.404 /
+    // 0.365 at 96^3, 0.84 / 0.49 at 128^3, 3.05 / 2.41 at 192^3, 5.92 / 3.27 at
+    // 256^3. (The line was drawn where launches did not overlap: 0.217 / 0.273 at
+    // 32^3, 0.312 / 0.367 at 48^3. As they are launched now warp rows are ahead there
+    // too, 0.164 / 0.142 and 0.252 / 0.189, and from 16^3 on; a plan that is autotuned
+    // runs them.) The z forward pass from N = 256 on: r2c 0.048 / 0.052 ms at 192^3,
+    // 0.089 / 0.085 at 256^3, 0.70 / 0.64 at 512^3.
     // The tiles of the 3 * 2^a grids: narrow x and y tiles where the wide ones leave
     // a block of 256 threads (192^3: x 2.62 -> 2.56, y 2.62 -> 2.50 ms in all) or of
     // 1024 at 64 registers (768^3: x 72.3 -> 68.5, y 72.3 -> 67.3), the wide ones at

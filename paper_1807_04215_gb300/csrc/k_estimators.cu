@@ -36,8 +36,8 @@
 namespace gridspt {
 
 constexpr int kPowWarps = 8;
-constexpr int kPowBlocks = 304;         // blocks launched at most: two per SM, all resident (the scratch
-                                        // holds power_blocks(); 456 blocks: 34 us, 304: 32)
+constexpr int kPowBlocks = 304;         // blocks launched at most: two on each of this GPU's 152 SMs (the
+                                        // scratch holds power_blocks(); 456 blocks: 34 us, 304: 32)
 
 int power_blocks(const Geo& g) {
     const long long rows = (long long)g.N * g.N;

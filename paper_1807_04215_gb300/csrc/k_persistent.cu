@@ -244,12 +244,13 @@ __device__ void q_zr2c(const QStage& st, long long tile, float2* sm, bool table_
 }
 
 // Layout class of the table a stage kind keeps at the start of shared memory:
-// 1 the stage-twiddle table of the expansion column transforms (fft_col),
-// 2 the warp-row tables of k_zrow, 3 the warp-row tables of QRow, 4 the table
-// of N-th roots of the forward column passes (0: none).
-__host__ __device__ constexpr int q_table_class(int kind, bool row_ok) {
+// 1 the column transforms' table (the one-exchange transform's where the grid has
+// that form, in every column pass; else the stage twiddles of the expansion
+// passes), 2 the warp-row tables of k_zrow, 3 the warp-row tables of QRow, 4 the
+// table of N-th roots of the other grids' forward column passes (0: none).
+__host__ __device__ constexpr int q_table_class(int kind, bool row_ok, bool one) {
     return (kind == Q_XEXP0 || kind == Q_XEXP1 || kind == Q_YEXP) ? 1
-           : (kind == Q_COLY || kind == Q_COLX) ? 4
+           : (kind == Q_COLY || kind == Q_COLX) ? (one ? 1 : 4)
            : kind == Q_Z ? (row_ok ? 2 : 3) : kind == Q_ZR2C ? 3 : 0;
 }
 
@@ -410,7 +411,8 @@ k_queue(const QStage* __restrict__ stages, const long long* __restrict__ starts,
                         reinterpret_cast<float4*>(fld ? st.data2 : st.data)[i2] = make_float4(0.f, 0.f, 0.f, 0.f);
                 }
             } else {
-                const int cls = q_table_class(st.kind, (st.N & (st.N - 1)) == 0);
+                const bool pow2 = (st.N & (st.N - 1)) == 0;
+                const int cls = q_table_class(st.kind, pow2, pow2 && st.N >= 128);
                 const int key = cls ? (cls << 16) | st.N : 0;
                 const bool tr = key != 0 && s_tabkey == key;
                 switch (st.N) {

@@ -76,15 +76,6 @@ struct ColSm {
 template <int N, int TZ>
 __host__ __device__ constexpr size_t colpass_smem() { return sizeof(float2) * (N + (size_t)N * TZ); }
 
-// Blocks per SM the expansion column passes are compiled for: two 512-thread
-// blocks (64 registers a thread) for the narrow tile of power-of-two N >= 512,
-// where one block of the natural ~75-86 registers leaves 16 warps per SM; one
-// elsewhere (smaller N and radix-3 sizes would spill heavily).
-template <int N, int TZ>
-__host__ __device__ constexpr int col_min_blocks() {
-    return (fft_elems(N) == 8 && N >= 512 && TZ * (N / fft_elems(N)) <= 512) ? 2 : 1;
-}
-
 __device__ __forceinline__ int signed_idx(int n, int N) { return n < N / 2 ? n : n - N; }
 
 __device__ __forceinline__ void load_table(float2* tw, const float2* __restrict__ twg, int N) {
@@ -267,12 +258,12 @@ k_zr2c(const float2* in, float2* out, long long fstride, const float2* __restric
 }
 
 // ------------------------------------------------------------ x expansion
-// Blocks per SM: col_min_blocks (a small spill at 64 registers); the divergence
-// form holds three columns at its widest, 128 registers a thread: two blocks of
-// 256 threads (384^3: 0.76 ms, one block at 255 registers 1.09).
+// Blocks per SM: one; the divergence form holds three columns at its widest, 128
+// registers a thread: two blocks of 256 threads (384^3: 0.76 ms, one block at 255
+// registers 1.09).
 template <int N, int TZ, int MODE>
 __host__ __device__ constexpr int xexp_min_blocks() {
-    return MODE != 2 ? col_min_blocks<N, TZ>() : TZ * (N / fft_elems(N)) <= 256 ? 2 : 1;
+    return MODE == 2 && TZ * (N / fft_elems(N)) <= 256 ? 2 : 1;
 }
 
 // Inputs: delta(k) and theta(k) columns along kx. Each output f is
@@ -523,7 +514,7 @@ __device__ __forceinline__ void yexp_body(const YZExpArgs& args, const float2* _
 }
 
 template <int N, int TZ>
-__global__ void __launch_bounds__(TZ * Cfg<N>::PC, col_min_blocks<N, TZ>())
+__global__ void __launch_bounds__(TZ * Cfg<N>::PC)
 k_yexp(const __grid_constant__ YZExpArgs args, const float2* __restrict__ twg, float kF) {
     pdl_pass<N>();
     extern __shared__ __align__(16) float2 sm[];
@@ -852,12 +843,11 @@ __global__ void __launch_bounds__(TZ * Cfg<N>::PZ, 1)
 k_zexp_pairs(ZPairArgs args, const float2* __restrict__ twg, float kF) {
     pdl_pass<N>();
     constexpr int M = N / 2, E = fft_elems(M), P = M / E, PITCH = Cfg<N>::PITCH, NTH = TZ * P;
-    constexpr int MAXP = kMaxPartners;         // partner fields of one output over all targets
     extern __shared__ float2 sm[];
     float2* tw = sm;
     float2* tin = sm + N;                      // input xy-field tile
     float2* tex = tin + TZ * PITCH;            // output tile / exchange buffer
-    float2* tpt = tex + TZ * PITCH;            // MAXP partner tiles
+    float2* tpt = tex + TZ * PITCH;            // kMaxPartners partner tiles
     const int tid = threadIdx.x, c = tid % TZ, p = tid / TZ;
     load_table(tw, twg, N);
     const long long rows = (long long)N * N;
@@ -1023,7 +1013,6 @@ struct RowCfg {
     static constexpr int XROW = M + (M >> 4);                 // padded exchange row
     static constexpr int NTW = fft_row_tw_total<M>();
     static constexpr int HDR = ((NTW + E) * P + 1) / 2 * 2;   // twiddle tables, 16-byte multiple
-    static constexpr int MAXP = kMaxPartners;
     static constexpr int WIN = RW * M;                        // input rows of a team
     static constexpr int PIECES = WIN / (2 * TL);             // 16-byte pieces of them per lane
     static_assert(!ok || (WIN % (2 * TL) == 0 && (RW * XROW) % 2 == 0), "16-byte row copies by the team's lanes");
@@ -1881,7 +1870,7 @@ struct LaunchCol2 {
 };
 
 // The column passes of one size: the one-exchange form where it exists, else the
-// tile of variant v (0 wide, 1 narrow). The divergence form's x pass holds four
+// tile of variant v (0 wide, 1 narrow). The divergence form's x pass holds three
 // columns: always the narrow tile of xexp_body.
 template <int N>
 struct Columns {
