@@ -761,11 +761,20 @@ __global__ void k_convert(const float* __restrict__ src, T* __restrict__ dst, lo
 long long mlp_params(int I, int H, int O) { return (long long)I * H + H + (long long)H * H + H + (long long)H * O + O; }
 int mlp_bwd_blocks(int B) { return (B + kGradRows - 1) / kGradRows; }
 
-// All of a block's shared memory as the limit for every call: two threads with networks
-// of different widths must not lower it under one another's launch.
-template <typename K>
-static cudaError_t smem_attr(K k) {
-    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+// All of a block's shared memory as the limit, set once per kernel and device: two threads
+// with networks of different widths must not lower it under one another's launch (and the
+// call takes a fifth of a microsecond of the host's three a launch).
+template <auto K>
+static cudaError_t smem_attr() {
+    static std::atomic<unsigned long long> set{0};                 // bit d: set on device d
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (set.load() & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+    if (e == cudaSuccess) set.fetch_or(bit);
+    return e;
 }
 
 // Rows per block: two while that gives at most two blocks per SM (304), eight
@@ -795,7 +804,7 @@ static cudaError_t mlp_forward_r(const float* x, int B, int I, int H, int O, con
     wbytes = (wbytes + 15) & ~15;
     const size_t sm = 2 * (size_t)wbytes +
                       sizeof(float) * ((size_t)row_pitch<R>() * ((H > I ? H : I) + H) + 2 * H + O);
-    cudaError_t e = smem_attr(k_mlp_forward<T, R>);
+    cudaError_t e = smem_attr<k_mlp_forward<T, R>>();
     if (e != cudaSuccess) return e;
     const int wide = H > O ? H : O, ct = FwdTile<R>::CT;
     int nt = (((wide + ct - 1) / ct) * (R / FwdTile<R>::RT) + 31) / 32 * 32;
@@ -810,7 +819,7 @@ template <typename T>
 static cudaError_t mlp_forward_rows(const float* x, int B, int I, int H, int O, const void* theta, float* y, float* act,
                                     cudaStream_t s) {
     const size_t sm = sizeof(float) * kDenseRows * (size_t)((I > H ? I : H) + (H > O ? H : O));
-    cudaError_t e = smem_attr(k_mlp_forward_rows<T>);
+    cudaError_t e = smem_attr<k_mlp_forward_rows<T>>();
     if (e != cudaSuccess) return e;
     k_mlp_forward_rows<T><<<(unsigned)((B + kDenseRows - 1) / kDenseRows), 256, sm, s>>>(
         x, B, I, H, O, static_cast<const T*>(theta), y, act);
@@ -841,7 +850,7 @@ static cudaError_t mlp_delta_r(int B, int I, int H, int O, const void* theta, co
         wbytes = std::max(wbytes, H * delta_pitch<T>(delta_cols<T>(all, H)) * (int)sizeof(T));
     wbytes = (wbytes + 15) & ~15;
     const size_t sm = 2 * (size_t)wbytes + sizeof(float) * (size_t)row_pitch<R>() * ((O > H ? O : H) + H);
-    cudaError_t e = smem_attr(k_mlp_delta<T, R>);
+    cudaError_t e = smem_attr<k_mlp_delta<T, R>>();
     if (e != cudaSuccess) return e;
     const int need = (H * (R == 2 ? 1 : 2) + 31) / 32 * 32, nt = need < 256 ? 256 : need, blocks = (B + R - 1) / R;
     pdl(k_mlp_delta<T, R>, (unsigned)blocks, nt, sm, s)(B, I, H, O, static_cast<const T*>(theta), act, dy, d2, d1, wbytes,
@@ -865,7 +874,7 @@ static cudaError_t mlp_backward(const float* x, int B, int I, int H, int O, cons
     parts = (B + per - 1) / per;
     cudaError_t e;
     if (2LL * H * B + (parts > 1 ? parts * np : 0) > room || (tiles <= 3 && B > 64 && B < 1024)) {
-        e = smem_attr(k_mlp_backward_rows<T>);
+        e = smem_attr<k_mlp_backward_rows<T>>();
         if (e != cudaSuccess) return e;
         k_mlp_backward_rows<T><<<mlp_bwd_blocks(B), 256, sizeof(float) * (size_t)kGradRows * (I + 6 * H + O), s>>>(
             x, B, I, H, O, static_cast<const T*>(theta), act, dy, ws);
