@@ -1180,7 +1180,8 @@ __device__ __forceinline__ void zrow_body(const ZPairArgs& args, const float2* _
                 // belongs to lane P - p, index E - 1 - i, goes there by shuffle. Lane 0
                 // pairs i with E - i: it shifts its values by one and adds k = M / 2, its
                 // own partner. Half the shared-memory reads and products of forming each (the
-                // pass is bound by shared-memory wavefronts, 0.75 a point: 87 % busy):
+                // pass is bound by shared-memory wavefronts, 0.75 a point before this; with it the
+                // load/store data pipe is at 74 .. 86 % of its peak at 256^3):
                 // 512^3 z passes of orders 1 .. 4 2.47 -> 2.26, 3.53 -> 3.40, 4.23 -> 4.00,
                 // 3.30 -> 3.08 ms.
                 float2 mir[E / 2], Ev, Ov;
