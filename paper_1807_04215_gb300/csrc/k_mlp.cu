@@ -860,6 +860,8 @@ static cudaError_t mlp_delta_r(int B, int I, int H, int O, const void* theta, co
 // Parts of the rows that the gradient tiles are split into: one tile an SM, 128 rows a
 // part at least. Backward of 16384 rows (bf16), unsplit / split: 3 -> 16 -> 16 -> 16
 // (3 tiles) 223 / 31 us, 3 -> 16 -> 16 -> 160 (12) 244 / 59, 3 -> 64 -> 64 -> 160 (60) 261 / 160.
+// The parts' sums are added in order; against 64 bits the gradients are off by 0.4 to 1.0 of
+// the unsplit ones' error (16 .. 97 hidden units, 300 .. 16384 rows).
 static int grad_parts(int B, int tiles) { return std::max(1, std::min(152 / tiles, B / 128)); }
 
 // The deltas of all rows, then the gradient tiles over the rows: in parts of rows
